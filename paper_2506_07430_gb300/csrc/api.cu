@@ -29,6 +29,7 @@ struct kpm_ctx {
     DevBuf d_h1, d_eri, d_dip, d_V32, d_diag;
     SpinTables ta, tb_own;
     SpinTables* tb = nullptr;
+    PairTables pairs;              // row kernels of the FP64 and FP32 sigma
     std::unique_ptr<TcSigma> tc;  // tensor-core sigma (KPM_MIXED)
     std::unique_ptr<PauliH> pauli;  // Pauli-string form of H (built on first use)
 
@@ -157,8 +158,37 @@ void require_device() {
     }
 }
 
+// operands of the FP64 / FP32 sigma of this context (x, y and ncol left to the caller)
+void sigma_operands(kpm_ctx* c, BatchMol& m) {
+    const bool f64 = c->prec == KPM_FP64;
+    const SpinTables& A = c->ta;
+    const SpinTables& B = *c->tb;
+    sigma_shape(m, A, B, f64);
+    m.tgtA = A.tgt.as<int32_t>();
+    m.pqA = A.pq.as<uint16_t>();
+    m.sgnA = A.sgn.as<int8_t>();
+    m.fcolA = A.fcol.as<int32_t>();
+    m.fvalA = f64 ? A.fval64.p : A.fval32.p;
+    m.tgtBT = B.tgtT.as<int32_t>();
+    m.pqBT = B.pqT.as<uint16_t>();
+    m.sgnBT = B.sgnT.as<int8_t>();
+    m.fcolB = B.fcol.as<int32_t>();
+    m.fvalB = f64 ? B.fval64.p : B.fval32.p;
+    m.V = f64 ? c->d_eri.p : c->d_V32.p;
+    m.diag = f64 ? nullptr : c->d_diag.as<float2>();
+    m.maskA = A.masks.as<uint32_t>();
+    c->pairs.fill(m);
+}
+
 void sigma_dispatch(kpm_ctx* c, const void* x, void* y, int ncol) {
-    if (c->prec == KPM_FP64) {
+    if (c->pairs.path != SIGMA_GATHER) {
+        BatchMol m{};
+        sigma_operands(c, m);
+        m.x = x;
+        m.y = y;
+        m.ncol = ncol;
+        sigma_rows(m, c->st);
+    } else if (c->prec == KPM_FP64) {
         SigmaArgs a{&c->ta, c->tb, c->d_eri.p, c->n, c->dim};
         sigma_gather_f64(a, (const double*)x, (double*)y, ncol, c->st);
     } else if (c->prec == KPM_FP32) {
@@ -435,69 +465,66 @@ void batch_steps(kpm_ctx* const* ctxs, int count, int nsteps) {
         c0->desc_host_cap = need;
     }
     BatchMol* h = c0->desc_host;
-    int64_t sblk = 0, ublk = 0;
-    size_t smem = 16;
-    for (int i = 0; i < count; ++i) {
-        kpm_ctx* c = ctxs[i];
-        const SpinTables& A = c->ta;
-        const SpinTables& B = *c->tb;
-        BatchMol m{};
-        m.nsa = A.ns;
-        m.nsb = B.ns;
-        m.tgtA = A.tgt.as<int32_t>();
-        m.pqA = A.pq.as<uint16_t>();
-        m.sgnA = A.sgn.as<int8_t>();
-        m.fcolA = A.fcol.as<int32_t>();
-        m.fvalA = f64 ? A.fval64.p : A.fval32.p;
-        m.tgtBT = B.tgtT.as<int32_t>();
-        m.pqBT = B.pqT.as<uint16_t>();
-        m.sgnBT = B.sgnT.as<int8_t>();
-        m.fcolB = B.fcol.as<int32_t>();
-        m.fvalB = f64 ? B.fval64.p : B.fval32.p;
-        m.V = f64 ? c->d_eri.p : c->d_V32.p;
-        m.diag = f64 ? nullptr : c->d_diag.as<float2>();
-        m.nexcA = A.nexc;
-        m.nnbrA = A.nnbr;
-        m.nexcB = B.nexc;
-        m.nnbrB = B.nnbr;
-        m.n = c->n;
-        m.ncol = c->rec_ncol;
-        m.a = c->rec_a;
-        m.b = c->rec_b;
-        m.partials = c->partials.as<double>();
-        m.counters = c->counters.as<unsigned>();
-        m.dots = c->dots.as<double>();
-        m.dstride = (int64_t)c->rec_max_steps * 2;
-        m.step0 = c->rec_steps;
-        m.nblk = reduce_blocks(c->dim);
-        m.sblk0 = sblk;
-        m.ublk0 = ublk;
-        sblk += (B.ns + 127) / 128 * A.ns * m.ncol;
-        ublk += (int64_t)m.nblk * m.ncol;
-        smem = std::max(smem, (size_t)A.nnbr * ((f64 ? 8 : 4) + 4) + (size_t)A.nexc * 12 + 16);
-        // even batch steps: the current assignment; odd: swapped
-        m.x = c->rec_cur;
-        m.y = c->vS.p;
-        m.prev = c->rec_prev;
-        h[i] = m;
-        m.x = c->rec_prev;
-        m.prev = c->rec_cur;
-        h[(size_t)count + i] = m;
+    // by sigma path: the row kernels' molecules in one launch, the gather kernel's in
+    // another, and those large enough for the pair-tiled kernels one by one (they fill
+    // the chip alone); each path's molecules are consecutive in the table
+    int first[4] = {0, 0, 0, 0};    // rows, gather, slots
+    int64_t sblk[2] = {0, 0}, ublk = 0;
+    size_t smem[2] = {16, 16};
+    int threads = 64, k = 0;
+    static const int order[3] = {SIGMA_ROWS, SIGMA_GATHER, SIGMA_SLOTS};
+    for (int g = 0; g < 3; ++g) {
+        first[g] = k;
+        for (int i = 0; i < count; ++i) {
+            kpm_ctx* c = ctxs[i];
+            if (c->pairs.path != order[g]) continue;
+            BatchMol m{};
+            sigma_operands(c, m);
+            m.ncol = c->rec_ncol;
+            m.a = c->rec_a;
+            m.b = c->rec_b;
+            m.partials = c->partials.as<double>();
+            m.counters = c->counters.as<unsigned>();
+            m.dots = c->dots.as<double>();
+            m.dstride = (int64_t)c->rec_max_steps * 2;
+            m.step0 = c->rec_steps;
+            m.nblk = reduce_blocks(c->dim);
+            m.ublk0 = ublk;
+            ublk += (int64_t)m.nblk * m.ncol;
+            if (g < 2) {
+                m.sblk0 = sblk[g];
+                sblk[g] += (g == 0 ? 1 : (m.nsb + 127) / 128) * m.nsa * m.ncol;
+                smem[g] = std::max(smem[g], g == 0 ? m.smem
+                                                   : (size_t)m.nnbrA * ((f64 ? 8 : 4) + 4) +
+                                                         (size_t)m.nexcA * 12 + 16);
+                if (g == 0) threads = std::max(threads, m.threads);
+            }
+            // even batch steps: the current assignment; odd: swapped
+            m.x = c->rec_cur;
+            m.y = c->vS.p;
+            m.prev = c->rec_prev;
+            h[k] = m;
+            m.x = c->rec_prev;
+            m.prev = c->rec_cur;
+            h[(size_t)count + k] = m;
+            ++k;
+        }
     }
+    first[3] = k;
     c0->batch_desc.ensure(need * sizeof(BatchMol));
     KPM_CUDA(cudaMemcpyAsync(c0->batch_desc.p, h, need * sizeof(BatchMol), cudaMemcpyHostToDevice,
                              st));
     KPM_CUDA(cudaEventRecord(c0->ev_desc, st));
     const BatchMol* d = c0->batch_desc.as<BatchMol>();
-    for (int k = 0; k < nsteps; ++k) {
-        const BatchMol* dk = d + (size_t)(k & 1) * count;
-        if (f64) {
-            sigma_gather_batch_f64(dk, count, sblk, smem, st);
-            cheb_update_batch_f64(dk, count, ublk, k, st);
-        } else {
-            sigma_gather_batch_f32(dk, count, sblk, smem, st);
-            cheb_update_batch_f32(dk, count, ublk, k, st);
-        }
+    for (int s = 0; s < nsteps; ++s) {
+        const size_t half = (size_t)(s & 1) * count;
+        const BatchMol* dk = d + half;
+        sigma_rows_batch(dk, first[1], sblk[0], smem[0], threads, st);
+        if (f64) sigma_gather_batch_f64(dk + first[1], first[2] - first[1], sblk[1], smem[1], st);
+        else sigma_gather_batch_f32(dk + first[1], first[2] - first[1], sblk[1], smem[1], st);
+        for (int i = first[2]; i < first[3]; ++i) sigma_rows(h[half + i], st);
+        if (f64) cheb_update_batch_f64(dk, count, ublk, s, st);
+        else cheb_update_batch_f32(dk, count, ublk, s, st);
     }
     for (int i = 0; i < count; ++i) {
         kpm_ctx* c = ctxs[i];
@@ -589,6 +616,8 @@ kpm_status kpm_create(const double* h1, const double* eri, const double* dipole,
             c->d_diag.alloc((size_t)c->dim * sizeof(float2));
             exact_diagonal(c->ta, *c->tb, c->d_eri.as<double>(), norb, c->d_diag.as<float2>(), c->st);
         }
+        if (prec == KPM_FP64 || prec == KPM_FP32)
+            c->pairs.build(c->ta, *c->tb, c->d_eri.as<double>(), prec == KPM_FP64, c->st);
         if (prec == KPM_MIXED || prec == KPM_MIXED_BF16) {
             // W over unordered pairs {p<=q}: rows (pq|rs) and the one-body row k_pq.
             // wmax = max |W|, wcol = max over output pairs of the column sum of |W|.

@@ -134,6 +134,46 @@ void dipole_apply_f64(const SpinTables& ta, const SpinTables& tb, const double* 
 void dipole_apply_f32(const SpinTables& ta, const SpinTables& tb, const double* d_dip,
                       const double* psi, float* y, cudaStream_t st);
 
+// ---------------------------------------------------------------- sigma (row kernels)
+
+// Which kernels apply H in FP64 and FP32 (sigma_path): a CTA per alpha string over the
+// whole row (k_sigma_rows), the pair-tiled FP32 kernels (k_opp_slots, k_same_dense), or
+// a thread per determinant (k_sigma_gather).
+enum SigmaPath { SIGMA_GATHER = 0, SIGMA_ROWS = 1, SIGMA_SLOTS = 2 };
+
+SigmaPath sigma_path(const SpinTables& A, const SpinTables& B, bool f64);
+
+struct BatchMol;
+
+// Tables over unordered off-diagonal orbital pairs s = {p < q}, index q (q - 1) / 2 + p,
+// of one context's FP64 or FP32 row kernels (sigma_rows.cu).  T is double or float.
+struct PairTables {
+    struct Spin {
+        DevBuf otgt;    // int32  [ns][noff] targets of the off-diagonal entries
+        DevBuf oslot;   // uint16 [ns][noff] their pair | sign << 15
+        DevBuf slotT;   // uint16 [noff][ns] their pair, string-fastest
+        DevBuf back;    // uint8  [ns][noff] the entry of the target that leads back
+        DevBuf revT;    // uint32 [noff][ns] target | back << 16 | sign << 31, by back
+        DevBuf stgt;    // uint16 [NO][ns] target under a pair | sign << 15 (ns: none)
+        DevBuf v;       // [NO][ns] sum over a string's occupied i of (ii|pq): FP64, or
+                        // float hi + lo
+        DevBuf c;       // double [n][ns] the same of (ii|qq)
+        DevBuf dense;   // float [ns][ld] off-diagonal string Hamiltonian (k_same_dense)
+        int64_t ld = 0;
+    };
+    SigmaPath path = SIGMA_GATHER;
+    bool f64 = false;
+    DevBuf woo;         // T [NO][NO] (pq|rs)
+    Spin a, b_own;
+    Spin* b = nullptr;
+    void build(const SpinTables& A, const SpinTables& B, const double* eri, bool f64,
+               cudaStream_t st);
+    void fill(BatchMol& m) const;   // after sigma_shape
+private:
+    void build_spin(Spin& t, const SpinTables& T, const double* eri, SigmaPath path, bool f64,
+                    cudaStream_t st);
+};
+
 // ---------------------------------------------------------------- batched steps
 
 // One molecule of a batched recursion step (kpm_moments_batch): the operands of
@@ -169,7 +209,34 @@ struct BatchMol {
     int nblk;           // reduction blocks per column: reduce_blocks(nsa * nsb)
     int64_t sblk0;      // first block of this molecule in the flattened sigma grid
     int64_t ublk0;      // first block of this molecule in the flattened update grid
+    // row kernels (PairTables); shapes from sigma_shape
+    int path;           // SigmaPath
+    int noffA, noffB;   // off-diagonal table entries per string, m (n - m)
+    int NO, K;          // pairs n (n - 1) / 2; terms of D: noffA + 1 (FP32: + 2), or 0
+                        // without electrons
+    int fc, ft, parts, stage_x, threads, ts;   // geometry (rows_geometry, opp_choose)
+    int64_t ldA, ldB;
+    size_t smem;
+    const int32_t* otgtA;
+    const uint16_t* oslotA;
+    const uint16_t* slotTB;
+    const uint32_t* revTB;
+    const uint16_t* stgtB;
+    const uint32_t* maskA;
+    const void* woo;
+    const void* vA;
+    const void* vB;
+    const double* cB;
+    const float* denseA;
+    const float* denseB;
 };
+
+void sigma_shape(BatchMol& m, const SpinTables& A, const SpinTables& B, bool f64);
+// m.x, m.y, m.ncol and the operands set; m.path SIGMA_ROWS or SIGMA_SLOTS
+void sigma_rows(const BatchMol& m, cudaStream_t st);
+// SIGMA_ROWS molecules only; blocks = sum of nsa * ncol, smem and threads the largest
+void sigma_rows_batch(const BatchMol* mols, int nmol, int64_t blocks, size_t smem, int threads,
+                      cudaStream_t st);
 
 // Sigma of every molecule of mols[0 .. nmol) in one launch of `blocks` blocks
 // (sum over molecules of ceil(nsb / 128) * nsa * ncol); smem: the largest

@@ -95,7 +95,12 @@ size_t estimate_bytes(int n, int na, int nb, int ncol, kpm_precision prec) {
         int64_t nexc = m * (n - m + 1);
         int64_t nnbr = 1 + (int64_t)m * (n - m) + binom(m, 2) * binom(n - m, 2);
         int P = ((n * (n + 1) / 2 + 1 + 15) / 16) * 16;
-        return (size_t)ns * (4 + 14 * nexc + 16 * nnbr + 4 * P);
+        // (off-diagonal lists, pair targets and merged-diagonal sums of the row kernels too)
+        const int64_t pairs = prec == KPM_FP64 || prec == KPM_FP32
+                                  ? 13 * nexc + 10 * n * (n - 1) / 2 + 8 * n +
+                                        (prec == KPM_FP32 ? 4 * (ns + 3) : 0)
+                                  : 0;
+        return (size_t)ns * (4 + 14 * nexc + 16 * nnbr + 4 * P + pairs);
     };
     v += tables(na, sa) + (na == nb ? 0 : tables(nb, sb));
     v += (size_t)n * n * n * n * 12 + (64 << 20);
