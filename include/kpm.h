@@ -363,8 +363,9 @@ kpm_status kpm_synchronize(kpm_ctx* ctx);
  * kpm_tuned_params -- the launch choices the library's autotuner made for this
  * context at creation: the rasterisation group (row tiles that sweep the column
  * tiles together, for L2 reuse) of the beta and alpha same-spin GEMMs of the
- * tensor-core paths, picked from {4, 8, 16, 32} by timing each once per device
- * and shape (16 for shapes too small to tune).  The choice never changes
+ * tensor-core paths (one launch holds both, so the two are equal), picked from
+ * {4, 8, 16, 32} by timing each once per device and shape (16 for shapes too
+ * small to tune).  The choice never changes
  * results.  FP64 / FP32 contexts report 0.  Errors: KPM_EINVAL for NULL ctx.
  */
 kpm_status kpm_tuned_params(const kpm_ctx* ctx, int* group_beta, int* group_alpha);

@@ -1173,8 +1173,8 @@ kpm_status kpm_test_rowpass_stall(kpm_ctx* ctx, int enable) {
 
 kpm_status kpm_tuned_params(const kpm_ctx* ctx, int* group_beta, int* group_alpha) {
     if (!ctx) { g_err = "NULL context"; return KPM_EINVAL; }
-    if (group_beta) *group_beta = ctx->tc ? ctx->tc->dense.group_m[0] : 0;
-    if (group_alpha) *group_alpha = ctx->tc ? ctx->tc->dense.group_m[1] : 0;
+    if (group_beta) *group_beta = ctx->tc ? ctx->tc->dense.group_m : 0;
+    if (group_alpha) *group_alpha = ctx->tc ? ctx->tc->dense.group_m : 0;
     return KPM_OK;
 }
 

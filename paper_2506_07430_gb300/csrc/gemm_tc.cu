@@ -11,13 +11,16 @@
 // out[m][n] = sum_k A[m][k] B[n][k] with both operands K-major,
 //   beta:  A = F_b (m = I_b, k = J),      B = C (n = I_a, k = J)
 //   alpha: A = C^T (m = I_b, k = J),      B = F_a (n = I_a, k = J)
-// and in both cases the epilogue adds out[m][n] into y[n * ldy + m], so the 32
-// lanes of a warp (consecutive m) write consecutive addresses.
+// Both add into y[n * ldy + m] of the same tile, so one launch accumulates the k-blocks
+// of the first and then of the second, and its epilogue reads and writes y once; the
+// 32 lanes of a warp (consecutive m) write consecutive addresses.  Against one launch
+// per product with an epilogue of one column at a time: sigma at 16 orbitals 48.7 ->
+// 45.4 ms, at 14 orbitals (3 columns) 7.59 -> 6.47 ms, at 10 orbitals 371 -> 203 us.
 //
 // Operands are split into two FP16 pieces with power-of-two scales (x = hi + lo);
 // three MMAs per k-step (A_hi B_hi + A_lo B_hi + A_hi B_lo) accumulate in FP32
 // in tensor memory.  The diagonals of F_a, F_b are kept out of the split matrices;
-// the epilogue of the alpha product adds the whole diagonal of H (same-spin
+// the epilogue adds the whole diagonal of H (same-spin
 // diagonals and the opposite-spin Coulomb sums, evaluated in FP64 and stored as
 // float hi + lo per determinant) times x, hi and lo multiplied separately.
 //
@@ -206,12 +209,11 @@ __host__ __device__ constexpr uint32_t gemm_idesc() {
 }
 
 struct GemmArgs {
-    int M, N, K;               // out is M x N; operands have K columns
-    float* y;                  // y[n * ldy + m] += scale * out[m][n]
+    int M, N;                  // M = N_b (m = I_b), N = N_a (n = I_a); sums over N_b, then N_a
+    float* y;                  // y[n * ldy + m] += sums / (wscale sa) + diagonal
     int64_t ldy;
-    float scale;               // or, if amax != nullptr, scale / (sa(amax)) with the operand scale
-    const float* amax;         // max |x| of the split vector operand (operand scale), or null
-    float wscale;              // scale of the matrix operand
+    const float* amax;         // max |x| of the split vector operand (operand scale sa)
+    float ratio, inv_wa;       // wscale_a / wscale_b, 1 / wscale_a (powers of two)
     // exact diagonal term (if x != nullptr): y[n*ldy+m] += d[n*ldy+m] * x[n*ldy+m], the
     // diagonal H_II evaluated in FP64 and stored as float (hi, lo)
     const float* x;
@@ -219,12 +221,18 @@ struct GemmArgs {
     int* err;
     int group_m;               // row tiles per rasterisation group (tuned; see DenseSS::autotune)
     // k-blocks holding a nonzero of the matrix operand, per tile of that operand (CSR:
-    // kbl[kbs[t] .. kbs[t + 1]) ascending); the tile is the row tile m0 / GM_BM when
-    // kb_by_n == 0 (matrix in A) or the column tile n0 / GM_BN (matrix in B).  A
-    // skipped k-block only adds zero products, so the sums are unchanged.  Null: all.
-    const int* kbs;
-    const int* kbl;
-    int kb_by_n;
+    // kbl[kbs[t] .. kbs[t + 1]) ascending): F_b by pairs of row tiles, F_a by column
+    // tile.  A skipped k-block only adds zero products, so the sums are unchanged.
+    const int* kbs_b;
+    const int* kbl_b;
+    const int* kbs_a;
+    const int* kbl_a;
+};
+
+// operand pieces (hi, lo) of the two products: F_b and the rows of x, the rows of x^T
+// and F_a
+struct GemmMaps {
+    CUtensorMap fb[2], x[2], t[2], fa[2];
 };
 
 // bounded wait that also gives up when another role has aborted; roles off the
@@ -264,9 +272,7 @@ __device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
 // growing like sqrt(K); in chunks, each accumulator sums a short run and the
 // running sum takes one rounding per chunk.
 __global__ void __cluster_dims__(GM_PAIR, 1, 1) __launch_bounds__(GM_THREADS, 1)
-k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-       const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1,
-       const GemmArgs g) {
+k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -295,18 +301,15 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
     // its A loads read the zero fill and its epilogue writes nothing)
     const int m0 = (mp * GM_PAIR + (int)crank) * GM_BM;
     const int n0 = ((b % gsize) / gm) * GM_BN;
-    // k-blocks the pair visits (both CTAs the same, as they share the B loads): all
-    // of K, or the blocks where the matrix operand's tile (the pair's 256 rows of
-    // A, or the 256-row B tile) has a nonzero
-    int nk = (g.K + GM_BK - 1) / GM_BK;
-    const int* klist = nullptr;
-    if (g.kbs) {
-        const int t = g.kb_by_n ? n0 / GM_BN : mp;
-        klist = g.kbl + g.kbs[t];
-        nk = g.kbs[t + 1] - g.kbs[t];
-    }
-    const int ck = GM_CK;                                      // k-blocks per chunk
-    const int nchunk = (nk + ck - 1) / ck;
+    // k-blocks the pair visits (both CTAs the same, as they share the B loads): those
+    // of F_b where the pair's 256 rows have a nonzero, then those of F_a where the
+    // 256-row B tile has one; accumulation chunks do not cross from one to the other
+    const int* kl1 = g.kbl_b + g.kbs_b[mp];
+    const int nk1 = g.kbs_b[mp + 1] - g.kbs_b[mp];
+    const int* kl2 = g.kbl_a + g.kbs_a[n0 / GM_BN];
+    const int nk = nk1 + g.kbs_a[n0 / GM_BN + 1] - g.kbs_a[n0 / GM_BN];
+    constexpr int ck = GM_CK;                                  // k-blocks per chunk
+    const int nchunk1 = (nk1 + ck - 1) / ck, nchunk = nchunk1 + (nk - nk1 + ck - 1) / ck;
 
     if (tid == 0) {
         for (int s = 0; s < GM_STAGES; ++s) {
@@ -321,10 +324,12 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
         *issued = 0;
         *consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        prefetch_map(&mA0);
-        prefetch_map(&mA1);
-        prefetch_map(&mB0);
-        prefetch_map(&mB1);
+        for (int i = 0; i < 2; ++i) {
+            prefetch_map(&maps.fb[i]);
+            prefetch_map(&maps.x[i]);
+            prefetch_map(&maps.t[i]);
+            prefetch_map(&maps.fa[i]);
+        }
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
@@ -347,29 +352,34 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
                     break;
                 unsigned char* st = smem + s * STAGE_BYTES;
                 mbar_expect_tx(&full[s], STAGE_BYTES);
-                const int kx = (klist ? klist[kb] : kb) * GM_BK;
-                tma_load_2d(su32(st), &mA0, kx, m0, &full[s]);
-                tma_load_2d(su32(st + A_BYTES), &mA1, kx, m0, &full[s]);
+                const bool beta = kb < nk1;
+                const int kx = (beta ? kl1[kb] : kl2[kb - nk1]) * GM_BK;
+                const CUtensorMap* mA = beta ? maps.fb : maps.t;
+                const CUtensorMap* mB = beta ? maps.x : maps.fa;
+                tma_load_2d(su32(st), mA, kx, m0, &full[s]);
+                tma_load_2d(su32(st + A_BYTES), mA + 1, kx, m0, &full[s]);
                 // this CTA's half of the B rows, into both CTAs
                 const uint32_t hb = crank * B_HALF;
                 const int nh = n0 + (int)crank * (GM_BN / GM_PAIR);
-                tma_load_2d_mc(su32(st + 2 * A_BYTES + hb), &mB0, kx, nh, &full[s], 0x3);
-                tma_load_2d_mc(su32(st + 2 * A_BYTES + B_BYTES + hb), &mB1, kx, nh, &full[s], 0x3);
+                tma_load_2d_mc(su32(st + 2 * A_BYTES + hb), mB, kx, nh, &full[s], 0x3);
+                tma_load_2d_mc(su32(st + 2 * A_BYTES + B_BYTES + hb), mB + 1, kx, nh, &full[s], 0x3);
                 *(volatile int*)issued = kb + 1;
             }
         }
     } else if (warp == GM_MMA_WARP) {
         if (lane == 0) {
-            // MMA issuer: chunk c accumulates k-blocks [c ck, (c + 1) ck) into buffer c & 1
+            // MMA issuer: chunk c accumulates its k-blocks (at most ck) into buffer c & 1
             constexpr uint32_t idesc = gemm_idesc();
             for (int c = 0; c < nchunk; ++c) {
                 const uint32_t d = tmem + (uint32_t)((c & 1) * GM_BN);
                 if (c >= 2 && !wait_or_abort(&acce[c & 1], ((c >> 1) - 1) & 1, abort_flag, g.err))
                     break;
                 tc_after();
-                const int kb1 = min(nk, (c + 1) * ck);
+                const bool beta = c < nchunk1;
+                const int kb0 = beta ? c * ck : nk1 + (c - nchunk1) * ck;
+                const int kb1 = min(beta ? nk1 : nk, kb0 + ck);
                 bool ok = true;
-                for (int kb = c * ck; kb < kb1; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     const int s = kb % GM_STAGES;
                     if (!wait_or_abort(&full[s], (kb / GM_STAGES) & 1, abort_flag, g.err)) {
                         ok = false;
@@ -385,7 +395,7 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
 #pragma unroll
                     for (int j = 0; j < GM_BK / 16; ++j) {
                         const uint32_t off = j * 32;  // 16 FP16 = 32 bytes along K in the row
-                        const uint32_t acc0 = (kb != c * ck || j != 0) ? 1u : 0u;
+                        const uint32_t acc0 = (kb != kb0 || j != 0) ? 1u : 0u;
                         mma_ss(d, sw_desc(a1 + off), sw_desc(b0 + off), idesc, acc0);
                         mma_ss(d, sw_desc(a0 + off), sw_desc(b1 + off), idesc, 1);
                     }
@@ -413,6 +423,11 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
                 ok = wait_or_abort(&accf[c & 1], (c >> 1) & 1, abort_flag, g.err, GM_BACKOFF_NS);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
+            // from the scale of F_b's product to that of F_a's (a power of two)
+            if (c == nchunk1 && g.ratio != 1.f) {
+#pragma unroll
+                for (int u = 0; u < GM_EPI_COLS; ++u) rs[u] *= g.ratio;
+            }
             tc_after();
             const uint32_t src = trow + (uint32_t)((c & 1) * GM_BN);
 #pragma unroll
@@ -427,8 +442,8 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
             if (lane == 0) mbar_arrive_(&acce[c & 1]);
         }
         if (ok && !*abort_flag) {
-            float scale = g.scale / g.wscale;
-            if (g.amax) {
+            float scale = (nchunk == nchunk1 ? g.ratio : 1.f) * g.inv_wa;
+            {
                 const float mx = *g.amax;
                 if (mx > 0.f && isfinite(mx)) {
                     int e;
@@ -436,21 +451,41 @@ k_gemm(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensor
                     scale = scale / ldexpf(1.f, 14 - max(e, -90));
                 }
             }
-            const int m = m0 + quad * 32 + lane;
-            if (m < g.M) {
+            // The sums move to the shared memory of the (now idle) stages, which frees
+            // their registers for 16 columns' loads in flight at a time: one column at a
+            // time waits for memory 128 times, 45 us a tile, most of the product's time
+            // at small sizes.  (Every stage's loads have been consumed by the MMAs whose
+            // accumulators were drained, so none is in flight into this memory.)
+            float* mine = reinterpret_cast<float*>(smem) + warp * (GM_EPI_COLS * 32) + lane;
 #pragma unroll
-                for (int u = 0; u < GM_EPI_COLS; ++u) {
-                    const int n = n0 + h * GM_EPI_COLS + u;
-                    if (n < g.N) {
-                        const int64_t o = (int64_t)n * g.ldy + m;
-                        float v = g.y[o] + rs[u] * scale;
+            for (int u = 0; u < GM_EPI_COLS; ++u) mine[u * 32] = rs[u];
+            const int m = m0 + quad * 32 + lane;
+            const int nb = n0 + h * GM_EPI_COLS;
+            constexpr int EG = 16;
+            const int ncols = m < g.M ? min(GM_EPI_COLS, g.N - nb) : 0;
+#pragma unroll 1
+            for (int u0 = 0; u0 < ncols; u0 += EG) {
+                const int64_t o0 = (int64_t)(nb + u0) * g.ldy + m;
+                float yv[EG], xv[EG];
+                float2 dv[EG];
+#pragma unroll
+                for (int u = 0; u < EG; ++u) {
+                    if (u0 + u < ncols) {
+                        const int64_t o = o0 + u * g.ldy;
+                        yv[u] = g.y[o];
                         if (g.x) {
-                            // hi and lo multiply separately: the diagonal keeps its FP64 value
-                            const float2 d = g.dfull[o];
-                            const float xv = g.x[o];
-                            v = fmaf(d.x, xv, fmaf(d.y, xv, v));
+                            xv[u] = __ldg(g.x + o);
+                            dv[u] = __ldg(g.dfull + o);
                         }
-                        g.y[o] = v;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < EG; ++u) {
+                    if (u0 + u < ncols) {
+                        float v = yv[u] + mine[(u0 + u) * 32] * scale;
+                        // hi and lo multiply separately: the diagonal keeps its FP64 value
+                        if (g.x) v = fmaf(dv[u].x, xv[u], fmaf(dv[u].y, xv[u], v));
+                        g.y[o0 + u * g.ldy] = v;
                     }
                 }
             }
@@ -765,31 +800,23 @@ void DenseSS::split(const float* x, const float* amax, cudaStream_t st) {
     KPM_LAUNCHED();
 }
 
-// beta: out[m = I_b][n = I_a] = sum_J Fb[I_b][J] x[I_a][J]   (x rows from split())
-void DenseSS::launch_beta(float* y, const float* amax, int group, cudaStream_t st) {
-    CUtensorMap a0 = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
-    CUtensorMap a1 = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
-    CUtensorMap b0 = make_map(xh.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
-    CUtensorMap b1 = make_map(xl.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
-    GemmArgs g{(int)nb, (int)na, (int)nb, y, nb, 1.0f, amax, (float)wscale_b,
-               nullptr, nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(), 0};
-    dim3 grid(gemm_grid(nb, na));
-    k_gemm<<<grid, GM_THREADS, smem, st>>>(a0, a1, b0, b1, g);
-    KPM_LAUNCHED();
-}
-
-// alpha: out[m = I_b][n = I_a] = sum_J x^T[I_b][J] Fa[I_a][J], plus the exact diagonals
-void DenseSS::launch_alpha(const float* x, float* y, const float* amax, int group,
-                           cudaStream_t st) {
+// y[I_a][I_b] += sum_J Fb[I_b][J] x[I_a][J] (x rows from split())
+//             + sum_J x^T[I_b][J] Fa[I_a][J] + H_II x[I_a][I_b]
+void DenseSS::launch(const float* x, float* y, const float* amax, int group, cudaStream_t st) {
     const float* diag = diag_full ? x : nullptr;
-    CUtensorMap a0 = make_map(th.as<__half>(), nb, na, pa, GM_BM);
-    CUtensorMap a1 = make_map(tl.as<__half>(), nb, na, pa, GM_BM);
-    CUtensorMap b0 = make_map(fa_hi->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
-    CUtensorMap b1 = make_map(fa_lo->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
-    GemmArgs g{(int)nb, (int)na, (int)na, y, nb, 1.0f, amax, (float)wscale_a,
-               diag, diag ? diag_full : nullptr, err, group, kbs_a.as<int>(), kbl_a.as<int>(), 1};
-    dim3 grid(gemm_grid(nb, na));
-    k_gemm<<<grid, GM_THREADS, smem, st>>>(a0, a1, b0, b1, g);
+    GemmMaps maps;
+    maps.fb[0] = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
+    maps.fb[1] = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
+    maps.x[0] = make_map(xh.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
+    maps.x[1] = make_map(xl.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
+    maps.t[0] = make_map(th.as<__half>(), nb, na, pa, GM_BM);
+    maps.t[1] = make_map(tl.as<__half>(), nb, na, pa, GM_BM);
+    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
+    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
+    GemmArgs g{(int)nb, (int)na, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
+               diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
+               kbs_a.as<int>(), kbl_a.as<int>()};
+    k_gemm<<<gemm_grid(nb, na), GM_THREADS, smem, st>>>(maps, g);
     KPM_LAUNCHED();
 }
 
@@ -801,11 +828,10 @@ void DenseSS::apply(const float* x, float* y, const float* amax, cudaStream_t st
     dim3 tb(32, 8), gt((unsigned)((nb + 31) / 32), (unsigned)((na + 63) / 64));
     k_split_transpose<<<gt, tb, 0, st>>>(x, na, nb, th.as<__half>(), tl.as<__half>(), pa, amax);
     KPM_LAUNCHED();
-    launch_beta(y, amax, group_m[0], st);
-    launch_alpha(x, y, amax, group_m[1], st);
+    launch(x, y, amax, group_m, st);
 }
 
-// Picks the rasterisation group of each GEMM by timing the candidates once per
+// Picks the rasterisation group of the GEMM by timing the candidates once per
 // device and shape (process-wide cache).  The group only decides which CTA
 // computes which output tile, never how a tile is computed, so results do not
 // depend on the choice.  Small shapes, where the whole problem sits in L2, keep
@@ -815,14 +841,13 @@ void DenseSS::autotune(cudaStream_t st) {
     int dev = 0;
     KPM_CUDA(cudaGetDevice(&dev));
     static std::mutex mu;
-    static std::map<std::array<int64_t, 3>, std::array<int, 2>> cache;
+    static std::map<std::array<int64_t, 3>, int> cache;
     const std::array<int64_t, 3> key{dev, na, nb};
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
         if (it != cache.end()) {
-            group_m[0] = it->second[0];
-            group_m[1] = it->second[1];
+            group_m = it->second;
             return;
         }
     }
@@ -845,30 +870,25 @@ void DenseSS::autotune(cudaStream_t st) {
     KPM_CUDA(cudaEventCreate(&e0));
     KPM_CUDA(cudaEventCreate(&e1));
     const int cand[4] = {4, 8, 16, 32};
-    for (int which = 0; which < 2; ++which) {
-        auto run = [&](int gsz) {
-            if (which == 0) launch_beta(ys.as<float>(), one.as<float>(), gsz, st);
-            else launch_alpha(ys.as<float>(), ys.as<float>(), one.as<float>(), gsz, st);
-        };
-        run(group_m[which]);  // warm-up
-        float best = 0.f;
-        for (int c : cand) {
-            KPM_CUDA(cudaEventRecord(e0, st));
-            run(c);
-            KPM_CUDA(cudaEventRecord(e1, st));
-            KPM_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            KPM_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            if (best == 0.f || ms < best) {
-                best = ms;
-                group_m[which] = c;
-            }
+    auto run = [&](int gsz) { launch(ys.as<float>(), ys.as<float>(), one.as<float>(), gsz, st); };
+    run(group_m);  // warm-up
+    float best = 0.f;
+    for (int c : cand) {
+        KPM_CUDA(cudaEventRecord(e0, st));
+        run(c);
+        KPM_CUDA(cudaEventRecord(e1, st));
+        KPM_CUDA(cudaEventSynchronize(e1));
+        float ms = 0.f;
+        KPM_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        if (best == 0.f || ms < best) {
+            best = ms;
+            group_m = c;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     std::lock_guard<std::mutex> lk(mu);
-    cache[key] = {group_m[0], group_m[1]};
+    cache[key] = group_m;
 }
 
 }  // namespace kpm

@@ -20,13 +20,13 @@ struct DenseSS {
     DevBuf xh, xl, th, tl;                    // split copies of x and x^T
     DevBuf fmax;                              // scratch for max |F_off|
     // per tile of the split matrix, the k-blocks that hold a nonzero (CSR; see
-    // block_lists): beta GEMM (F_b, 128-row tiles), alpha GEMM (F_a, 256-row tiles)
+    // block_lists): F_b by pairs of 128-row tiles, F_a by 256-row tiles
     DevBuf kbs_b, kbl_b, kbs_a, kbl_a;
     int64_t kb_nonzero[2] = {0, 0}, kb_total[2] = {0, 0};
     size_t smem = 0;
     int* err = nullptr;
     // exact diagonal H_II of the whole H (same-spin diagonals and the opposite-spin
-    // Coulomb sum, FP64 stored as float hi + lo, [N_a][N_b]), added by the alpha
+    // Coulomb sum, FP64 stored as float hi + lo, [N_a][N_b]), added by the
     // product's epilogue; the split matrices and the row pass leave it out
     const float2* diag_full = nullptr;
 
@@ -39,12 +39,11 @@ struct DenseSS {
     // diag_full * x (the whole exact diagonal of H); amax = device max|x|.
     // Uses xh/xl from split(x) on the same stream.
     void apply(const float* x, float* y, const float* amax, cudaStream_t st);
-    // Rasterisation group (row tiles per group) of the beta and alpha GEMMs, chosen
-    // by autotune() at set-up; 16 by default.
-    int group_m[2] = {16, 16};
+    // Rasterisation group (row tiles per group), chosen by autotune() at set-up; 16 by
+    // default.
+    int group_m = 16;
     void autotune(cudaStream_t st);
-    void launch_beta(float* y, const float* amax, int group, cudaStream_t st);
-    void launch_alpha(const float* x, float* y, const float* amax, int group, cudaStream_t st);
+    void launch(const float* x, float* y, const float* amax, int group, cudaStream_t st);
 };
 
 }  // namespace kpm
