@@ -65,14 +65,7 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                   "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[8]) {
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
@@ -151,27 +144,25 @@ struct RowPass {
     int64_t xpitch;          // multiple of 128
     float* Y;
     int64_t Nr, Nc;
-    const uint4* tslot8;     // [P/8][Nc]: 8 16-bit entries per chunk of 8 slots (slot 8c+u in
-                             // half u of the 128-bit word): target string | sign << 15,
-                             // Nc + (J mod 32) when the slot of column J is absent
+    const uint2* tslot4;     // [P/4][tpitch]: 4 16-bit entries per group of 4 slots: target
+                             // string | sign << 15, Nc + (J mod 32) when the slot of column
+                             // J is absent or J is past the row
+    int64_t tpitch;          // Nc rounded up to 128
     const int32_t* rtgt;     // [Nr][rnexc] row-string targets of the off-diagonal entries
     const uint16_t* rslot;   // [Nr][rnexc] their slot | sign << 15
     int rnexc;               // off-diagonal table entries per row string, m (n - m)
     int ndiag;               // 1 if the row strings hold electrons (a diagonal column), else 0
     int KR;                  // K of the row GEMM: rnexc + ndiag rounded up to 16 (at least 16)
-    const uint32_t* rmask;   // [Nr] occupation masks of the row strings
-    const double* wdiag;     // [n][P] W[qq][s] (unscaled, FP64; zero for diagonal slots s)
+    const double* wr;        // [Nr][P] w_R[s] (unscaled, FP64)
     const uint16_t* wrow;    // W by input slot: NW pieces of [P][P] 16-bit (bits of the format)
     uint32_t ncols;          // TMEM columns allocated
-    const float* amax;       // device max|x| (operand scaling)
-    const float* rowmax;     // [Nr] max |x| of each row (per-row fixed-point range)
+    const float2* rscale;    // [Nr] scale of B_R, scale of the row's integer sums (k_rowscale)
     float wscale;            // power-of-two scale applied to W in the image
-    int nexc_c;              // table entries per column string (contributions per target)
     int NS;                  // slots in use (n(n+1)/2); slots [NS, P) are padding
     int nst;                 // A stages in shared memory (2 or 3)
     int prefetch;            // L2 prefetch of the A rows this many tiles ahead (0: none)
     // wide layout (more than 32736 column strings, or a row's sigma beyond shared
-    // memory): 16-bit targets without the sign (absent: 0xFFFF), the sign taken from
+    // memory): 16-bit targets without the sign (absent, past the row: 0xFFFF), the sign taken from
     // the column string's occupations, and the targets split into npass ranges of
     // span strings, one pass over the row's tiles per range
     int npass;
@@ -193,6 +184,11 @@ constexpr int RP_WARPS = RP_SCATTER_WARPS + RP_COPY_WARPS + 1;
 constexpr int RP_THREADS = 32 * RP_WARPS;
 constexpr int RP_MAXK = 96;                  // largest KR: 9 * 10 = 90 entries rounded up
 static_assert(RP_COPY_WARPS * 32 >= RP_MAXK, "one copy lane per entry (L2 prefetch)");
+constexpr int RP_ROW_THREADS = 32 * (RP_SCATTER_WARPS + 1);   // scatter and MMA warps
+// barrier of the scatter and MMA warps (the copy warps run ahead across rows)
+__device__ __forceinline__ void row_barrier() {
+    asm volatile("bar.sync 1, %0;" ::"n"(RP_ROW_THREADS) : "memory");
+}
 // sink cells after the row's sigma: an absent slot of column J targets cell
 // Nc + (J mod 32), so the scatter adds every slot without a branch and the 32
 // lanes of a warp (32 consecutive J) sink into 32 different banks
@@ -208,6 +204,11 @@ constexpr int RP_SINK = 32;
 #endif
 constexpr uint32_t A_LBO = 2048;             // A stage: K-group (8 entries) stride, bytes
 constexpr uint32_t A_SBO = 128;              // A stage: MN-group (8 columns) stride, bytes
+
+// byte offset of the A stages, after sigma's Nrow targets and sink cells
+__host__ __device__ constexpr size_t rowpass_a_offset(int64_t Nrow) {
+    return (4 * (size_t)(Nrow + RP_SINK) + 1023) & ~(size_t)1023;
+}
 
 // operand scale of x (power of two): FP16 pieces of x * sa stay below 2^15
 __device__ __forceinline__ float x_scale(float mx, bool fp16) {
@@ -253,13 +254,6 @@ __device__ __forceinline__ uint16_t scale16(uint16_t bits, float sc) {
     }
 }
 
-
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t& r0, uint32_t& r1) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
-                 : "=r"(r0), "=r"(r1)
-                 : "r"(taddr)
-                 : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
@@ -318,7 +312,7 @@ __device__ __forceinline__ bool wait_phase(uint64_t* mbar, uint32_t parity, vola
 //     stage t % nst once MMA(t - nst) has released it; once they have landed
 //     (and been fenced for the async proxy), each arrives on "A full"; with
 //     them, one lane per entry prefetches that entry's rows of tile
-//     t + p.prefetch into L2 (a quarter of the gathered segments miss L2);
+//     t + p.prefetch into L2 where x does not stay there;
 //   MMA (warp 19, one thread): MMA(t) once A(t) is full and the scatter warps
 //     have released D buffer t & 1; tcgen05.commit then signals "stage free"
 //     and "D full";
@@ -327,9 +321,17 @@ __device__ __forceinline__ bool wait_phase(uint64_t* mbar, uint32_t parity, vola
 //     slot into the row's sigma in shared memory with 32-bit fixed-point
 //     atomics (order-independent: bitwise reproducible; an absent slot adds
 //     into the lane's sink cell after the row, so there is no branch).  The 4
-//     warps of a quadrant share the NS used slots evenly (chunks of 8
-//     round-robin, the remaining chunks split in pairs of slots).
-// Rows are separated by CTA barriers (set-up of the next row's B_R and sigma).
+//     warps of a quadrant take P / 4 slots each, a number known at compile time,
+//     and the tile loop is unrolled by two over two sets of table words: with the
+//     slots in use counted at run time and one set copied to another, a slot cost
+//     23 instructions (integer moves, selects, branches), three times the
+//     conversion, target and atomic it needs.
+// The copy warps know nothing of rows but their targets and run ahead across them.
+// The others meet twice between rows: after the last tile, and again once they have
+// written and cleared sigma and built the next row's B_R (its slots prefetched a row
+// ahead, its scale from k_rowscale).  At 14 orbitals the turn took 31,000 cycles, a
+// fifth of the row, with the scale, its reductions and the copies of the first tiles
+// in it.
 //
 // Fixed-point range: integer addition wraps, so only each final row sum has to
 // fit in 32 bits, and it does whenever every term |D| < 2^31 / nexc_c.  Per row
@@ -345,30 +347,21 @@ __device__ __forceinline__ bool wait_phase(uint64_t* mbar, uint32_t parity, vola
 // of the diagonal of H is added exactly by the same-spin GEMM's epilogue.
 template <int P, bool FP16, int NW, bool WIDE>
 __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
-    constexpr int MAXF = P >= 32 ? P / 32 : 1;     // full chunks per scatter warp (upper bound)
+    constexpr int SPW = P / 4;                     // slots per scatter warp
     extern __shared__ __align__(1024) unsigned char smem[];
     const int KR = p.KR;
     const int64_t Nc = p.Nc;
     const uint32_t a_piece = (uint32_t)KR * 256u;                     // one piece of one stage
     const uint32_t nst = (uint32_t)p.nst;
-    uint8_t* sA = smem;                                               // [nst stages][2 pieces]
-    uint8_t* sB = smem + 2 * nst * a_piece;                           // NW pieces of P x KR
-    const uint32_t b_piece = (uint32_t)(P * KR * 2);
     // targets held per pass: all Nc, or a span of them (wide layout)
     const int64_t Nrow = WIDE ? p.span : Nc;
-    int* srow = reinterpret_cast<int*>(sB + NW * b_piece);            // Nrow + RP_SINK, fixed point
-    int64_t* rowoff = reinterpret_cast<int64_t*>(
-        (reinterpret_cast<uintptr_t>(srow + Nrow + RP_SINK) + 15) & ~uintptr_t(15));  // [RP_MAXK]
-    uint16_t* rsl = reinterpret_cast<uint16_t*>(rowoff + RP_MAXK);    // [RP_MAXK]
-    float* rmx = reinterpret_cast<float*>(
-        (reinterpret_cast<uintptr_t>(rsl + RP_MAXK) + 15) & ~uintptr_t(15));  // [RP_MAXK]
-    float* rsc = rmx + RP_MAXK;                                       // [4] row scales
-    unsigned* rred = reinterpret_cast<unsigned*>(rsc + 4);            // [2] row reductions
-    double* wdg = reinterpret_cast<double*>(
-        (reinterpret_cast<uintptr_t>(rred + 2) + 15) & ~uintptr_t(15));  // [P] w_R (FP64)
-    uint32_t* bm = reinterpret_cast<uint32_t*>(wdg + P);   // [P] orbitals strictly inside slot s
-    uintptr_t tail = (reinterpret_cast<uintptr_t>(bm + P) + 15) & ~uintptr_t(15);
-    uint64_t* afree = reinterpret_cast<uint64_t*>(tail);   // [3] stage s free (MMA done)
+    int* srow = reinterpret_cast<int*>(smem);                         // Nrow + RP_SINK, fixed point
+    uint8_t* sA = smem + rowpass_a_offset(Nrow);                      // [nst stages][2 pieces]
+    uint8_t* sB = sA + 2 * nst * a_piece;                             // NW pieces of P x KR
+    const uint32_t b_piece = (uint32_t)(P * KR * 2);
+    uint16_t* rsl = reinterpret_cast<uint16_t*>(sB + NW * b_piece);   // [2][RP_MAXK] row slots
+    uint32_t* bm = reinterpret_cast<uint32_t*>(rsl + 2 * RP_MAXK);    // [P] orbitals inside slot s
+    uint64_t* afree = reinterpret_cast<uint64_t*>(bm + P);            // [3] stage s free (MMA done)
     uint64_t* afull = afree + 3;                           // [3] stage s copied
     uint64_t* dfull = afree + 6;                           // [2] D buffer d written
     uint64_t* dfree = afree + 8;                           // [2] D buffer d read (16 warps)
@@ -403,6 +396,22 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         tmem_alloc(tmem_holder, p.ncols);
         tmem_relinquish();
     }
+
+    // work items: (row, pass over a range of targets); one pass per row unless wide
+    const int npass = WIDE ? p.npass : 1;
+    const int64_t nitems = p.Nr * npass;
+    const int ncolk = p.rnexc + p.ndiag;                   // K columns in use
+    // slots of an item's row: off-diagonal entries, then the diagonal column (marker
+    // 0xFFFE), then padding
+    auto load_slots = [&](int64_t idx, uint16_t* dst, int e) {
+        if (e < RP_MAXK && idx < nitems) {
+            const int64_t ir = WIDE ? idx / npass : idx;
+            dst[e] = e < p.rnexc ? __ldg(p.rslot + ir * p.rnexc + e)
+                                 : (uint16_t)(e < ncolk ? 0xFFFEu : 0xFFFFu);
+        }
+    };
+    for (int64_t j = tid; j < Nrow + RP_SINK; j += RP_THREADS) srow[j] = 0;
+    load_slots(blockIdx.x, rsl, tid);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -411,143 +420,58 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
     const uint32_t sA_addr = smem_u32(sA), sB_addr = smem_u32(sB);
     const uint32_t SBO_B = 16u * (uint32_t)KR;
     const int ntiles = (int)((Nc + 127) / 128);
-    const float sa = x_scale(*p.amax, FP16);
-    const int64_t nrows = p.Nr;
-    const int ncolk = p.rnexc + p.ndiag;                   // K columns in use
-
-    // scatter geometry (warps 0-15): used chunks of 8 slots, full chunks per
-    // warp, and the remainder shared out two slots at a time
-    const int quad = warp & 3, wq = (warp >> 2) & 3;
-    const int m = quad * 32 + lane;
-    const int nchr = (p.NS + 7) / 8;
-    const int nfull = nchr / 4;
-    const int rem = nchr - 4 * nfull;                      // 0..3 chunks -> 2 rem slots per warp
-    const int tail0 = nfull * 32 + wq * 2 * rem;           // first remainder slot of this warp
 
     // tiles processed by this CTA over all rows: tile g uses A stage g % nst
     // (the k-th use of a stage completes its barriers' phase k, parity k & 1)
     // and D buffer g & 1
     uint32_t g = 0;
 
-    // work items: (row, pass over a range of targets); one pass per row unless wide
-    const int npass = WIDE ? p.npass : 1;
-    for (int64_t idx = blockIdx.x; idx < nrows * npass; idx += gridDim.x) {
-        const int64_t ir = WIDE ? idx / npass : idx;
-        const int64_t lo = WIDE ? (idx - ir * npass) * Nrow : 0;   // first target of the pass
-        // ---- row set-up: zero sigma; the row's source rows, slots and signs; B_R
-        if (tid == 0) {
-            rred[0] = 0u;
-            rred[1] = 0u;
-        }
-        for (int64_t j = tid; j < Nrow + RP_SINK; j += RP_THREADS) srow[j] = 0;
-        for (int e = tid; e < RP_MAXK; e += RP_THREADS) {
-            // off-diagonal entries, then the diagonal column (marker 0xFFFE), then padding
-            if (e < p.rnexc) {
-                const int32_t t = p.rtgt[ir * p.rnexc + e];
-                rowoff[e] = (int64_t)t * p.xpitch;
-                rsl[e] = p.rslot[ir * p.rnexc + e];
-                rmx[e] = p.rowmax[t];
-            } else if (e < ncolk) {
-                rowoff[e] = ir * p.xpitch;
-                rsl[e] = (uint16_t)0xFFFEu;
-                rmx[e] = p.rowmax[ir];
-            } else {
-                rowoff[e] = -1;
-                rsl[e] = (uint16_t)0xFFFFu;
-                rmx[e] = 0.f;
-            }
-        }
-        __syncthreads();
-        // w_R[s] in FP64; this row's fixed-point range c_s (in units of the W image;
-        // piece 0 of W is within 2^-8 of W in either format: 1 % margin) and max |B|
-        if (tid < P) {
-            double wr = 0.0;
-            for (uint32_t mk = __ldg(p.rmask + ir); mk; mk &= mk - 1)
-                wr += __ldg(p.wdiag + (size_t)(__ffs(mk) - 1) * P + tid);
-            wdg[tid] = wr;
-            const float wrs = (float)fabs(wr) * p.wscale;
-            float c = p.ndiag ? rmx[p.rnexc] * wrs : 0.f, wm = p.ndiag ? wrs : 0.f;
-            for (int e = 0; e < p.rnexc; ++e) {
-                const float w = fabsf(f16bits<FP16>(__ldg(p.wrow + (size_t)(rsl[e] & 0x7FFFu) * P + tid)));
-                c = fmaf(rmx[e], w, c);
-                wm = fmaxf(wm, w);
-            }
-            atomicMax(rred, __float_as_uint(c));
-            atomicMax(rred + 1, __float_as_uint(wm));
-        }
-        __syncthreads();
-        if (tid == 0) {
-            const float cmax = __uint_as_float(rred[0]) / p.wscale * 1.01f;
-            const float wmax = __uint_as_float(rred[1]) / p.wscale * 1.01f;
-            // each target receives at most nexc_c terms of magnitude <= cmax
-            const float bound = 1.02f * (float)p.nexc_c * cmax;
-            float fx = 1.f;
-            if (bound > 0.f && isfinite(bound)) {
-                int f;
-                frexpf(bound, &f);  // bound < 2^f
-                fx = ldexpf(1.f, 31 - max(f, -90));
-                // B_R = W fx / sa stays below 2^15 in FP16
-                if (FP16 && wmax > 0.f) {
-                    const float lim = 30000.f * sa / wmax;
-                    while (fx > lim) fx *= 0.5f;
-                }
-            }
-            rsc[0] = fx;
-            rsc[1] = fx / (sa * p.wscale);
-            rsc[2] = 1.f / fx;
-        }
-        __syncthreads();
-        const float bscale_r = rsc[1];
-        // B_R[s][e] = sgn_e W[slot e][s] bscale (NW pieces, canonical K-major layout
-        // without swizzle); the diagonal column from w_R in FP64
-        for (int i = tid; i < KR * P; i += RP_THREADS) {
-            const int e = i / P, nn = i - (i / P) * P;
-            const uint16_t r = rsl[e];
-            uint16_t v[NW];
-            if (r == 0xFFFEu) {
-                split16<FP16, NW>(wdg[nn] * (double)p.wscale * (double)bscale_r, v);
-            } else {
-#pragma unroll
-                for (int j = 0; j < NW; ++j) {
-                    v[j] = 0;
-                    if (r != 0xFFFFu) {
-                        v[j] = scale16<FP16>(__ldg(p.wrow + (size_t)j * P * P +
-                                                   (size_t)(r & 0x7FFFu) * P + nn), bscale_r);
-                        v[j] ^= (uint16_t)(r & 0x8000u);   // exact negation
-                    }
-                }
-            }
-            const uint32_t off = (uint32_t)(nn >> 3) * SBO_B + (uint32_t)(e >> 3) * 128u +
-                                 (uint32_t)(nn & 7) * 16u + (uint32_t)(e & 7) * 2u;
-#pragma unroll
-            for (int j = 0; j < NW; ++j) *reinterpret_cast<uint16_t*>(sB + j * b_piece + off) = v[j];
-        }
-        fence_proxy_async_smem();
-        __syncthreads();
-
-        if (warp >= RP_SCATTER_WARPS && warp < RP_MMA_WARP) {
-            // ---- copies: (piece, K-group) pairs u < KR / 4, u = cw + RP_COPY_WARPS i
-            // for copy warp cw; per pair this lane copies entry kc * 8 + (lane & 7),
-            // column groups (lane >> 3) + 4 v, v < 4
-            constexpr int MAXU = (RP_MAXK / 4 + RP_COPY_WARPS - 1) / RP_COPY_WARPS;
-            const int cw = warp - RP_SCATTER_WARPS;
-            const int eo = lane & 7, g0 = lane >> 3;
-            const int nu = KR / 4, kpg = KR / 8;
-            int64_t so[MAXU];                       // element offset in the piece, -1: padding
-                                                    // (beyond 2^31 at 18 orbitals)
+    if (warp >= RP_SCATTER_WARPS && warp < RP_MMA_WARP) {
+        // ---- copies: (piece, K-group) pairs u < KR / 4, u = cw + RP_COPY_WARPS i
+        // for copy warp cw; per pair this lane copies entry kc * 8 + (lane & 7),
+        // column groups (lane >> 3) + 4 v, v < 4
+        constexpr int MAXU = (RP_MAXK / 4 + RP_COPY_WARPS - 1) / RP_COPY_WARPS;
+        const int cw = warp - RP_SCATTER_WARPS;
+        const int eo = lane & 7, g0 = lane >> 3;
+        const int nu = KR / 4, kpg = KR / 8;
+        // element offset of entry e's row of x (beyond 2^31 at 18 orbitals), -1: padding
+        auto row_of = [&](int64_t ir, int e) -> int64_t {
+            if (e < p.rnexc) return (int64_t)__ldg(p.rtgt + ir * p.rnexc + e) * p.xpitch;
+            return e < ncolk ? ir * p.xpitch : -1;
+        };
+        // copies of tile gi have landed: make them visible to the tensor core
+        auto publish = [&](uint32_t gi, bool newest_pending) {
+            if (newest_pending) cp_async_wait<1>(); else cp_async_wait<0>();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(afull + gi % nst);
+        };
+        bool ok = true;
+        for (int64_t idx = blockIdx.x; idx < nitems && ok; idx += gridDim.x) {
+            const int64_t ir = WIDE ? idx / npass : idx;
+            int64_t so[MAXU];
 #pragma unroll
             for (int i = 0; i < MAXU; ++i) {
                 const int u = cw + RP_COPY_WARPS * i;
                 so[i] = -1;
                 if (u < nu) {
-                    const int kc = u < kpg ? u : u - kpg;
-                    const int64_t ro = rowoff[kc * 8 + eo];
+                    const int64_t ro = row_of(ir, (u < kpg ? u : u - kpg) * 8 + eo);
                     so[i] = ro >= 0 ? ro + 8 * g0 : -1;
                 }
             }
-            auto copies = [&](int t, uint32_t stage) {
+            // entry cw * 32 + lane: both pieces of its 128 columns (256 bytes each)
+            const int64_t pro = p.prefetch > 0 && cw * 32 + lane < KR ? row_of(ir, cw * 32 + lane) : -1;
+            for (int t = 0; t < ntiles; ++t, ++g) {
+                if (g >= nst) {
+                    // stage g % nst is free once MMA(g - nst) has completed
+                    if (lane == 0)
+                        ok = wait_phase(afree + g % nst, (g / nst - 1) & 1u, abort_flag, p.err,
+                                        p.wait_cycles, RP_BACKOFF_NS);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (!ok) break;
+                }
                 const int32_t j0 = t * 128;
-                const uint32_t st = sA_addr + stage * 2u * a_piece + (uint32_t)g0 * A_SBO +
+                const uint32_t st = sA_addr + (g % nst) * 2u * a_piece + (uint32_t)g0 * A_SBO +
                                     (uint32_t)eo * 16u;
 #pragma unroll
                 for (int i = 0; i < MAXU; ++i) {
@@ -556,223 +480,295 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
                         const bool lo = u >= kpg;
                         const int kc = lo ? u - kpg : u;
                         const uint16_t* base = lo ? p.Xl : p.Xh;
-                        const bool ok = so[i] >= 0;
-                        const uint16_t* src = base + (ok ? so[i] + j0 : 0);
+                        const bool in = so[i] >= 0;
+                        const uint16_t* src = base + (in ? so[i] + j0 : 0);
                         const uint32_t dst = st + (lo ? a_piece : 0u) + (uint32_t)kc * A_LBO;
-                        const uint32_t nb = ok ? 16u : 0u;
+                        const uint32_t nb = in ? 16u : 0u;
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
                             // column groups g0 + 4 v: 32 elements apart in x, 4 core matrices in A
                             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
                                          ::"r"(dst + (uint32_t)v * 4u * A_SBO),
-                                         "l"(src + (ok ? 32 * v : 0)), "r"(nb) : "memory");
+                                         "l"(src + (in ? 32 * v : 0)), "r"(nb) : "memory");
                         }
                     }
                 }
                 cp_async_commit();
-            };
-            // copies of tile gi have landed: make them visible to the tensor core
-            auto publish = [&](uint32_t gi, bool newest_pending) {
-                if (newest_pending) cp_async_wait<1>(); else cp_async_wait<0>();
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(afull + gi % nst);
-            };
-            bool ok = true;
-            for (int t = 0; t < ntiles && ok; ++t) {
-                const uint32_t gt = g + (uint32_t)t;
-                if (gt >= nst) {
-                    // stage gt % nst is free once MMA(gt - nst) has completed
-                    if (lane == 0)
-                        ok = wait_phase(afree + gt % nst, (gt / nst - 1) & 1u, abort_flag, p.err,
-                                        p.wait_cycles, RP_BACKOFF_NS);
-                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                    if (!ok) break;
+                if (pro >= 0 && t + p.prefetch < ntiles) {
+                    const int64_t off = pro + (int64_t)(t + p.prefetch) * 128;
+                    prefetch_l2(p.Xh + off, 256u);
+                    prefetch_l2(p.Xl + off, 256u);
                 }
-                copies(t, gt % nst);
-                if (p.prefetch > 0 && t + p.prefetch < ntiles) {
-                    // entry cw * 32 + lane: both pieces of its 128 columns (256 bytes each)
-                    const int e = cw * 32 + lane;
-                    const int64_t ro = e < KR ? rowoff[e] : -1;
-                    if (ro >= 0) {
-                        const int64_t off = ro + (int64_t)(t + p.prefetch) * 128;
-                        prefetch_l2(p.Xh + off, 256u);
-                        prefetch_l2(p.Xl + off, 256u);
-                    }
-                }
-                if (t >= 1) publish(gt - 1, true);
+                if (g >= 1) publish(g - 1, true);
             }
-            if (ok && ntiles > 0) publish(g + (uint32_t)ntiles - 1, false);
-            cp_async_wait<0>();
-        } else if (warp == RP_MMA_WARP) {
-            // ---- MMAs (one thread); with p.stall set nothing is issued or committed
-            if (lane == 0 && !p.stall) {
-                const int ksteps = KR / 16;
-                const uint64_t bdesc0 = smem_desc(sB_addr, 128u, SBO_B);
-                for (int t = 0; t < ntiles; ++t) {
-                    const uint32_t gi = g + (uint32_t)t;
-                    const uint32_t sg = gi % nst;
-                    const uint32_t st = sA_addr + sg * 2u * a_piece;
-                    const uint32_t d = tbase + (gi & 1u) * (uint32_t)P;
-                    if (!wait_phase(afull + sg, (gi / nst) & 1u, abort_flag, p.err, p.wait_cycles,
-                                    RP_BACKOFF_NS))
-                        break;
-                    if (gi >= 2 && !wait_phase(dfree + (gi & 1u), ((gi >> 1) - 1) & 1u,
-                                               abort_flag, p.err, p.wait_cycles, RP_BACKOFF_NS))
-                        break;
-                    tc_fence_after();
-                    // descriptor address fields advance by (bytes >> 4): K step = 2 K-groups
-                    // of A (2 * A_LBO bytes) and 256 bytes of B
-                    const uint64_t a_hi = smem_desc(st, A_LBO, A_SBO);
-                    const uint64_t a_lo = a_hi + (a_piece >> 4);
-                    // the small correction products first (A_lo B_0, then A_hi B_j for
-                    // j >= 1), the main product A_hi B_0 last: the accumulator rounds
-                    // each addition toward zero, so each addition should land on a
-                    // running sum as small as possible (see GM_CK in gemm_tc.cu)
+        }
+        if (ok && g >= 1) publish(g - 1, false);
+        cp_async_wait<0>();
+    } else {
+        // index among the scatter and MMA warps
+        const int rt = warp == RP_MMA_WARP ? RP_SCATTER_WARPS * 32 + lane : tid;
+        // B_R[s][e] = sgn_e W[slot e][s] bscale (NW pieces, canonical K-major layout
+        // without swizzle), two entries e at a time; the diagonal column from w_R in FP64
+        auto build_b = [&](int64_t idx, const uint16_t* sl) {
+            const int64_t ir = WIDE ? idx / npass : idx;
+            const float bscale = __ldg(&p.rscale[ir].x);
+#pragma unroll 4
+            for (int i = rt; i < KR / 2 * P; i += RP_ROW_THREADS) {
+                const int e = i / P * 2, nn = i - (i / P) * P;
+                uint32_t v[NW];
 #pragma unroll
-                    for (int q = 0; q < NW + 1; ++q) {
-                        // q = 0: A_lo B_0; 1 <= q < NW: A_hi B_q; q = NW: A_hi B_0
-                        const uint64_t ad0 = q == 0 ? a_lo : a_hi;
-                        const uint64_t bd0 = bdesc0 + (uint64_t)((q == 0 || q == NW ? 0 : q) *
-                                                                 (b_piece >> 4));
+                for (int j = 0; j < NW; ++j) v[j] = 0u;
 #pragma unroll
-                        for (int j = 0; j < RP_MAXK / 16; ++j) {
-                            if (j < ksteps)
-                                mma_ss(d, ad0 + (uint64_t)(j * (2 * A_LBO >> 4)),
-                                       bd0 + (uint64_t)(j * 16), idesc, (q | j) != 0);
+                for (int h = 0; h < 2; ++h) {
+                    const uint16_t r = sl[e + h];
+                    if (r < 0xFFFEu) {
+#pragma unroll
+                        for (int j = 0; j < NW; ++j) {
+                            const uint16_t w = scale16<FP16>(
+                                __ldg(p.wrow + (size_t)j * P * P + (size_t)(r & 0x7FFFu) * P + nn),
+                                bscale);
+                            v[j] |= (uint32_t)(w ^ (uint16_t)(r & 0x8000u)) << (16 * h);  // exact negation
                         }
+                    } else if (r == 0xFFFEu) {
+                        uint16_t w[NW];
+                        split16<FP16, NW>(__ldg(p.wr + ir * P + nn) * (double)p.wscale * (double)bscale, w);
+#pragma unroll
+                        for (int j = 0; j < NW; ++j) v[j] |= (uint32_t)w[j] << (16 * h);
                     }
-                    mma_commit(afree + sg);
-                    mma_commit(dfull + (gi & 1u));
                 }
+                const uint32_t off = (uint32_t)(nn >> 3) * SBO_B + (uint32_t)(e >> 3) * 128u +
+                                     (uint32_t)(nn & 7) * 16u + (uint32_t)(e & 7) * 2u;
+#pragma unroll
+                for (int j = 0; j < NW; ++j) *reinterpret_cast<uint32_t*>(sB + j * b_piece + off) = v[j];
             }
-            __syncwarp();
-        } else {
-            // ---- scatter
-            uint32_t w[MAXF][4], wt[3];
-            // columns past Nc (the ragged last tile) sink every slot: cell Nc + lane
-            // (the tile starts at a multiple of 128, so J mod 32 = lane)
-            // (wide layout: absent slots and ragged columns read 0xFFFF, which no range
-            // holds, so they add into the sink cell Nrow + lane)
-            const uint32_t sink = WIDE ? 0xFFFFu : (uint32_t)Nc + (uint32_t)lane;
-            const uint32_t sink2 = sink | (sink << 16);
-            uint32_t mj = 0, cmj = 0;     // wide layout: occupations of this column's string
-            auto load_words = [&](int t) {
-                const int64_t jc = (int64_t)t * 128 + m;
-                const bool in = jc < Nc;
-                const int64_t jcc = in ? jc : Nc - 1;
+        };
+        int par = 0;
+        if (blockIdx.x < nitems) build_b(blockIdx.x, rsl);
+        load_slots((int64_t)blockIdx.x + gridDim.x, rsl + RP_MAXK, rt);
+        fence_proxy_async_smem();
+        row_barrier();
+        // scatter geometry: column m of the tile, slots [wq SPW, (wq + 1) SPW)
+        const int quad = warp & 3, wq = (warp >> 2) & 3;
+        const int m = quad * 32 + lane;
+        for (int64_t idx = blockIdx.x; idx < nitems; idx += gridDim.x) {
+            const int64_t ir = WIDE ? idx / npass : idx;
+            const int64_t lo = WIDE ? (idx - ir * npass) * Nrow : 0;   // first target of the pass
+            if (warp == RP_MMA_WARP) {
+                // ---- MMAs (one thread); with p.stall set nothing is issued or committed
+                if (lane == 0 && !p.stall) {
+                    const int ksteps = KR / 16;
+                    const uint64_t bdesc0 = smem_desc(sB_addr, 128u, SBO_B);
+                    for (int t = 0; t < ntiles; ++t) {
+                        const uint32_t gi = g + (uint32_t)t;
+                        const uint32_t sg = gi % nst;
+                        const uint32_t st = sA_addr + sg * 2u * a_piece;
+                        const uint32_t d = tbase + (gi & 1u) * (uint32_t)P;
+                        if (!wait_phase(afull + sg, (gi / nst) & 1u, abort_flag, p.err, p.wait_cycles,
+                                        RP_BACKOFF_NS))
+                            break;
+                        if (gi >= 2 && !wait_phase(dfree + (gi & 1u), ((gi >> 1) - 1) & 1u,
+                                                   abort_flag, p.err, p.wait_cycles, RP_BACKOFF_NS))
+                            break;
+                        tc_fence_after();
+                        // descriptor address fields advance by (bytes >> 4): K step = 2 K-groups
+                        // of A (2 * A_LBO bytes) and 256 bytes of B
+                        const uint64_t a_hi = smem_desc(st, A_LBO, A_SBO);
+                        const uint64_t a_lo = a_hi + (a_piece >> 4);
+                        // the small correction products first (A_lo B_0, then A_hi B_j for
+                        // j >= 1), the main product A_hi B_0 last: the accumulator rounds
+                        // each addition toward zero, so each addition should land on a
+                        // running sum as small as possible (see GM_CK in gemm_tc.cu)
 #pragma unroll
-                for (int k = 0; k < MAXF; ++k) {
-                    if (k < nfull) {
-                        const uint4 v = __ldg(p.tslot8 + (int64_t)(wq + 4 * k) * Nc + jcc);
-                        w[k][0] = in ? v.x : sink2; w[k][1] = in ? v.y : sink2;
-                        w[k][2] = in ? v.z : sink2; w[k][3] = in ? v.w : sink2;
+                        for (int q = 0; q < NW + 1; ++q) {
+                            // q = 0: A_lo B_0; 1 <= q < NW: A_hi B_q; q = NW: A_hi B_0
+                            const uint64_t ad0 = q == 0 ? a_lo : a_hi;
+                            const uint64_t bd0 = bdesc0 + (uint64_t)((q == 0 || q == NW ? 0 : q) *
+                                                                     (b_piece >> 4));
+#pragma unroll
+                            for (int j = 0; j < RP_MAXK / 16; ++j) {
+                                if (j < ksteps)
+                                    mma_ss(d, ad0 + (uint64_t)(j * (2 * A_LBO >> 4)),
+                                           bd0 + (uint64_t)(j * 16), idesc, (q | j) != 0);
+                            }
+                        }
+                        mma_commit(afree + sg);
+                        mma_commit(dfull + (gi & 1u));
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    if (i < rem) {
-                        const int s0 = tail0 + 2 * i;      // even: a pair within one chunk
-                        const uint32_t* q = reinterpret_cast<const uint32_t*>(
-                            p.tslot8 + (int64_t)(s0 >> 3) * Nc + jcc);
-                        const uint32_t v = __ldg(q + ((s0 & 7) >> 1));
-                        wt[i] = in ? v : sink2;
-                    }
-                }
-                if (WIDE) mj = __ldg(p.cmask + jcc);
-            };
-            // one slot: sigma[tgt] += sign * round(D), unconditionally (an absent
-            // slot's target is this lane's sink cell)
-            auto add = [&](uint32_t word, int half, int slot, uint32_t dbits) {
-                if (WIDE) {
-                    // target within this pass's range, else the lane's sink cell; sign
-                    // from the column string's occupations inside the slot
-                    const uint32_t t = half ? (word >> 16) : (word & 0xFFFFu);
-                    const uint32_t loc = t - (uint32_t)lo;
-                    const uint32_t tg = loc < (uint32_t)Nrow ? loc : (uint32_t)Nrow + (uint32_t)lane;
-                    const uint32_t sg = (uint32_t)(__popc(cmj & bm[slot]) & 1) << 31;
-                    const int q = __float2int_rn(__uint_as_float(dbits ^ sg));
-                    atomicAdd(srow + tg, q);
-                } else {
-                    const uint32_t tg = half ? (word >> 16) & 0x7FFFu : word & 0x7FFFu;
-                    const uint32_t sg = half ? (word & 0x80000000u) : (word << 16) & 0x80000000u;
-                    const int q = __float2int_rn(__uint_as_float(dbits ^ sg));
-                    atomicAdd(srow + tg, q);
-                }
-            };
-            bool ok = true;
-            if (ntiles > 0) load_words(0);
-            for (int t = 0; t < ntiles && ok; ++t) {
-                const uint32_t gt = g + (uint32_t)t;
-                if (lane == 0)
-                    ok = wait_phase(dfull + (gt & 1u), (gt >> 1) & 1u, abort_flag, p.err,
-                                    p.wait_cycles, RP_SCATTER_BACKOFF_NS);
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t dcol = tbase + ((uint32_t)(quad * 32) << 16) +
-                                      (gt & 1u) * (uint32_t)P;
-                uint32_t dr[MAXF][8], dt[6];
-#pragma unroll
-                for (int k = 0; k < MAXF; ++k)
-                    if (k < nfull) tmem_ld8(dcol + (uint32_t)((wq + 4 * k) * 8), dr[k]);
-                // remainder: pairs of slots (tail0 is even; 4-aligned when rem == 2)
-                if (rem == 2) {
-                    uint32_t r4[8];
-                    tmem_ld4(dcol + (uint32_t)tail0, r4);
-                    dt[0] = r4[0]; dt[1] = r4[1]; dt[2] = r4[2]; dt[3] = r4[3];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 3; ++i)
-                        if (i < rem) tmem_ld2(dcol + (uint32_t)(tail0 + 2 * i), dt[2 * i], dt[2 * i + 1]);
-                }
-                tmem_ld_wait();
-                tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(dfree + (gt & 1u));
-                // this tile's words; start loading the next tile's
-                uint32_t cw[MAXF][4], ct[3];
+            } else {
+                // ---- scatter
+                uint2 wa[SPW / 4], wb[WIDE ? 1 : SPW / 4];
+                uint32_t mj = 0;      // wide layout: occupations of this column's string
+                const uint2* tw = p.tslot4 + (int64_t)wq * (SPW / 4) * p.tpitch + m;
+                auto load_words = [&](int t, uint2 (&w)[SPW / 4]) {
 #pragma unroll
-                for (int k = 0; k < MAXF; ++k)
+                    for (int k = 0; k < SPW / 4; ++k) w[k] = __ldg(tw + (int64_t)k * p.tpitch + t * 128);
+                };
+                // one slot: sigma[tgt] += sign * round(D), unconditionally (an absent
+                // slot's target is this lane's sink cell)
+                auto add = [&](uint32_t word, int half, int slot, uint32_t dbits) {
+                    if (WIDE) {
+                        // target within this pass's range, else the lane's sink cell; sign
+                        // from the column string's occupations inside the slot
+                        const uint32_t t = half ? (word >> 16) : (word & 0xFFFFu);
+                        const uint32_t loc = t - (uint32_t)lo;
+                        const uint32_t tg = loc < (uint32_t)Nrow ? loc : (uint32_t)Nrow + (uint32_t)lane;
+                        const uint32_t sg = (uint32_t)(__popc(mj & bm[slot]) & 1) << 31;
+                        atomicAdd(srow + tg, __float2int_rn(__uint_as_float(dbits ^ sg)));
+                    } else {
+                        // byte offset of the target; sign bit
+                        const uint32_t tg = half ? (word >> 14) & 0x1FFFCu : (word << 2) & 0x1FFFCu;
+                        const uint32_t sg = (half ? word : word << 16) & 0x80000000u;
+                        atomicAdd(reinterpret_cast<int*>(smem + tg),
+                                  __float2int_rn(__uint_as_float(dbits ^ sg)));
+                    }
+                };
+                bool ok = true;
+                // tile t with its words w; the next tile's words go to wn
+                auto tile = [&](int t, uint2 (&w)[SPW / 4], uint2 (&wn)[WIDE ? 1 : SPW / 4]) {
+                    const uint32_t gt = g + (uint32_t)t;
+                    if (lane == 0)
+                        ok = wait_phase(dfull + (gt & 1u), (gt >> 1) & 1u, abort_flag, p.err,
+                                        p.wait_cycles, RP_SCATTER_BACKOFF_NS);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (!ok) return;
+                    tc_fence_after();
+                    const uint32_t dcol = tbase + ((uint32_t)(quad * 32) << 16) +
+                                          (gt & 1u) * (uint32_t)P + (uint32_t)(wq * SPW);
+                    uint32_t dr[SPW];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) cw[k][i] = w[k][i];
+                    for (int k = 0; k < SPW / 4; ++k) tmem_ld4(dcol + 4u * k, dr + 4 * k);
+                    tmem_ld_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(dfree + (gt & 1u));
+                    if constexpr (!WIDE) {
+                        if (t + 1 < ntiles) load_words(t + 1, wn);
+                    } else {
+                        const int64_t jc = (int64_t)t * 128 + m;
+                        mj = __ldg(p.cmask + (jc < Nc ? jc : Nc - 1));
+                    }
 #pragma unroll
-                for (int i = 0; i < 3; ++i) ct[i] = wt[i];
-                cmj = mj;
-                if (!WIDE && t + 1 < ntiles) load_words(t + 1);
-#pragma unroll
-                for (int k = 0; k < MAXF; ++k) {
-                    if (k < nfull) {
-#pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            add(cw[k][u >> 1], u & 1, (wq + 4 * k) * 8 + u, dr[k][u]);
+                    for (int k = 0; k < SPW / 4; ++k) {
+                        add(w[k].x, 0, wq * SPW + 4 * k, dr[4 * k]);
+                        add(w[k].x, 1, wq * SPW + 4 * k + 1, dr[4 * k + 1]);
+                        add(w[k].y, 0, wq * SPW + 4 * k + 2, dr[4 * k + 2]);
+                        add(w[k].y, 1, wq * SPW + 4 * k + 3, dr[4 * k + 3]);
+                    }
+                    // (wide layout: one word set, reloaded after the adds: 160-176 slots
+                    // leave no registers for two)
+                    if (WIDE && t + 1 < ntiles) load_words(t + 1, w);
+                };
+                if (ntiles > 0) load_words(0, wa);
+                for (int t = 0; t < ntiles && ok; t += 2) {
+                    if constexpr (WIDE) {
+                        tile(t, wa, wb);
+                        if (ok && t + 1 < ntiles) tile(t + 1, wa, wb);
+                    } else {
+                        tile(t, wa, wb);
+                        if (ok && t + 1 < ntiles) tile(t + 1, wb, wa);
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    if (i < rem) {
-                        add(ct[i], 0, tail0 + 2 * i, dt[2 * i]);
-                        add(ct[i], 1, tail0 + 2 * i + 1, dt[2 * i + 1]);
-                    }
-                }
-                // (wide layout: the next tile's words after the adds, which frees the
-                // registers of one word set at 160-176 slots: 6 % faster at 18 orbitals)
-                if (WIDE && t + 1 < ntiles) load_words(t + 1);
             }
+            g += (uint32_t)ntiles;
+            row_barrier();
+            // (after an abort every wait returns at once, and the remaining rows pass
+            // without work: a break here could miss some warps, as the copy warps may
+            // abort at any time)
+            // sigma out, cleared for the next item, whose B_R is built meanwhile
+            {
+                const float inv = __ldg(&p.rscale[ir].y);
+                const int64_t nout = Nc - lo < Nrow ? Nc - lo : Nrow;   // this pass's targets
+                for (int64_t j = rt; j < Nrow; j += RP_ROW_THREADS) {
+                    if (j < nout) p.Y[ir * Nc + lo + j] = (float)srow[j] * inv;
+                    srow[j] = 0;
+                }
+                const int64_t nx = idx + gridDim.x;
+                if (nx < nitems) {
+                    build_b(nx, rsl + (par ^ 1) * RP_MAXK);
+                    load_slots(nx + gridDim.x, rsl + par * RP_MAXK, rt);
+                }
+                par ^= 1;
+                fence_proxy_async_smem();
+            }
+            row_barrier();
         }
-        g += (uint32_t)ntiles;
-        __syncthreads();
-        if (*abort_flag) break;
-        {
-            const int64_t nout = Nc - lo < Nrow ? Nc - lo : Nrow;   // this pass's targets
-            for (int64_t j = tid; j < nout; j += RP_THREADS)
-                p.Y[ir * Nc + lo + j] = (float)srow[j] * rsc[2];
-        }
-        __syncthreads();
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tbase, p.ncols);
+}
+
+// Scale of B_R and of the row's integer sums (see "Fixed-point range"), one warp per
+// row: c_s (in units of the W image; piece 0 of W is within 2^-8 of W in either
+// format: 1 % margin) and max |B| over the lanes' slots s.
+template <bool FP16>
+__global__ void __launch_bounds__(256)
+k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
+           const uint16_t* __restrict__ rslot, const uint16_t* __restrict__ wrow,
+           const double* __restrict__ wr, int64_t Nr, int rnexc, int ndiag, int P, float wscale,
+           int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
+    constexpr int SL = (176 + 31) / 32;
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (r >= Nr) return;
+    float c[SL], wm = 0.f;
+    const float own = rowmax[r];
+#pragma unroll
+    for (int u = 0; u < SL; ++u) {
+        const int s = lane + 32 * u;
+        c[u] = 0.f;
+        if (s < P && ndiag) {
+            const float w = (float)fabs(wr[r * P + s]) * wscale;
+            c[u] = own * w;
+            wm = fmaxf(wm, w);
+        }
+    }
+    for (int e0 = 0; e0 < rnexc; e0 += 32) {
+        const int e = e0 + lane;
+        const float rm = e < rnexc ? rowmax[rtgt[r * rnexc + e]] : 0.f;
+        const int sl = e < rnexc ? rslot[r * rnexc + e] & 0x7FFF : 0;
+        const int cnt = min(32, rnexc - e0);
+#pragma unroll 4
+        for (int k = 0; k < cnt; ++k) {
+            const float m = __shfl_sync(0xffffffffu, rm, k);
+            const uint16_t* row = wrow + (size_t)__shfl_sync(0xffffffffu, sl, k) * P + lane;
+#pragma unroll
+            for (int u = 0; u < SL; ++u) {
+                if (lane + 32 * u < P) {
+                    const float w = fabsf(f16bits<FP16>(__ldg(row + 32 * u)));
+                    c[u] = fmaf(m, w, c[u]);
+                    wm = fmaxf(wm, w);
+                }
+            }
+        }
+    }
+    float cm = c[0];
+#pragma unroll
+    for (int u = 1; u < SL; ++u) cm = fmaxf(cm, c[u]);
+    for (int o = 16; o > 0; o >>= 1) {
+        cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+        wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
+    }
+    if (lane != 0) return;
+    const float sa = x_scale(*amax, FP16);
+    const float cmax = cm / wscale * 1.01f;
+    const float wmax = wm / wscale * 1.01f;
+    // each target receives at most nexc_c terms of magnitude <= cmax
+    const float bound = 1.02f * (float)nexc_c * cmax;
+    float fx = 1.f;
+    if (bound > 0.f && isfinite(bound)) {
+        int f;
+        frexpf(bound, &f);  // bound < 2^f
+        fx = ldexpf(1.f, 31 - max(f, -90));
+        // B_R = W fx / sa stays below 2^15 in FP16
+        if (FP16 && wmax > 0.f) {
+            const float lim = 30000.f * sa / wmax;
+            while (fx > lim) fx *= 0.5f;
+        }
+    }
+    out[r] = make_float2(fx / (sa * wscale), 1.f / fx);
 }
 
 // max |x| of each row (rowmax[r]) and of all rows (out, float bits: non-negative
@@ -837,26 +833,27 @@ __global__ void k_wimg(const double* __restrict__ eri, int n, int P, int NS, int
 }
 
 // slot table: for string j and its entry (pq -> tgt, sgn), slot s = {p,q} holds
-// tgt | (sgn < 0) << 15; slots without an entry hold the sink ns + (j mod 32).
-// Stored per chunk of 8 slots: the 128-bit word (s/8, j) holds slots
-// 8*(s/8) .. 8*(s/8)+7, slot s in 16-bit half s%8.
+// tgt | (sgn < 0) << 15; slots without an entry, and columns [ns, pitch), hold the sink
+// ns + (j mod 32).  Stored per group of 4 slots: the 64-bit word (s/4, j) of pitch
+// words per group holds slot s in 16-bit part s%4.
 // Wide layout (wide != 0): a slot holds the target alone, 0xFFFF when absent.
-__global__ void k_slot_fill(uint16_t* __restrict__ tslot, int64_t count, int64_t ns, int wide) {
+__global__ void k_slot_fill(uint16_t* __restrict__ tslot, int64_t count, int64_t ns,
+                            int64_t pitch, int wide) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x)
-        tslot[i] = wide ? (uint16_t)0xFFFFu : (uint16_t)(ns + ((i >> 3) % ns & 31));
+        tslot[i] = wide ? (uint16_t)0xFFFFu : (uint16_t)(ns + ((i >> 2) % pitch & 31));
 }
 
 __global__ void k_slot_table(const int32_t* __restrict__ tgt, const uint16_t* __restrict__ pq,
-                             const int8_t* __restrict__ sgn, int64_t ns, int nexc, int n,
-                             uint16_t* __restrict__ tslot, int wide) {
+                             const int8_t* __restrict__ sgn, int64_t ns, int64_t pitch, int nexc,
+                             int n, uint16_t* __restrict__ tslot, int wide) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ns * nexc) return;
     const int64_t j = i / nexc;
     int a = pq[i] / n, b = pq[i] % n;
     if (a > b) { int t = a; a = b; b = t; }
     const int s = b * (b + 1) / 2 + a;
-    tslot[((int64_t)(s >> 3) * ns + j) * 8 + (s & 7)] =
+    tslot[((int64_t)(s >> 2) * pitch + j) * 4 + (s & 3)] =
         wide ? (uint16_t)tgt[i] : (uint16_t)(tgt[i] | (sgn[i] < 0 ? 0x8000 : 0));
 }
 
@@ -879,20 +876,26 @@ __global__ void k_row_offdiag(const int32_t* __restrict__ tgt, const uint16_t* _
     }
 }
 
-// wd[q][s] = W[qq][s] = (qq|pr) for slot s = {p, r}, FP64 unscaled; zero for the
-// diagonal slots (p == r), whose part of the diagonal of H is added exactly elsewhere
-__global__ void k_wdiag(const double* __restrict__ eri, int n, int P, int NS,
-                        double* __restrict__ wd) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * P) return;
-    const int q = idx / P, so = idx % P;
-    double w = 0.0;
+// w[R][s] = sum_{q in R} W[qq][s] = (qq|pr) for slot s = {p, r}, FP64 unscaled, over
+// the orbitals q of row string R ascending; zero for the diagonal slots (p == r), whose
+// part of the diagonal of H is added exactly elsewhere
+__global__ void k_wdiag(const double* __restrict__ eri, const uint32_t* __restrict__ masks, int n,
+                        int P, int NS, int64_t Nr, double* __restrict__ w) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= Nr * P) return;
+    const int64_t r = i / P;
+    const int so = (int)(i - r * P);
+    double v = 0.0;
     if (so < NS) {
         int po, qo;
         slot_pair(so, po, qo);
-        if (po != qo) w = eri[(((int64_t)q * n + q) * n + po) * n + qo];
+        if (po != qo)
+            for (uint32_t mk = masks[r]; mk; mk &= mk - 1) {
+                const int q = __ffs(mk) - 1;
+                v += __ldg(eri + (((int64_t)q * n + q) * n + po) * n + qo);
+            }
     }
-    wd[idx] = w;
+    w[i] = v;
 }
 
 // x [R][Cn] -> hi/lo BF16 pieces [R][pitch] (BF16 needs no scale); zero padding
@@ -918,9 +921,8 @@ uint32_t tmem_cols(int P) {
 
 // Nrow: targets held in shared memory (all column strings, or one pass's span)
 size_t rowpass_smem(int P, int NW, int KR, int64_t Nrow, int nst) {
-    return (size_t)2 * nst * KR * 256 + (size_t)2 * NW * P * KR + 4 * (size_t)(Nrow + RP_SINK) +
-           16 + 10 * RP_MAXK + 16 + 4 * RP_MAXK + 24 + 16 + 8 * (size_t)P + 4 * (size_t)P + 16 +
-           10 * 8 + 16;
+    return rowpass_a_offset(Nrow) + (size_t)2 * nst * KR * 256 + (size_t)2 * NW * P * KR +
+           4 * RP_MAXK + 4 * (size_t)P + 10 * 8 + 16;
 }
 
 // W in RP_NW 16-bit pieces (2: ~2^-22 relative per (pq|rs); 3: ~2^-33, a fourth
@@ -1030,8 +1032,10 @@ void TcSigma::init(const SpinTables& A, const SpinTables& B, const double* d_h1,
                 n, rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>());
             KPM_LAUNCHED();
         }
-        wdiag.alloc((size_t)n * P * sizeof(double));
-        k_wdiag<<<(n * P + 255) / 256, 256, 0, st>>>(d_eri, n, P, NS, wdiag.as<double>());
+        const int64_t nw_ = A.ns * (int64_t)P;
+        wdiag.alloc((size_t)nw_ * sizeof(double));
+        k_wdiag<<<(unsigned)((nw_ + 255) / 256), 256, 0, st>>>(
+            d_eri, A.masks.as<uint32_t>(), n, P, NS, A.ns, wdiag.as<double>());
         KPM_LAUNCHED();
     }
     err.alloc(sizeof(int));
@@ -1078,20 +1082,23 @@ void TcSigma::set_layout(int passes, cudaStream_t st) {
         KPM_THROW(KPM_EUNSUPPORTED, "tensor-core sigma: %lld targets per pass need %zu B of shared memory",
                   (long long)sp, sm);
     KPM_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const size_t count = (size_t)P * tb->ns;
+    const int64_t pitch = (tb->ns + 127) / 128 * 128;
+    const size_t count = (size_t)P * pitch;
     if (!slot_b.p || w != wide) {
         slot_b.alloc(count * sizeof(uint16_t));
-        k_slot_fill<<<1024, 256, 0, st>>>(slot_b.as<uint16_t>(), (int64_t)count, tb->ns, w ? 1 : 0);
+        k_slot_fill<<<1024, 256, 0, st>>>(slot_b.as<uint16_t>(), (int64_t)count, tb->ns,
+                                          pitch, w ? 1 : 0);
         KPM_LAUNCHED();
         const int64_t ne = tb->ns * tb->nexc;
         if (ne > 0) {
             k_slot_table<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(
                 tb->tgt.as<int32_t>(), tb->pq.as<uint16_t>(), tb->sgn.as<int8_t>(), tb->ns,
-                tb->nexc, n, slot_b.as<uint16_t>(), w ? 1 : 0);
+                pitch, tb->nexc, n, slot_b.as<uint16_t>(), w ? 1 : 0);
             KPM_LAUNCHED();
         }
     }
     kernel = kfn;
+    if (w && !wide) rp_prefetch = 4;   // (never tuned; x is far larger than L2)
     wide = w;
     npass = np;
     span = sp;
@@ -1127,6 +1134,7 @@ void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
             xh = xbh.as<uint16_t>();
             xl = xbl.as<uint16_t>();
         }
+        row_scales(am, st);
         // opposite-spin part: rows alpha, columns beta; writes Y
         launch_rowpass(xh, xl, Y, nst, rp_prefetch, st);
         // same-spin parts (dense GEMMs) and the exact diagonal, added into Y
@@ -1134,16 +1142,23 @@ void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
     }
 }
 
+void TcSigma::row_scales(const float* am, cudaStream_t st) {
+    rscale.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float2));
+    const unsigned g = (unsigned)((nsa + 7) / 8);
+    auto* fn = fp16 ? k_rowscale<true> : k_rowscale<false>;
+    fn<<<g, 256, 0, st>>>(rowmax.as<float>(), rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(),
+                          wimg.as<uint16_t>(), wdiag.as<double>(), nsa, noff, ndiag, P, wscale,
+                          tb->nexc, am, rscale.as<float2>());
+    KPM_LAUNCHED();
+}
+
 void TcSigma::launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* Y, int stages,
                              int prefetch, cudaStream_t st) {
     const uint32_t nc = tmem_cols(P);
     const int64_t xp = dense.xpitch;
-    const float* am = reinterpret_cast<const float*>(amax.p);
-    RowPass p1{xh, xl, xp, Y, nsa, nsb, slot_b.as<uint4>(),
-               rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(), noff, ndiag, KR,
-               ta->masks.as<uint32_t>(), wdiag.as<double>(),
-               wimg.as<uint16_t>(), nc, am, rowmax.as<float>(), wscale, tb->nexc, NS, stages,
-               prefetch, npass, span, tb->masks.as<uint32_t>(), err.as<int>(),
+    RowPass p1{xh, xl, xp, Y, nsa, nsb, slot_b.as<uint2>(), (nsb + 127) / 128 * 128,
+               rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(), noff, ndiag, KR, wdiag.as<double>(),
+               wimg.as<uint16_t>(), nc, rscale.as<float2>(), wscale, NS, stages, prefetch, npass, span, tb->masks.as<uint32_t>(), err.as<int>(),
                stall_next ? STALL_WAIT_CYCLES : WAIT_CYCLES, stall_next ? 1 : 0};
     stall_next = false;
     const int64_t items = nsa * (int64_t)npass;
@@ -1200,6 +1215,7 @@ void TcSigma::autotune(cudaStream_t st) {
     KPM_CUDA(cudaMemsetAsync(amax.p, 0, sizeof(unsigned), st));
     rowmax.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float));
     KPM_CUDA(cudaMemsetAsync(rowmax.p, 0, rowmax.bytes, st));
+    row_scales(reinterpret_cast<const float*>(amax.p), st);
     cudaEvent_t e0, e1;
     KPM_CUDA(cudaEventCreate(&e0));
     KPM_CUDA(cudaEventCreate(&e1));

@@ -25,16 +25,20 @@ struct TcSigma {
     int ndiag = 0;                // 1: one K column for the diagonal entries (m >= 1)
     DevBuf rslot_a;               // uint16 [N_a][noff] off-diagonal entry -> slot | sign << 15
     DevBuf rtgt_a;                // int32  [N_a][noff] off-diagonal entry -> target string
-    DevBuf wdiag;                 // double [n][P] W[qq][s] (diagonal slots zero)
+    DevBuf wdiag;                 // double [N_a][P] sum over R's orbitals q of W[qq][s] (diagonal
+                                  // slots zero)
     DevBuf xbh, xbl;              // BF16 pieces of x (KPM_MIXED_BF16; FP16 pieces live in dense)
-    DevBuf slot_b;                // uint16 [P/8][N_b][8] pair-slot -> target | sign << 15 (N_b: none)
+    DevBuf slot_b;                // uint16 [P/4][N_b up to 128][4] pair-slot -> target | sign << 15
+                                  // (N_b + J mod 32: none)
     DenseSS dense;                // same-spin parts (dense GEMMs with F_a, F_b)
     DevBuf err;                   // int error flag (1: a bounded wait ran out)
     DevBuf amax;                  // max |x| (float bits): operand scale, fixed-point range
     DevBuf rowmax;                // [N_a] max |x| per row: per-row fixed-point range of the row pass
+    DevBuf rscale;                // float2 [N_a] scales of a row (k_rowscale)
     int nst = 2;                  // A stages of the row pass (at most 3, where shared memory
                                   // allows; autotuned)
-    int rp_prefetch = 4;          // L2 prefetch distance of the row pass, tiles (autotuned)
+    int rp_prefetch = 0;          // L2 prefetch distance of the row pass, tiles (autotuned; none
+                                  // where x stays in L2: issuing it costs 3000 cycles a tile)
     // row-pass layout: plain (15-bit targets with the sign, one pass) or wide (16-bit
     // targets, sign from the column string, targets split into npass ranges of span)
     bool wide = false;
@@ -52,6 +56,8 @@ struct TcSigma {
               const double* d_eri, const float2* d_diag, int n, double wmax, double wcolsum,
               bool use_fp16, cudaStream_t st);
     void apply(const float* x, float* y, int ncol, cudaStream_t st);
+    // Scales of every row from rowmax and max|x| (am), for the next row pass.
+    void row_scales(const float* am, cudaStream_t st);
     // One row-pass launch (opposite-spin part of y, overwriting it) from the split
     // rows xh, xl, with the given A stages and prefetch distance.
     void launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* y, int stages,
