@@ -210,9 +210,10 @@ __host__ __device__ constexpr uint32_t gemm_idesc() {
 
 struct GemmArgs {
     int M, N;                  // M = N_b (m = I_b), N = N_a (n = I_a); sums over N_b, then N_a
+    int ncol;                  // columns of the block: operand rows, x and y follow one another
     float* y;                  // y[n * ldy + m] += sums / (wscale sa) + diagonal
     int64_t ldy;
-    const float* amax;         // max |x| of the split vector operand (operand scale sa)
+    const float* amax;         // [ncol] max |x| of the split vector operand (operand scale sa)
     float ratio, inv_wa;       // wscale_a / wscale_b, 1 / wscale_a (powers of two)
     // exact diagonal term (if x != nullptr): y[n*ldy+m] += d[n*ldy+m] * x[n*ldy+m], the
     // diagonal H_II evaluated in FP64 and stored as float (hi, lo)
@@ -292,7 +293,13 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     const int GROUP_M = g.group_m;
     const int nM = (g.M + GM_BM - 1) / GM_BM, nN = (g.N + GM_BN - 1) / GM_BN;
     const int nMP = (nM + GM_PAIR - 1) / GM_PAIR;
-    const int b = blockIdx.x / GM_PAIR;
+    const int per_col = nMP * nN;              // tile pairs of a column
+    const int col = blockIdx.x / GM_PAIR / per_col;
+    const int b = blockIdx.x / GM_PAIR - col * per_col;
+    const int64_t dim = (int64_t)g.N * g.ldy;
+    // rows of this column's x (n) and x^T (m) in the operands; a tile past its last row
+    // reads the next column's, which only reach sums that are not stored
+    const int xrow = col * g.N, trow_ = col * g.M;
     const int gsize = GROUP_M * nN;
     const int first_m = (b / gsize) * GROUP_M;
     const int gm = min(nMP - first_m, GROUP_M);
@@ -356,11 +363,12 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 const int kx = (beta ? kl1[kb] : kl2[kb - nk1]) * GM_BK;
                 const CUtensorMap* mA = beta ? maps.fb : maps.t;
                 const CUtensorMap* mB = beta ? maps.x : maps.fa;
-                tma_load_2d(su32(st), mA, kx, m0, &full[s]);
-                tma_load_2d(su32(st + A_BYTES), mA + 1, kx, m0, &full[s]);
+                const int ma = beta ? m0 : trow_ + m0;
+                tma_load_2d(su32(st), mA, kx, ma, &full[s]);
+                tma_load_2d(su32(st + A_BYTES), mA + 1, kx, ma, &full[s]);
                 // this CTA's half of the B rows, into both CTAs
                 const uint32_t hb = crank * B_HALF;
-                const int nh = n0 + (int)crank * (GM_BN / GM_PAIR);
+                const int nh = (beta ? xrow : 0) + n0 + (int)crank * (GM_BN / GM_PAIR);
                 tma_load_2d_mc(su32(st + 2 * A_BYTES + hb), mB, kx, nh, &full[s], 0x3);
                 tma_load_2d_mc(su32(st + 2 * A_BYTES + B_BYTES + hb), mB + 1, kx, nh, &full[s], 0x3);
                 *(volatile int*)issued = kb + 1;
@@ -444,7 +452,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
         if (ok && !*abort_flag) {
             float scale = (nchunk == nchunk1 ? g.ratio : 1.f) * g.inv_wa;
             {
-                const float mx = *g.amax;
+                const float mx = g.amax[col];
                 if (mx > 0.f && isfinite(mx)) {
                     int e;
                     frexpf(mx, &e);
@@ -463,6 +471,8 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             const int nb = n0 + h * GM_EPI_COLS;
             constexpr int EG = 16;
             const int ncols = m < g.M ? min(GM_EPI_COLS, g.N - nb) : 0;
+            float* y = g.y + col * dim;
+            const float* x = g.x + col * dim;
 #pragma unroll 1
             for (int u0 = 0; u0 < ncols; u0 += EG) {
                 const int64_t o0 = (int64_t)(nb + u0) * g.ldy + m;
@@ -472,9 +482,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 for (int u = 0; u < EG; ++u) {
                     if (u0 + u < ncols) {
                         const int64_t o = o0 + u * g.ldy;
-                        yv[u] = g.y[o];
+                        yv[u] = y[o];
                         if (g.x) {
-                            xv[u] = __ldg(g.x + o);
+                            xv[u] = __ldg(x + o);
                             dv[u] = __ldg(g.dfull + o);
                         }
                     }
@@ -485,7 +495,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                         float v = yv[u] + mine[(u0 + u) * 32] * scale;
                         // hi and lo multiply separately: the diagonal keeps its FP64 value
                         if (g.x) v = fmaf(dv[u].x, xv[u], fmaf(dv[u].y, xv[u], v));
-                        g.y[o0 + u * g.ldy] = v;
+                        y[o0 + u * g.ldy] = v;
                     }
                 }
             }
@@ -517,24 +527,24 @@ __global__ void k_absmax_offdiag(const double* __restrict__ fval, int64_t ns, in
 }
 
 // Split rows: src[r][c] (float, r < R, c < Cn, row pitch ld) -> hi/lo FP16 [r][pitch],
-// scaled by 2^(14 - e(amax)); pad columns [Cn, pitch) with zeros.  One thread per 4
+// scaled by 2^(14 - e(amax[r / per])); pad columns [Cn, pitch) with zeros.  One thread per 4
 // columns of a row (pitch a multiple of 4): two 8-byte loads where the row is 8-byte
 // aligned, one 8-byte store per piece.
 __global__ void k_split_rows(const float* __restrict__ src, int64_t R, int64_t Cn, int64_t ld,
                              __half* __restrict__ hi, __half* __restrict__ lo, int64_t pitch,
-                             const float* amax) {
-    float sa = 1.f;
-    {
-        const float mx = *amax;
-        if (mx > 0.f && isfinite(mx)) {
-            int e;
-            frexpf(mx, &e);
-            sa = ldexpf(1.f, 14 - max(e, -90));
-        }
-    }
+                             int64_t per, const float* amax) {
     const int64_t q = pitch >> 2;
     const bool v2 = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 7) == 0;
     for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
+        float sa = 1.f;
+        {
+            const float mx = amax[r / per];
+            if (mx > 0.f && isfinite(mx)) {
+                int e;
+                frexpf(mx, &e);
+                sa = ldexpf(1.f, 14 - max(e, -90));
+            }
+        }
         for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < q;
              g += (int64_t)gridDim.x * blockDim.x) {
             const int64_t c = 4 * g;
@@ -561,16 +571,19 @@ __global__ void k_split_rows(const float* __restrict__ src, int64_t R, int64_t C
     }
 }
 
-// Transposed split: dst[c][r] = src[r][c] for src R x Cn, dst rows Cn of pitch >= R
+// Transposed split of each column (blockIdx.z): dst[c][r] = src[r][c] for src R x Cn, dst rows Cn of pitch >= R
 // (pitch even, padding rows [R, pitch) written as zeros).  Tiles of 64 rows x 32
 // columns through shared memory; each thread stores two consecutive r as a half2.
 __global__ void k_split_transpose(const float* __restrict__ src, int64_t R, int64_t Cn,
                                   __half* __restrict__ hi, __half* __restrict__ lo,
                                   int64_t pitch, const float* amax) {
     __shared__ float t[64][33];
+    src += (int64_t)blockIdx.z * R * Cn;
+    hi += (int64_t)blockIdx.z * Cn * pitch;
+    lo += (int64_t)blockIdx.z * Cn * pitch;
     float sa = 1.f;
     {
-        const float mx = *amax;
+        const float mx = amax[blockIdx.z];
         if (mx > 0.f && isfinite(mx)) {
             int e;
             frexpf(mx, &e);
@@ -766,6 +779,7 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     pa = half_pitch(na);
     pb = half_pitch(nb);
     xpitch = (nb + 127) / 128 * 128;
+    cb = batch_columns(na * nb);
     err = err_flag;
     smem = GM_STAGES * STAGE_BYTES + 1024 + 256;
     KPM_CUDA(cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -789,46 +803,47 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     block_lists(A, GM_BN, kbs_a, kbl_a, &kb_nonzero[1], &kb_total[1], st);
 }
 
-void DenseSS::split(const float* x, const float* amax, cudaStream_t st) {
-    xh.ensure((size_t)na * xpitch * 2);
-    xl.ensure((size_t)na * xpitch * 2);
+void DenseSS::split(const float* x, const float* amax, int nc, cudaStream_t st) {
+    xh.ensure((size_t)cb * na * xpitch * 2);
+    xl.ensure((size_t)cb * na * xpitch * 2);
     if (xpitch & 3) KPM_THROW(KPM_EINVAL, "split rows: pitch not a multiple of 4");
-    const int64_t q = xpitch / 4;
-    dim3 gs((unsigned)((q + 255) / 256), (unsigned)(na < 65535 ? (na > 0 ? na : 1) : 65535));
-    k_split_rows<<<gs, 256, 0, st>>>(x, na, nb, nb, xh.as<__half>(), xl.as<__half>(), xpitch,
-                                       amax);
+    const int64_t q = xpitch / 4, rows = nc * na;
+    dim3 gs((unsigned)((q + 255) / 256), (unsigned)(rows < 65535 ? (rows > 0 ? rows : 1) : 65535));
+    k_split_rows<<<gs, 256, 0, st>>>(x, rows, nb, nb, xh.as<__half>(), xl.as<__half>(), xpitch,
+                                     na, amax);
     KPM_LAUNCHED();
 }
 
 // y[I_a][I_b] += sum_J Fb[I_b][J] x[I_a][J] (x rows from split())
 //             + sum_J x^T[I_b][J] Fa[I_a][J] + H_II x[I_a][I_b]
-void DenseSS::launch(const float* x, float* y, const float* amax, int group, cudaStream_t st) {
+void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int group,
+                     cudaStream_t st) {
     const float* diag = diag_full ? x : nullptr;
     GemmMaps maps;
     maps.fb[0] = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
     maps.fb[1] = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
-    maps.x[0] = make_map(xh.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
-    maps.x[1] = make_map(xl.as<__half>(), na, nb, xpitch, GM_BN / GM_PAIR);
-    maps.t[0] = make_map(th.as<__half>(), nb, na, pa, GM_BM);
-    maps.t[1] = make_map(tl.as<__half>(), nb, na, pa, GM_BM);
+    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, GM_BN / GM_PAIR);
+    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, GM_BN / GM_PAIR);
+    maps.t[0] = make_map(th.as<__half>(), nc * nb, na, pa, GM_BM);
+    maps.t[1] = make_map(tl.as<__half>(), nc * nb, na, pa, GM_BM);
     maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
     maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
-    GemmArgs g{(int)nb, (int)na, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
+    GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
                diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
                kbs_a.as<int>(), kbl_a.as<int>()};
-    k_gemm<<<gemm_grid(nb, na), GM_THREADS, smem, st>>>(maps, g);
+    k_gemm<<<nc * gemm_grid(nb, na), GM_THREADS, smem, st>>>(maps, g);
     KPM_LAUNCHED();
 }
 
-void DenseSS::apply(const float* x, float* y, const float* amax, cudaStream_t st) {
+void DenseSS::apply(const float* x, float* y, const float* amax, int nc, cudaStream_t st) {
     // transposed split copy of x (cols beta x rows alpha); the row split is xh/xl
-    th.ensure((size_t)nb * pa * 2);
-    tl.ensure((size_t)nb * pa * 2);
+    th.ensure((size_t)cb * nb * pa * 2);
+    tl.ensure((size_t)cb * nb * pa * 2);
     if (pa & 1) KPM_THROW(KPM_EINVAL, "split transpose: odd pitch");
-    dim3 tb(32, 8), gt((unsigned)((nb + 31) / 32), (unsigned)((na + 63) / 64));
+    dim3 tb(32, 8), gt((unsigned)((nb + 31) / 32), (unsigned)((na + 63) / 64), (unsigned)nc);
     k_split_transpose<<<gt, tb, 0, st>>>(x, na, nb, th.as<__half>(), tl.as<__half>(), pa, amax);
     KPM_LAUNCHED();
-    launch(x, y, amax, group_m, st);
+    launch(x, y, amax, nc, group_m, st);
 }
 
 // Picks the rasterisation group of the GEMM by timing the candidates once per
@@ -852,10 +867,10 @@ void DenseSS::autotune(cudaStream_t st) {
         }
     }
     // scratch operands (zeros: the timing does not depend on the values)
-    xh.ensure((size_t)na * xpitch * 2);
-    xl.ensure((size_t)na * xpitch * 2);
-    th.ensure((size_t)nb * pa * 2);
-    tl.ensure((size_t)nb * pa * 2);
+    xh.ensure((size_t)cb * na * xpitch * 2);
+    xl.ensure((size_t)cb * na * xpitch * 2);
+    th.ensure((size_t)cb * nb * pa * 2);
+    tl.ensure((size_t)cb * nb * pa * 2);
     KPM_CUDA(cudaMemsetAsync(xh.p, 0, xh.bytes, st));
     KPM_CUDA(cudaMemsetAsync(xl.p, 0, xl.bytes, st));
     KPM_CUDA(cudaMemsetAsync(th.p, 0, th.bytes, st));
@@ -870,7 +885,7 @@ void DenseSS::autotune(cudaStream_t st) {
     KPM_CUDA(cudaEventCreate(&e0));
     KPM_CUDA(cudaEventCreate(&e1));
     const int cand[4] = {4, 8, 16, 32};
-    auto run = [&](int gsz) { launch(ys.as<float>(), ys.as<float>(), one.as<float>(), gsz, st); };
+    auto run = [&](int gsz) { launch(ys.as<float>(), ys.as<float>(), one.as<float>(), 1, gsz, st); };
     run(group_m);  // warm-up
     float best = 0.f;
     for (int c : cand) {

@@ -7,6 +7,12 @@ namespace kpm {
 // Row pitch (elements) of an FP16 matrix with `cols` columns: 16-byte rows.
 int64_t half_pitch(int64_t cols);
 
+// Columns of a block that the tensor-core sigma takes in one set of launches: three (x, y
+// and z of a request) up to 2^24 determinants, where one column's tiles leave a last wave
+// half empty or (below 13 orbitals) most SMs idle; their split copies take 16 bytes per
+// column and determinant.
+inline int batch_columns(int64_t dim) { return dim <= ((int64_t)1 << 24) ? 3 : 1; }
+
 // sigma += F_b-part + F_a-part of H applied to x (FP32 [N_a][N_b]); see gemm_tc.cu.
 struct DenseSS {
     int64_t na = 0, nb = 0, pa = 0, pb = 0;   // strings and FP16 row pitches per spin
@@ -17,7 +23,8 @@ struct DenseSS {
     DevBuf* fa_lo = nullptr;
     DevBuf* da = nullptr;
     int64_t xpitch = 0;                       // row pitch of xh/xl: N_b rounded up to 128
-    DevBuf xh, xl, th, tl;                    // split copies of x and x^T
+    int cb = 1;                               // columns per launch (batch_columns)
+    DevBuf xh, xl, th, tl;                    // split copies of x and x^T, cb columns
     DevBuf fmax;                              // scratch for max |F_off|
     // per tile of the split matrix, the k-blocks that hold a nonzero (CSR; see
     // block_lists): F_b by pairs of 128-row tiles, F_a by 256-row tiles
@@ -33,17 +40,18 @@ struct DenseSS {
     // Builds the split matrices; `same`: alpha and beta strings are identical.
     void init(const SpinTables& A, const SpinTables& B, bool same, int* err_flag,
               cudaStream_t st);
-    // xh/xl = x split into scaled FP16 pieces [N_a][xpitch] (zero padding).
-    void split(const float* x, const float* amax, cudaStream_t st);
+    // xh/xl = nc columns of x split into scaled FP16 pieces [nc][N_a][xpitch] (zero
+    // padding); amax = device max|x| of each column.
+    void split(const float* x, const float* amax, int nc, cudaStream_t st);
     // y += (F_a (x) 1 + 1 (x) F_b) x with the off-diagonal parts of F_a, F_b, plus
     // diag_full * x (the whole exact diagonal of H); amax = device max|x|.
     // Uses xh/xl from split(x) on the same stream.
-    void apply(const float* x, float* y, const float* amax, cudaStream_t st);
+    void apply(const float* x, float* y, const float* amax, int nc, cudaStream_t st);
     // Rasterisation group (row tiles per group), chosen by autotune() at set-up; 16 by
     // default.
     int group_m = 16;
     void autotune(cudaStream_t st);
-    void launch(const float* x, float* y, const float* amax, int group, cudaStream_t st);
+    void launch(const float* x, float* y, const float* amax, int nc, int group, cudaStream_t st);
 };
 
 }  // namespace kpm

@@ -33,6 +33,7 @@
 #include <unordered_map>
 
 #include "common.cuh"
+#include "gemm_tc.cuh"
 
 using namespace kpm;
 
@@ -88,7 +89,7 @@ size_t estimate_bytes(int n, int na, int nb, int ncol, kpm_precision prec) {
     v += prec == KPM_FP64 ? 0 : (size_t)dim * 8;   // exact diagonal (hi, lo floats)
     if (prec == KPM_MIXED || prec == KPM_MIXED_BF16) {
         // split FP16 copies of x and x^T, dense split string Hamiltonians
-        v += (size_t)dim * 8 + (size_t)4 * sa * ((sa + 7) / 8 * 8);
+        v += (size_t)dim * 8 * batch_columns(dim) + (size_t)4 * sa * ((sa + 7) / 8 * 8);
         if (na != nb) v += (size_t)4 * sb * ((sb + 7) / 8 * 8);
     }
     auto tables = [&](int m, int64_t ns) {
@@ -100,7 +101,7 @@ size_t estimate_bytes(int n, int na, int nb, int ncol, kpm_precision prec) {
                                   ? 13 * nexc + 10 * n * (n - 1) / 2 + 8 * n +
                                         (prec == KPM_FP32 ? 4 * (ns + 3) : 0)
                                   : 0;
-        return (size_t)ns * (4 + 14 * nexc + 16 * nnbr + 4 * P + pairs);
+        return (size_t)ns * (4 + 14 * nexc + 16 * nnbr + 12 * P + pairs);
     };
     v += tables(na, sa) + (na == nb ? 0 : tables(nb, sb));
     v += (size_t)n * n * n * n * 12 + (64 << 20);

@@ -143,7 +143,8 @@ struct RowPass {
     const uint16_t* Xl;      // scaled by sa(amax); columns [Nc, xpitch) hold zeros
     int64_t xpitch;          // multiple of 128
     float* Y;
-    int64_t Nr, Nc;
+    int64_t Nr, Nc;          // rows and columns of one block column
+    int nblk;                // block columns (x, Y and rscale hold them one after the other)
     const uint2* tslot4;     // [P/4][tpitch]: 4 16-bit entries per group of 4 slots: target
                              // string | sign << 15, Nc + (J mod 32) when the slot of column
                              // J is absent or J is past the row
@@ -156,7 +157,7 @@ struct RowPass {
     const double* wr;        // [Nr][P] w_R[s] (unscaled, FP64)
     const uint16_t* wrow;    // W by input slot: NW pieces of [P][P] 16-bit (bits of the format)
     uint32_t ncols;          // TMEM columns allocated
-    const float2* rscale;    // [Nr] scale of B_R, scale of the row's integer sums (k_rowscale)
+    const float2* rscale;    // [nblk][Nr] scale of B_R, scale of the row's integer sums (k_rowscale)
     float wscale;            // power-of-two scale applied to W in the image
     int NS;                  // slots in use (n(n+1)/2); slots [NS, P) are padding
     int nst;                 // A stages in shared memory (2 or 3)
@@ -399,13 +400,16 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
 
     // work items: (row, pass over a range of targets); one pass per row unless wide
     const int npass = WIDE ? p.npass : 1;
-    const int64_t nitems = p.Nr * npass;
+    const int64_t nitems = p.Nr * npass * p.nblk;
+    // an item's row over all block columns, and within its own
+    auto row_all = [&](int64_t idx) { return WIDE ? idx / npass : idx; };
+    auto row_own = [&](int64_t rg) { return p.nblk == 1 ? rg : rg % p.Nr; };
     const int ncolk = p.rnexc + p.ndiag;                   // K columns in use
     // slots of an item's row: off-diagonal entries, then the diagonal column (marker
     // 0xFFFE), then padding
     auto load_slots = [&](int64_t idx, uint16_t* dst, int e) {
         if (e < RP_MAXK && idx < nitems) {
-            const int64_t ir = WIDE ? idx / npass : idx;
+            const int64_t ir = row_own(row_all(idx));
             dst[e] = e < p.rnexc ? __ldg(p.rslot + ir * p.rnexc + e)
                                  : (uint16_t)(e < ncolk ? 0xFFFEu : 0xFFFFu);
         }
@@ -434,10 +438,12 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         const int cw = warp - RP_SCATTER_WARPS;
         const int eo = lane & 7, g0 = lane >> 3;
         const int nu = KR / 4, kpg = KR / 8;
-        // element offset of entry e's row of x (beyond 2^31 at 18 orbitals), -1: padding
-        auto row_of = [&](int64_t ir, int e) -> int64_t {
-            if (e < p.rnexc) return (int64_t)__ldg(p.rtgt + ir * p.rnexc + e) * p.xpitch;
-            return e < ncolk ? ir * p.xpitch : -1;
+        // element offset of entry e's row of x for row rg (beyond 2^31 at 18 orbitals), -1:
+        // padding
+        auto row_of = [&](int64_t rg, int e) -> int64_t {
+            const int64_t ir = row_own(rg);
+            if (e < p.rnexc) return (rg - ir + __ldg(p.rtgt + ir * p.rnexc + e)) * p.xpitch;
+            return e < ncolk ? rg * p.xpitch : -1;
         };
         // copies of tile gi have landed: make them visible to the tensor core
         auto publish = [&](uint32_t gi, bool newest_pending) {
@@ -448,19 +454,19 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         };
         bool ok = true;
         for (int64_t idx = blockIdx.x; idx < nitems && ok; idx += gridDim.x) {
-            const int64_t ir = WIDE ? idx / npass : idx;
+            const int64_t rg = row_all(idx);
             int64_t so[MAXU];
 #pragma unroll
             for (int i = 0; i < MAXU; ++i) {
                 const int u = cw + RP_COPY_WARPS * i;
                 so[i] = -1;
                 if (u < nu) {
-                    const int64_t ro = row_of(ir, (u < kpg ? u : u - kpg) * 8 + eo);
+                    const int64_t ro = row_of(rg, (u < kpg ? u : u - kpg) * 8 + eo);
                     so[i] = ro >= 0 ? ro + 8 * g0 : -1;
                 }
             }
             // entry cw * 32 + lane: both pieces of its 128 columns (256 bytes each)
-            const int64_t pro = p.prefetch > 0 && cw * 32 + lane < KR ? row_of(ir, cw * 32 + lane) : -1;
+            const int64_t pro = p.prefetch > 0 && cw * 32 + lane < KR ? row_of(rg, cw * 32 + lane) : -1;
             for (int t = 0; t < ntiles; ++t, ++g) {
                 if (g >= nst) {
                     // stage g % nst is free once MMA(g - nst) has completed
@@ -510,8 +516,8 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         // B_R[s][e] = sgn_e W[slot e][s] bscale (NW pieces, canonical K-major layout
         // without swizzle), two entries e at a time; the diagonal column from w_R in FP64
         auto build_b = [&](int64_t idx, const uint16_t* sl) {
-            const int64_t ir = WIDE ? idx / npass : idx;
-            const float bscale = __ldg(&p.rscale[ir].x);
+            const int64_t rg = row_all(idx), ir = row_own(rg);
+            const float bscale = __ldg(&p.rscale[rg].x);
 #pragma unroll 4
             for (int i = rt; i < KR / 2 * P; i += RP_ROW_THREADS) {
                 const int e = i / P * 2, nn = i - (i / P) * P;
@@ -551,8 +557,8 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         const int quad = warp & 3, wq = (warp >> 2) & 3;
         const int m = quad * 32 + lane;
         for (int64_t idx = blockIdx.x; idx < nitems; idx += gridDim.x) {
-            const int64_t ir = WIDE ? idx / npass : idx;
-            const int64_t lo = WIDE ? (idx - ir * npass) * Nrow : 0;   // first target of the pass
+            const int64_t rg = row_all(idx);
+            const int64_t lo = WIDE ? (idx - rg * npass) * Nrow : 0;   // first target of the pass
             if (warp == RP_MMA_WARP) {
                 // ---- MMAs (one thread); with p.stall set nothing is issued or committed
                 if (lane == 0 && !p.stall) {
@@ -678,10 +684,10 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
             // abort at any time)
             // sigma out, cleared for the next item, whose B_R is built meanwhile
             {
-                const float inv = __ldg(&p.rscale[ir].y);
+                const float inv = __ldg(&p.rscale[rg].y);
                 const int64_t nout = Nc - lo < Nrow ? Nc - lo : Nrow;   // this pass's targets
                 for (int64_t j = rt; j < Nrow; j += RP_ROW_THREADS) {
-                    if (j < nout) p.Y[ir * Nc + lo + j] = (float)srow[j] * inv;
+                    if (j < nout) p.Y[rg * Nc + lo + j] = (float)srow[j] * inv;
                     srow[j] = 0;
                 }
                 const int64_t nx = idx + gridDim.x;
@@ -707,12 +713,14 @@ template <bool FP16>
 __global__ void __launch_bounds__(256)
 k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
            const uint16_t* __restrict__ rslot, const uint16_t* __restrict__ wrow,
-           const double* __restrict__ wr, int64_t Nr, int rnexc, int ndiag, int P, float wscale,
-           int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
+           const double* __restrict__ wr, int64_t Nr, int nblk, int rnexc, int ndiag, int P,
+           float wscale, int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
     constexpr int SL = (176 + 31) / 32;
-    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t rg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (r >= Nr) return;
+    if (rg >= Nr * nblk) return;
+    const int64_t blk = rg / Nr, r = rg - blk * Nr;
+    rowmax += blk * Nr;
     float c[SL], wm = 0.f;
     const float own = rowmax[r];
 #pragma unroll
@@ -752,7 +760,7 @@ k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
         wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
     }
     if (lane != 0) return;
-    const float sa = x_scale(*amax, FP16);
+    const float sa = x_scale(amax[blk], FP16);
     const float cmax = cm / wscale * 1.01f;
     const float wmax = wm / wscale * 1.01f;
     // each target receives at most nexc_c terms of magnitude <= cmax
@@ -768,12 +776,12 @@ k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
             while (fx > lim) fx *= 0.5f;
         }
     }
-    out[r] = make_float2(fx / (sa * wscale), 1.f / fx);
+    out[rg] = make_float2(fx / (sa * wscale), 1.f / fx);
 }
 
-// max |x| of each row (rowmax[r]) and of all rows (out, float bits: non-negative
-// floats order like unsigned integers)
-__global__ void k_rowmax(const float* __restrict__ x, int64_t nrow, int64_t ncol,
+// max |x| of each row (rowmax[r]) and of the rows of each block column of `per` rows
+// (out[r / per], float bits: non-negative floats order like unsigned integers)
+__global__ void k_rowmax(const float* __restrict__ x, int64_t nrow, int64_t ncol, int64_t per,
                          float* __restrict__ rowmax, unsigned* out) {
     __shared__ float wmx[8];
     for (int64_t r = blockIdx.x; r < nrow; r += gridDim.x) {
@@ -786,7 +794,7 @@ __global__ void k_rowmax(const float* __restrict__ x, int64_t nrow, int64_t ncol
             float m = wmx[0];
             for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, wmx[w]);
             rowmax[r] = m;
-            atomicMax(out, __float_as_uint(m));
+            atomicMax(out + r / per, __float_as_uint(m));
         }
         __syncthreads();
     }
@@ -1039,7 +1047,7 @@ void TcSigma::init(const SpinTables& A, const SpinTables& B, const double* d_h1,
         KPM_LAUNCHED();
     }
     err.alloc(sizeof(int));
-    amax.alloc(2 * sizeof(unsigned));
+    amax.alloc(batch_columns(dim) * sizeof(unsigned));
     KPM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
     dense.init(A, B, &A == &B, err.as<int>(), st);
     dense.diag_full = d_diag;
@@ -1108,60 +1116,63 @@ void TcSigma::set_layout(int passes, cudaStream_t st) {
 
 void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
     const int64_t xp = dense.xpitch;
-    for (int c = 0; c < ncol; ++c) {
+    const int cb = dense.cb;
+    rowmax.ensure((size_t)(nsa > 0 ? cb * nsa : 1) * sizeof(float));
+    for (int c = 0; c < ncol; c += cb) {
+        const int nc = ncol - c < cb ? ncol - c : cb;
+        const int64_t rows = nc * nsa;
         const float* X = x + (size_t)c * dim;
         float* Y = y + (size_t)c * dim;
         // max|x|: FP16 operand scales and the fixed-point range of the scatter
-        KPM_CUDA(cudaMemsetAsync(amax.p, 0, sizeof(unsigned), st));
-        rowmax.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float));
+        KPM_CUDA(cudaMemsetAsync(amax.p, 0, nc * sizeof(unsigned), st));
         {
-            const int64_t g = nsa < (int64_t)nsm * 8 ? nsa : (int64_t)nsm * 8;
-            k_rowmax<<<(unsigned)(g > 0 ? g : 1), 256, 0, st>>>(X, nsa, nsb, rowmax.as<float>(),
+            const int64_t g = rows < (int64_t)nsm * 8 ? rows : (int64_t)nsm * 8;
+            k_rowmax<<<(unsigned)(g > 0 ? g : 1), 256, 0, st>>>(X, rows, nsb, nsa, rowmax.as<float>(),
                                                                 amax.as<unsigned>());
         }
         KPM_LAUNCHED();
         const float* am = reinterpret_cast<const float*>(amax.p);
         // split x: the FP16 pieces serve the row pass and the beta GEMM
-        dense.split(X, am, st);
+        dense.split(X, am, nc, st);
         const uint16_t* xh = dense.xh.as<uint16_t>();
         const uint16_t* xl = dense.xl.as<uint16_t>();
         if (!fp16) {
-            xbh.ensure((size_t)nsa * xp * 2);
-            xbl.ensure((size_t)nsa * xp * 2);
-            k_split_rows_bf16<<<2048, 256, 0, st>>>(X, nsa, nsb, xbh.as<uint16_t>(),
+            xbh.ensure((size_t)cb * nsa * xp * 2);
+            xbl.ensure((size_t)cb * nsa * xp * 2);
+            k_split_rows_bf16<<<2048, 256, 0, st>>>(X, rows, nsb, xbh.as<uint16_t>(),
                                                     xbl.as<uint16_t>(), xp);
             KPM_LAUNCHED();
             xh = xbh.as<uint16_t>();
             xl = xbl.as<uint16_t>();
         }
-        row_scales(am, st);
+        row_scales(am, nc, st);
         // opposite-spin part: rows alpha, columns beta; writes Y
-        launch_rowpass(xh, xl, Y, nst, rp_prefetch, st);
+        launch_rowpass(xh, xl, Y, nc, nst, rp_prefetch, st);
         // same-spin parts (dense GEMMs) and the exact diagonal, added into Y
-        dense.apply(X, Y, am, st);
+        dense.apply(X, Y, am, nc, st);
     }
 }
 
-void TcSigma::row_scales(const float* am, cudaStream_t st) {
-    rscale.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float2));
-    const unsigned g = (unsigned)((nsa + 7) / 8);
+void TcSigma::row_scales(const float* am, int nc, cudaStream_t st) {
+    rscale.ensure((size_t)(nsa > 0 ? dense.cb * nsa : 1) * sizeof(float2));
+    const unsigned g = (unsigned)((nc * nsa + 7) / 8);
     auto* fn = fp16 ? k_rowscale<true> : k_rowscale<false>;
     fn<<<g, 256, 0, st>>>(rowmax.as<float>(), rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(),
-                          wimg.as<uint16_t>(), wdiag.as<double>(), nsa, noff, ndiag, P, wscale,
+                          wimg.as<uint16_t>(), wdiag.as<double>(), nsa, nc, noff, ndiag, P, wscale,
                           tb->nexc, am, rscale.as<float2>());
     KPM_LAUNCHED();
 }
 
-void TcSigma::launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* Y, int stages,
+void TcSigma::launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* Y, int nc, int stages,
                              int prefetch, cudaStream_t st) {
-    const uint32_t nc = tmem_cols(P);
+    const uint32_t tcols = tmem_cols(P);
     const int64_t xp = dense.xpitch;
-    RowPass p1{xh, xl, xp, Y, nsa, nsb, slot_b.as<uint2>(), (nsb + 127) / 128 * 128,
+    RowPass p1{xh, xl, xp, Y, nsa, nsb, nc, slot_b.as<uint2>(), (nsb + 127) / 128 * 128,
                rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(), noff, ndiag, KR, wdiag.as<double>(),
-               wimg.as<uint16_t>(), nc, rscale.as<float2>(), wscale, NS, stages, prefetch, npass, span, tb->masks.as<uint32_t>(), err.as<int>(),
+               wimg.as<uint16_t>(), tcols, rscale.as<float2>(), wscale, NS, stages, prefetch, npass, span, tb->masks.as<uint32_t>(), err.as<int>(),
                stall_next ? STALL_WAIT_CYCLES : WAIT_CYCLES, stall_next ? 1 : 0};
     stall_next = false;
-    const int64_t items = nsa * (int64_t)npass;
+    const int64_t items = nc * nsa * (int64_t)npass;
     int g1 = (int)(items < nsm ? items : nsm);
     void* args1[] = {&p1};
     if (prof) {
@@ -1215,7 +1226,7 @@ void TcSigma::autotune(cudaStream_t st) {
     KPM_CUDA(cudaMemsetAsync(amax.p, 0, sizeof(unsigned), st));
     rowmax.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float));
     KPM_CUDA(cudaMemsetAsync(rowmax.p, 0, rowmax.bytes, st));
-    row_scales(reinterpret_cast<const float*>(amax.p), st);
+    row_scales(reinterpret_cast<const float*>(amax.p), 1, st);
     cudaEvent_t e0, e1;
     KPM_CUDA(cudaEventCreate(&e0));
     KPM_CUDA(cudaEventCreate(&e1));
@@ -1225,14 +1236,14 @@ void TcSigma::autotune(cudaStream_t st) {
     const int pfs[3] = {0, 4, 8};
     float best = 0.f;
     int bst = nst, bpf = rp_prefetch;
-    launch_rowpass(zh.as<uint16_t>(), zl.as<uint16_t>(), y.as<float>(), nst, rp_prefetch, st);
+    launch_rowpass(zh.as<uint16_t>(), zl.as<uint16_t>(), y.as<float>(), 1, nst, rp_prefetch, st);
     for (int stg = 2; stg <= maxst; ++stg) {
         for (int pf : pfs) {
             // the faster of two launches
             float ms = 0.f;
             for (int rep = 0; rep < 2; ++rep) {
                 KPM_CUDA(cudaEventRecord(e0, st));
-                launch_rowpass(zh.as<uint16_t>(), zl.as<uint16_t>(), y.as<float>(), stg, pf, st);
+                launch_rowpass(zh.as<uint16_t>(), zl.as<uint16_t>(), y.as<float>(), 1, stg, pf, st);
                 KPM_CUDA(cudaEventRecord(e1, st));
                 KPM_CUDA(cudaEventSynchronize(e1));
                 float t = 0.f;

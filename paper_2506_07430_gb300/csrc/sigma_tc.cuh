@@ -57,10 +57,10 @@ struct TcSigma {
               bool use_fp16, cudaStream_t st);
     void apply(const float* x, float* y, int ncol, cudaStream_t st);
     // Scales of every row from rowmax and max|x| (am), for the next row pass.
-    void row_scales(const float* am, cudaStream_t st);
-    // One row-pass launch (opposite-spin part of y, overwriting it) from the split
-    // rows xh, xl, with the given A stages and prefetch distance.
-    void launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* y, int stages,
+    void row_scales(const float* am, int nc, cudaStream_t st);
+    // One row-pass launch (opposite-spin part of nc columns of y, overwriting it) from the
+    // split rows xh, xl, with the given A stages and prefetch distance.
+    void launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* y, int nc, int stages,
                         int prefetch, cudaStream_t st);
     // Times the row pass's stages x prefetch candidates once per device and shape.
     void autotune(cudaStream_t st);
