@@ -206,7 +206,7 @@ void dipole_dispatch(kpm_ctx* c, int comp, const double* psi, void* y) {
 }
 
 void update_dispatch(kpm_ctx* c, const void* s, const void* cur, void* prev, int first,
-                     double* dots, const unsigned* step) {
+                     double* dots, unsigned* step) {
     int64_t dstride = (int64_t)c->rec_max_steps * 2;
     if (c->prec == KPM_FP64)
         cheb_update_f64((const double*)s, (const double*)cur, (double*)prev, c->dim, c->rec_ncol,
@@ -346,7 +346,6 @@ void step_direct(kpm_ctx* c) {
     }
     update_dispatch(c, c->vS.p, c->rec_cur, c->rec_prev, 0, c->dots.as<double>(),
                     c->step_ctr.as<unsigned>());
-    step_inc(c->step_ctr.as<unsigned>(), c->st);
     std::swap(c->rec_prev, c->rec_cur);
     ++c->rec_steps;
 }
@@ -761,7 +760,7 @@ kpm_status kpm_bounds(kpm_ctx* ctx, int iters, uint64_t seed, double* emin, doub
         ctx->lz_v0.ensure(vb);
         ctx->lz_v1.ensure(vb);
         ctx->lz_w.ensure(vb);
-        ctx->lz_ab.ensure(sizeof(double) * (5 * (k + 1)));
+        ctx->lz_ab.ensure(sizeof(double) * (8 * (k + 1)));
         ctx->lz_scalar.ensure(sizeof(double) * 8);
         ensure_reduce_scratch(ctx, 1);
         double* al = ctx->lz_ab.as<double>();

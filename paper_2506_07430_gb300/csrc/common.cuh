@@ -93,7 +93,8 @@ struct SpinTables {
     DevBuf masks;            // uint32 [ns]
     DevBuf tgt, pq, sgn;     // int32/uint16/int8 [ns][nexc]  (API layout)
     DevBuf tgtT, pqT, sgnT;  // int32/uint16/int8 [nexc][ns]  (string-fastest, coalesced)
-    DevBuf pkT;              // uint32 [nexc][ns]: target | pq << 16 | (sign < 0) << 31
+    DevBuf pkT;              // uint32 [m (n - m)][ns]: off-diagonal entries, target |
+                             // (pq + (sign < 0 ? n n : 0)) << 16
     DevBuf fcol;             // int32  [nnbr][ns]  same-spin string Hamiltonian columns
     DevBuf fval64;           // double [nnbr][ns]
     DevBuf fval32;           // float  [nnbr][ns]
@@ -261,17 +262,17 @@ int reduce_blocks(int64_t dim);
 // alpha_next = first ? (s - b c)/a : 2 (s - b c)/a - prev, written over prev;
 // dots[col*stride + 0] = <c|c>, dots[col*stride + 1] = <next|c> (FP64).
 // dots of the step go to dots[2n], dots[2n+1] (per column, stride dots_col_stride),
-// n = *step when step is non-null (device counter), else n = 0 at `dots`.
+// n = *step when step is non-null (device counter, moved on by one at the end of the
+// update; counters holds ncol + 1 zeroed words), else n = 0 at `dots`.
 void cheb_update_f64(const double* s, const double* c, double* prev, int64_t dim, int ncol,
                      double a, double b, int first, double* partials, unsigned* counters,
-                     double* dots, int64_t dots_col_stride, const unsigned* step,
+                     double* dots, int64_t dots_col_stride, unsigned* step,
                      cudaStream_t st);
 void cheb_update_f32(const float* s, const float* c, float* prev, int64_t dim, int ncol,
                      double a, double b, int first, double* partials, unsigned* counters,
-                     double* dots, int64_t dots_col_stride, const unsigned* step,
+                     double* dots, int64_t dots_col_stride, unsigned* step,
                      cudaStream_t st);
 void step_set(unsigned* step, unsigned v, cudaStream_t st);
-void step_inc(unsigned* step, cudaStream_t st);
 
 // moments[col][2n], [2n+1] from dots[col][n][2] (doubling identities); with defl
 // (deflated recursions) defl[col] T_n(x0) is added to moment n.
@@ -299,7 +300,7 @@ void lanczos_scale(void* vnext, const void* w, int64_t dim, bool f64, const doub
                    double* beta_out, cudaStream_t st);
 void fill_random(void* v, int64_t dim, bool f64, uint64_t seed, cudaStream_t st);
 void scale_inplace(void* v, int64_t dim, bool f64, const double* norm2, cudaStream_t st);
-// scratch: 3k doubles of device memory.
+// scratch: 6k doubles of device memory.
 void tridiag_extremes(const double* alpha, const double* beta, int k, double* out4,
                       double* scratch, cudaStream_t st);
 

@@ -21,8 +21,10 @@ namespace kpm {
 static constexpr int RED_THREADS = 256;
 static constexpr int RED_MAX_BLOCKS = 1216;  // 8 x 152, fixed for determinism
 
+// Two elements a thread: with eight, a vector of 4,900 (8 orbitals) ran on 3 blocks and
+// its step's update took 12 us, most of it the latency of eight loads in turn.
 int reduce_blocks(int64_t dim) {
-    int64_t b = (dim + RED_THREADS * 8 - 1) / (RED_THREADS * 8);
+    int64_t b = (dim + RED_THREADS * 2 - 1) / (RED_THREADS * 2);
     if (b < 1) b = 1;
     if (b > RED_MAX_BLOCKS) b = RED_MAX_BLOCKS;
     return (int)b;
@@ -50,8 +52,9 @@ __device__ __forceinline__ void block_sum2(double& u, double& v) {
 }
 
 // Stores the partials of block blk (of nblk); the last block to finish sums
-// them in a fixed order into out[0], out[1] and re-arms the counter.
-__device__ __forceinline__ void finish_reduce(double u, double v, double* partials,
+// them in a fixed order into out[0], out[1], re-arms the counter and returns true in its
+// thread 0.
+__device__ __forceinline__ bool finish_reduce(double u, double v, double* partials,
                                               unsigned* counter, int nblk, int blk, double* out0,
                                               double* out1) {
     block_sum2(u, v);
@@ -64,7 +67,7 @@ __device__ __forceinline__ void finish_reduce(double u, double v, double* partia
         last = (prev == (unsigned)nblk - 1);
     }
     __syncthreads();
-    if (!last) return;
+    if (!last) return false;
     __threadfence();
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
@@ -77,13 +80,14 @@ __device__ __forceinline__ void finish_reduce(double u, double v, double* partia
         if (out1) *out1 = b;
         *counter = 0u;
     }
+    return threadIdx.x == 0;
 }
 
 // Block blk (of nblk) of column col of the update; dots of step n go to
 // dots[2n], dots[2n+1].  Shared by the single-molecule kernel and the batched
 // one, so that both do the same arithmetic and reduction.
 template <class T>
-__device__ __forceinline__ void cheb_update_cta(int blk, int nblk, int col,
+__device__ __forceinline__ bool cheb_update_cta(int blk, int nblk, int col,
                                                 const T* __restrict__ s, const T* __restrict__ c,
                                                 T* __restrict__ prev, int64_t dim, double a,
                                                 double b, int first, double* partials,
@@ -132,19 +136,28 @@ __device__ __forceinline__ void cheb_update_cta(int blk, int nblk, int col,
             tt += (double)gt;
         }
     }
-    finish_reduce(ss, tt, partials + (int64_t)col * 2 * nblk, counters + col, nblk, blk,
-                  dots + col * dstride, dots + col * dstride + 1);
+    return finish_reduce(ss, tt, partials + (int64_t)col * 2 * nblk, counters + col, nblk, blk,
+                         dots + col * dstride, dots + col * dstride + 1);
 }
 
 template <class T>
 __global__ void __launch_bounds__(RED_THREADS)
 k_cheb_update(const T* __restrict__ s, const T* __restrict__ c, T* __restrict__ prev, int64_t dim,
               double a, double b, int first, double* partials, unsigned* counters, double* dots,
-              int64_t dstride, const unsigned* step) {
+              int64_t dstride, unsigned* step) {
     // n from the device counter if given (replayable captured steps), else 0
     const int64_t n = step ? (int64_t)(*step) : 0;
-    cheb_update_cta<T>(blockIdx.x, gridDim.x, blockIdx.y, s, c, prev, dim, a, b, first, partials,
-                       counters, dots, dstride, n);
+    const bool last = cheb_update_cta<T>(blockIdx.x, gridDim.x, blockIdx.y, s, c, prev, dim, a, b,
+                                         first, partials, counters, dots, dstride, n);
+    // the column that finishes last moves the counter on: every block has read it
+    if (last && step) {
+        __threadfence();
+        unsigned* columns = counters + gridDim.y;
+        if (atomicAdd(columns, 1u) == gridDim.y - 1) {
+            *columns = 0u;
+            *step = (unsigned)n + 1u;
+        }
+    }
 }
 
 // Batched non-first update: the flattened grid covers every molecule's
@@ -189,7 +202,7 @@ void cheb_update_batch_f32(const BatchMol* mols, int nmol, int64_t blocks, int k
 template <class T>
 static void launch_update(const T* s, const T* c, T* prev, int64_t dim, int ncol, double a,
                           double b, int first, double* partials, unsigned* counters, double* dots,
-                          int64_t dstride, const unsigned* step, cudaStream_t st) {
+                          int64_t dstride, unsigned* step, cudaStream_t st) {
     dim3 grid(reduce_blocks(dim), ncol);
     k_cheb_update<T><<<grid, RED_THREADS, 0, st>>>(s, c, prev, dim, a, b, first, partials,
                                                    counters, dots, dstride, step);
@@ -198,28 +211,23 @@ static void launch_update(const T* s, const T* c, T* prev, int64_t dim, int ncol
 
 void cheb_update_f64(const double* s, const double* c, double* prev, int64_t dim, int ncol,
                      double a, double b, int first, double* partials, unsigned* counters,
-                     double* dots, int64_t dstride, const unsigned* step, cudaStream_t st) {
+                     double* dots, int64_t dstride, unsigned* step, cudaStream_t st) {
     launch_update<double>(s, c, prev, dim, ncol, a, b, first, partials, counters, dots, dstride,
                           step, st);
 }
 void cheb_update_f32(const float* s, const float* c, float* prev, int64_t dim, int ncol, double a,
                      double b, int first, double* partials, unsigned* counters, double* dots,
-                     int64_t dstride, const unsigned* step, cudaStream_t st) {
+                     int64_t dstride, unsigned* step, cudaStream_t st) {
     launch_update<float>(s, c, prev, dim, ncol, a, b, first, partials, counters, dots, dstride,
                          step, st);
 }
 
 __global__ void k_step_set(unsigned* step, unsigned v) { *step = v; }
-__global__ void k_step_inc(unsigned* step) { *step += 1u; }
 
 // device-side step counter of the recursion (read by k_cheb_update), so that a
 // captured step is replayable
 void step_set(unsigned* step, unsigned v, cudaStream_t st) {
     k_step_set<<<1, 1, 0, st>>>(step, v);
-    KPM_LAUNCHED();
-}
-void step_inc(unsigned* step, cudaStream_t st) {
-    k_step_inc<<<1, 1, 0, st>>>(step);
     KPM_LAUNCHED();
 }
 
@@ -439,9 +447,12 @@ void fill_random(void* v, int64_t dim, bool f64, uint64_t seed, cudaStream_t st)
 }
 
 // Extreme eigenvalues of the k x k symmetric tridiagonal T (diagonal alpha[0..k),
-// off-diagonal beta[0..k-1)) by Sturm-sequence bisection, and the Ritz residual
-// estimates |beta[k-1] * (last component of the unit eigenvector)|.
-// out4 = {theta_min, theta_max, res_min, res_max}.  One thread.
+// off-diagonal beta[0..k-1)) by Sturm counts, and the Ritz residual estimates
+// |beta[k-1] * (last component of the unit eigenvector)|.
+// out4 = {theta_min, theta_max, res_min, res_max}.  A Sturm count is a chain of k FP64
+// divisions, so a warp takes 32 shifts at a time (11 rounds to the last bit instead of
+// 55) and each end of the spectrum has a warp of its own: 40 steps, 2624 us in one thread
+// with bisection, 446 us here.
 __device__ int sturm_below(const double* al, const double* be, int k, double x) {
     int cnt = 0;
     double q = 1.0;
@@ -454,11 +465,23 @@ __device__ int sturm_below(const double* al, const double* be, int k, double x) 
     return cnt;
 }
 
+// (one warp) eigenvalue number idx in [lo, hi], to neighbouring doubles
 __device__ double tri_eig(const double* al, const double* be, int k, int idx, double lo, double hi) {
+    const int lane = threadIdx.x & 31;
     for (int it = 0; it < 200; ++it) {
-        double mid = 0.5 * (lo + hi);
+        const double mid = 0.5 * (lo + hi);
         if (mid <= lo || mid >= hi) break;
-        if (sturm_below(al, be, k, mid) > idx) hi = mid; else lo = mid;
+        // 32 shifts inside; where fewer doubles are left, all bisect
+        double x = lo + (hi - lo) * ((lane + 1) / 33.0);
+        const bool fine = __all_sync(0xffffffffu, x > lo && x < hi);
+        if (!fine) x = mid;
+        const unsigned above = __ballot_sync(0xffffffffu, sturm_below(al, be, k, x) > idx);
+        // first shift with the eigenvalue below it (32: none)
+        const int f = above ? __ffs(above) - 1 : 32;
+        const double xh = __shfl_sync(0xffffffffu, x, f & 31);
+        const double xl = __shfl_sync(0xffffffffu, x, (f + 31) & 31);
+        if (f < 32) hi = xh;
+        if (f > 0) lo = xl;
     }
     return 0.5 * (lo + hi);
 }
@@ -497,9 +520,23 @@ __device__ double last_component(const double* al, const double* be, int k, doub
     return fabs(x[k - 1]);
 }
 
-__global__ void k_tridiag(const double* al, const double* be, int k, double* out, double* w) {
-    if (threadIdx.x || blockIdx.x) return;
-    double lo = al[0], hi = al[0];
+// T in shared memory where it fits
+constexpr int TRI_SMEM = 2048;
+__device__ void tri_stage(const double*& al, const double*& be, int k, double* sa, double* sb) {
+    if (k > TRI_SMEM) return;
+    for (int i = threadIdx.x; i < k; i += blockDim.x) {
+        sa[i] = al[i];
+        sb[i] = be[i];
+    }
+    __syncthreads();
+    al = sa;
+    be = sb;
+}
+
+// Gershgorin bounds of the spectrum, widened
+__device__ void tri_bounds(const double* al, const double* be, int k, double& lo, double& hi) {
+    lo = al[0];
+    hi = al[0];
     for (int i = 0; i < k; ++i) {
         double r = (i ? fabs(be[i - 1]) : 0.0) + (i + 1 < k ? fabs(be[i]) : 0.0);
         lo = fmin(lo, al[i] - r);
@@ -507,36 +544,37 @@ __global__ void k_tridiag(const double* al, const double* be, int k, double* out
     }
     lo -= 1e-9 * (1.0 + fabs(lo));
     hi += 1e-9 * (1.0 + fabs(hi));
-    double tmin = tri_eig(al, be, k, 0, lo, hi);
-    double tmax = tri_eig(al, be, k, k - 1, lo, hi);
-    double bk = fabs(be[k - 1]);
-    out[0] = tmin;
-    out[1] = tmax;
-    out[2] = bk * last_component(al, be, k, tmin, w);
-    out[3] = bk * last_component(al, be, k, tmax, w);
+}
+
+__global__ void __launch_bounds__(64)
+k_tridiag(const double* al, const double* be, int k, double* out, double* w) {
+    __shared__ double sa[TRI_SMEM], sb[TRI_SMEM];
+    tri_stage(al, be, k, sa, sb);
+    double lo, hi;
+    tri_bounds(al, be, k, lo, hi);
+    const int end = threadIdx.x >> 5;    // 0: lowest, 1: highest
+    const double th = tri_eig(al, be, k, end ? k - 1 : 0, lo, hi);
+    if (threadIdx.x & 31) return;
+    out[end] = th;
+    out[2 + end] = fabs(be[k - 1]) * last_component(al, be, k, th, w + (size_t)end * 3 * k);
 }
 
 void tridiag_extremes(const double* alpha, const double* beta, int k, double* out4,
                       double* scratch, cudaStream_t st) {
-    k_tridiag<<<1, 1, 0, st>>>(alpha, beta, k, out4, scratch);
+    k_tridiag<<<1, 64, 0, st>>>(alpha, beta, k, out4, scratch);
     KPM_LAUNCHED();
 }
 
-// Lowest eigenpair of the k x k symmetric tridiagonal T: theta by Sturm
-// bisection, its unit eigenvector s by inverse iteration with the tridiagonal
+// Lowest eigenpair of the k x k symmetric tridiagonal T: theta by Sturm counts, its unit eigenvector s by inverse iteration with the tridiagonal
 // (Thomas) solver, shifted just below theta.  out[0] = theta, s_out[0..k).
-__global__ void k_tridiag_lowest(const double* al, const double* be, int k, double* out,
+__global__ void __launch_bounds__(32) k_tridiag_lowest(const double* al, const double* be, int k, double* out,
                                  double* s_out, double* w) {
-    if (threadIdx.x || blockIdx.x) return;
-    double lo = al[0], hi = al[0];
-    for (int i = 0; i < k; ++i) {
-        double r = (i ? fabs(be[i - 1]) : 0.0) + (i + 1 < k ? fabs(be[i]) : 0.0);
-        lo = fmin(lo, al[i] - r);
-        hi = fmax(hi, al[i] + r);
-    }
-    lo -= 1e-9 * (1.0 + fabs(lo));
-    hi += 1e-9 * (1.0 + fabs(hi));
+    __shared__ double sa[TRI_SMEM], sb[TRI_SMEM];
+    tri_stage(al, be, k, sa, sb);
+    double lo, hi;
+    tri_bounds(al, be, k, lo, hi);
     const double th = tri_eig(al, be, k, 0, lo, hi);
+    if (threadIdx.x) return;
     double* c = w;
     double* d = w + k;
     double scale = 0.0;
@@ -570,7 +608,7 @@ __global__ void k_tridiag_lowest(const double* al, const double* be, int k, doub
 
 void tridiag_lowest(const double* alpha, const double* beta, int k, double* theta, double* s,
                     double* scratch, cudaStream_t st) {
-    k_tridiag_lowest<<<1, 1, 0, st>>>(alpha, beta, k, theta, s, scratch);
+    k_tridiag_lowest<<<1, 32, 0, st>>>(alpha, beta, k, theta, s, scratch);
     KPM_LAUNCHED();
 }
 
