@@ -6,7 +6,7 @@
 // sinh(lambda) of the KPM review the paper cites (the Methods name "modified
 // kernels like the Jackson kernel"; Lorentz broadening suits Green's functions).
 // This is a type-III discrete cosine transform of the damped moments, evaluated as a
-// direct FP64 sum.  What bounds it is FP64 operations (1.67 per clock and SM) and the
+// direct FP64 sum.  What bounds it is FP64 operations (two per clock and SM) and the
 // latency of a chain of them (70 clocks each), so the 32 lanes of a warp take
 // n = lane, lane + 32, ... of one node, each by the three-term recurrence in steps of 32
 // (its error grows with the square of the steps taken, N / 32 instead of N), and

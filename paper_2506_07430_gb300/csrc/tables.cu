@@ -188,13 +188,21 @@ static int64_t binom64(int n, int k) {
     return r;
 }
 
-// packed transposed table: one 32-bit word per entry (targets < 2^16 for n <= 18)
+// packed transposed table of the off-diagonal entries, in table order: target
+// (< 2^16 for n <= 18) | (p n + q + (sign < 0 ? n n : 0)) << 16
 __global__ void k_pack_tables(const int32_t* __restrict__ tgtT, const uint16_t* __restrict__ pqT,
-                              const int8_t* __restrict__ sgnT, int64_t ne,
+                              const int8_t* __restrict__ sgnT, int64_t ns, int nexc, int n,
                               uint32_t* __restrict__ pkT) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ne) return;
-    pkT[i] = (uint32_t)tgtT[i] | ((uint32_t)pqT[i] << 16) | (sgnT[i] < 0 ? 0x80000000u : 0u);
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= ns) return;
+    int64_t k = 0;
+    for (int e = 0; e < nexc; ++e) {
+        const int64_t i = (int64_t)e * ns + r;
+        const int g = pqT[i];
+        if (g % (n + 1) == 0) continue;
+        pkT[k * ns + r] = (uint32_t)tgtT[i] | (uint32_t)(g + (sgnT[i] < 0 ? n * n : 0)) << 16;
+        ++k;
+    }
 }
 
 void build_spin_tables(SpinTables& t, int n, int m, const double* d_h1, const double* d_eri,
@@ -225,11 +233,11 @@ void build_spin_tables(SpinTables& t, int n, int m, const double* d_h1, const do
                                t.pq.as<uint16_t>(), t.sgn.as<int8_t>(), t.tgtT.as<int32_t>(),
                                t.pqT.as<uint16_t>(), t.sgnT.as<int8_t>());
     KPM_LAUNCHED();
-    t.pkT.alloc(ne * 4 + 4);
+    t.pkT.alloc((size_t)t.ns * m * (n - m) * 4 + 4);
     if (ne > 0) {
-        k_pack_tables<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(
-            t.tgtT.as<int32_t>(), t.pqT.as<uint16_t>(), t.sgnT.as<int8_t>(), (int64_t)ne,
-            t.pkT.as<uint32_t>());
+        k_pack_tables<<<bl, th, 0, st>>>(t.tgtT.as<int32_t>(), t.pqT.as<uint16_t>(),
+                                         t.sgnT.as<int8_t>(), t.ns, t.nexc, n,
+                                         t.pkT.as<uint32_t>());
         KPM_LAUNCHED();
     }
     k_same_spin<<<bl, th, 0, st>>>(t.masks.as<uint32_t>(), n, t.ns, t.nnbr, B, d_h1, d_eri,
