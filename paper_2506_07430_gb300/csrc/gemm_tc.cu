@@ -24,8 +24,9 @@
 // diagonals and the opposite-spin Coulomb sums, evaluated in FP64 and stored as
 // float hi + lo per determinant) times x, hi and lo multiplied separately.
 //
-// Kernel: CTA tile 128 x 256, k-block 32 (64 bytes per row: one SWIZZLE_64B atom
-// row), four-stage TMA pipeline (full/empty mbarriers), one warp issues TMA,
+// Kernel: CTA tile 128 x 256 (or narrower, see tile_columns), k-block 32 (64 bytes per
+// row: one SWIZZLE_64B atom row), TMA pipeline of four stages (narrower tiles six or
+// eight; full/empty mbarriers), one warp issues TMA,
 // one issues MMAs, eight warps drain accumulator chunks (see k_gemm) and run the
 // epilogue; clusters of two CTAs on vertically adjacent tiles share (multicast)
 // the B tile.  All waits are bounded.
@@ -55,19 +56,20 @@ namespace {
 #ifndef GM_BK_N
 #define GM_BK_N 32
 #endif
-// N of a tile: 256 (8 epilogue warps of 128 columns) or 192 (12 of 64 columns,
-// half the tensor-memory loads per warp and chunk; measured slower at 16 orbitals,
-// 20.4 vs 19.6 ms for both products)
-#ifndef GM_BN_N
-#define GM_BN_N 256
-#endif
-constexpr int GM_BM = 128, GM_BN = GM_BN_N, GM_BK = GM_BK_N, GM_STAGES = GM_BK == 64 ? 2 : 4;
+constexpr int GM_BM = 128, GM_BK = GM_BK_N;
 static_assert(GM_BK == 32 || GM_BK == 64, "k-block of 32 or 64");
-// epilogue warps: GM_BN / GM_EPI_COLS per TMEM lane quadrant, GM_EPI_COLS columns
-// each, drained 32 columns per tensor-memory load
-constexpr int GM_EPI_COLS = GM_BN == 256 ? 128 : 64;
-constexpr int GM_EPI_WARPS = 4 * GM_BN / GM_EPI_COLS;
-static_assert(GM_BN % GM_EPI_COLS == 0 && GM_EPI_COLS % 32 == 0, "epilogue geometry");
+// Column tiles of 256, 128 or 64 (tile_columns() picks).  Eight epilogue warps, half a
+// tile's columns each, drained 32 columns per tensor-memory load; narrower tiles have
+// deeper pipelines in the same shared memory.
+constexpr int GM_LIST_N = 256;               // rows of F_a per k-block list, for every tile
+constexpr int GM_EPI_WARPS = 8;
+template <int BN>
+struct Tile {
+    static constexpr int EPI_COLS = BN / 2;
+    static constexpr int STAGES = (BN == 256 ? 4 : BN == 128 ? 6 : 8) * 32 / GM_BK;
+    static constexpr uint32_t B_BYTES = BN * GM_BK * 2;   // per piece
+    static_assert(GM_LIST_N % BN == 0 && EPI_COLS % 32 == 0, "tile geometry");
+};
 constexpr int GM_TMA_WARP = GM_EPI_WARPS;       // producer (one thread)
 constexpr int GM_MMA_WARP = GM_EPI_WARPS + 1;   // MMA issue (one thread)
 constexpr int GM_THREADS = 32 * (GM_EPI_WARPS + 2);
@@ -85,12 +87,13 @@ constexpr int GM_CK = 64 / GM_BK;               // k-blocks per accumulation chu
 #define GM_BACKOFF_NS 256
 #endif
 constexpr uint32_t A_BYTES = GM_BM * GM_BK * 2;  // per piece
-constexpr uint32_t B_BYTES = GM_BN * GM_BK * 2;  // per piece
 // CTA pairs (clusters of two) on vertically adjacent tiles share the B tile: each
 // CTA loads half of its rows and multicasts them into both
 constexpr int GM_PAIR = 2;
-constexpr uint32_t B_HALF = B_BYTES / GM_PAIR;
-constexpr uint32_t STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
+template <int BN>
+constexpr uint32_t stage_bytes() { return 2 * A_BYTES + 2 * Tile<BN>::B_BYTES; }
+template <int BN>
+constexpr size_t gemm_smem() { return Tile<BN>::STAGES * stage_bytes<BN>() + 1024 + 256; }
 constexpr long long GM_WAIT = 4000000000LL;
 
 __device__ __forceinline__ uint32_t su32(const void* p) {
@@ -203,9 +206,10 @@ __device__ __forceinline__ uint64_t sw_desc(uint32_t saddr) {
     return d;
 }
 
+template <int BN>
 __host__ __device__ constexpr uint32_t gemm_idesc() {
-    // D F32, A/B F16, K-major, N = 256, M = 128
-    return (1u << 4) | ((uint32_t)(GM_BN >> 3) << 17) | ((uint32_t)(GM_BM >> 4) << 24);
+    // D F32, A/B F16, K-major, N = BN, M = 128
+    return (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(GM_BM >> 4) << 24);
 }
 
 struct GemmArgs {
@@ -266,20 +270,25 @@ __device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
 // initialised) and at the end (no multicast or remote arrive left in flight).
 //
 // Accumulation in chunks: the MMA thread restarts the accumulator every ck
-// k-blocks, alternating two tensor-memory accumulators of GM_BN columns; the
+// k-blocks, alternating two tensor-memory accumulators of BN columns; the
 // epilogue warps add each finished chunk into FP32 running sums held in
 // registers while the next chunk accumulates.  An FP32 accumulator that takes
 // one rounding per k-step over all of K (12870 at 16 orbitals) carries an error
 // growing like sqrt(K); in chunks, each accumulator sums a short run and the
 // running sum takes one rounding per chunk.
+template <int BN>
 __global__ void __cluster_dims__(GM_PAIR, 1, 1) __launch_bounds__(GM_THREADS, 1)
 k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
+    constexpr int STAGES = Tile<BN>::STAGES, EPI_COLS = Tile<BN>::EPI_COLS;
+    constexpr uint32_t B_BYTES = Tile<BN>::B_BYTES, B_HALF = B_BYTES / GM_PAIR;
+    constexpr uint32_t STAGE_BYTES = stage_bytes<BN>();
+    static_assert(STAGES * STAGE_BYTES >= GM_EPI_WARPS * EPI_COLS * 32 * 4, "epilogue staging");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + GM_STAGES * STAGE_BYTES);
-    uint64_t* empty = full + GM_STAGES;
-    uint64_t* accf = empty + GM_STAGES;   // [2] accumulator chunk finished
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint64_t* empty = full + STAGES;
+    uint64_t* accf = empty + STAGES;   // [2] accumulator chunk finished
     uint64_t* acce = accf + 2;            // [2] accumulator drained (epilogue warps)
     uint32_t* holder = reinterpret_cast<uint32_t*>(acce + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(holder + 1);
@@ -291,7 +300,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     // grouped rasterisation over pairs of row tiles: groups of GROUP_M pairs walk
     // all column tiles, so the group's A panels and the current B panels stay in L2
     const int GROUP_M = g.group_m;
-    const int nM = (g.M + GM_BM - 1) / GM_BM, nN = (g.N + GM_BN - 1) / GM_BN;
+    const int nM = (g.M + GM_BM - 1) / GM_BM, nN = (g.N + BN - 1) / BN;
     const int nMP = (nM + GM_PAIR - 1) / GM_PAIR;
     const int per_col = nMP * nN;              // tile pairs of a column
     const int col = blockIdx.x / GM_PAIR / per_col;
@@ -307,19 +316,19 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     // (with an odd number of row tiles the last pair's second tile lies past M:
     // its A loads read the zero fill and its epilogue writes nothing)
     const int m0 = (mp * GM_PAIR + (int)crank) * GM_BM;
-    const int n0 = ((b % gsize) / gm) * GM_BN;
+    const int n0 = ((b % gsize) / gm) * BN;
     // k-blocks the pair visits (both CTAs the same, as they share the B loads): those
     // of F_b where the pair's 256 rows have a nonzero, then those of F_a where the
-    // 256-row B tile has one; accumulation chunks do not cross from one to the other
+    // 256-row list tile of F_a around the B tile has one; accumulation chunks do not cross from one to the other
     const int* kl1 = g.kbl_b + g.kbs_b[mp];
     const int nk1 = g.kbs_b[mp + 1] - g.kbs_b[mp];
-    const int* kl2 = g.kbl_a + g.kbs_a[n0 / GM_BN];
-    const int nk = nk1 + g.kbs_a[n0 / GM_BN + 1] - g.kbs_a[n0 / GM_BN];
+    const int* kl2 = g.kbl_a + g.kbs_a[n0 / GM_LIST_N];
+    const int nk = nk1 + g.kbs_a[n0 / GM_LIST_N + 1] - g.kbs_a[n0 / GM_LIST_N];
     constexpr int ck = GM_CK;                                  // k-blocks per chunk
     const int nchunk1 = (nk1 + ck - 1) / ck, nchunk = nchunk1 + (nk - nk1 + ck - 1) / ck;
 
     if (tid == 0) {
-        for (int s = 0; s < GM_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init_(&full[s], 1);
             mbar_init_(&empty[s], GM_PAIR);   // the MMA commits of both CTAs
         }
@@ -353,9 +362,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
         if (lane == 0) {
             // TMA producer
             for (int kb = 0; kb < nk; ++kb) {
-                const int s = kb % GM_STAGES;
-                if (kb >= GM_STAGES &&
-                    !wait_or_abort(&empty[s], ((kb / GM_STAGES) - 1) & 1, abort_flag, g.err))
+                const int s = kb % STAGES;
+                if (kb >= STAGES &&
+                    !wait_or_abort(&empty[s], ((kb / STAGES) - 1) & 1, abort_flag, g.err))
                     break;
                 unsigned char* st = smem + s * STAGE_BYTES;
                 mbar_expect_tx(&full[s], STAGE_BYTES);
@@ -368,7 +377,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 tma_load_2d(su32(st + A_BYTES), mA + 1, kx, ma, &full[s]);
                 // this CTA's half of the B rows, into both CTAs
                 const uint32_t hb = crank * B_HALF;
-                const int nh = (beta ? xrow : 0) + n0 + (int)crank * (GM_BN / GM_PAIR);
+                const int nh = (beta ? xrow : 0) + n0 + (int)crank * (BN / GM_PAIR);
                 tma_load_2d_mc(su32(st + 2 * A_BYTES + hb), mB, kx, nh, &full[s], 0x3);
                 tma_load_2d_mc(su32(st + 2 * A_BYTES + B_BYTES + hb), mB + 1, kx, nh, &full[s], 0x3);
                 *(volatile int*)issued = kb + 1;
@@ -377,9 +386,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     } else if (warp == GM_MMA_WARP) {
         if (lane == 0) {
             // MMA issuer: chunk c accumulates its k-blocks (at most ck) into buffer c & 1
-            constexpr uint32_t idesc = gemm_idesc();
+            constexpr uint32_t idesc = gemm_idesc<BN>();
             for (int c = 0; c < nchunk; ++c) {
-                const uint32_t d = tmem + (uint32_t)((c & 1) * GM_BN);
+                const uint32_t d = tmem + (uint32_t)((c & 1) * BN);
                 if (c >= 2 && !wait_or_abort(&acce[c & 1], ((c >> 1) - 1) & 1, abort_flag, g.err))
                     break;
                 tc_after();
@@ -388,8 +397,8 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 const int kb1 = min(beta ? nk1 : nk, kb0 + ck);
                 bool ok = true;
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    const int s = kb % GM_STAGES;
-                    if (!wait_or_abort(&full[s], (kb / GM_STAGES) & 1, abort_flag, g.err)) {
+                    const int s = kb % STAGES;
+                    if (!wait_or_abort(&full[s], (kb / STAGES) & 1, abort_flag, g.err)) {
                         ok = false;
                         break;
                     }
@@ -419,12 +428,12 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             }
         }
     } else {
-        // epilogue warps: running sums of columns [128 h, 128 h + 128) for row m
+        // epilogue warps: running sums of columns [EPI_COLS h, EPI_COLS (h + 1)) for row m
         const int quad = warp & 3, h = warp >> 2;
-        const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * GM_EPI_COLS);
-        float rs[GM_EPI_COLS];
+        const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * EPI_COLS);
+        float rs[EPI_COLS];
 #pragma unroll
-        for (int u = 0; u < GM_EPI_COLS; ++u) rs[u] = 0.f;
+        for (int u = 0; u < EPI_COLS; ++u) rs[u] = 0.f;
         bool ok = true;
         for (int c = 0; c < nchunk && ok; ++c) {
             if (lane == 0)
@@ -434,12 +443,12 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             // from the scale of F_b's product to that of F_a's (a power of two)
             if (c == nchunk1 && g.ratio != 1.f) {
 #pragma unroll
-                for (int u = 0; u < GM_EPI_COLS; ++u) rs[u] *= g.ratio;
+                for (int u = 0; u < EPI_COLS; ++u) rs[u] *= g.ratio;
             }
             tc_after();
-            const uint32_t src = trow + (uint32_t)((c & 1) * GM_BN);
+            const uint32_t src = trow + (uint32_t)((c & 1) * BN);
 #pragma unroll
-            for (int q = 0; q < GM_EPI_COLS / 32; ++q) {
+            for (int q = 0; q < EPI_COLS / 32; ++q) {
                 uint32_t r[32];
                 ld32(src + (uint32_t)(q * 32), r);
 #pragma unroll
@@ -464,13 +473,13 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             // time waits for memory 128 times, 45 us a tile, most of the product's time
             // at small sizes.  (Every stage's loads have been consumed by the MMAs whose
             // accumulators were drained, so none is in flight into this memory.)
-            float* mine = reinterpret_cast<float*>(smem) + warp * (GM_EPI_COLS * 32) + lane;
+            float* mine = reinterpret_cast<float*>(smem) + warp * (EPI_COLS * 32) + lane;
 #pragma unroll
-            for (int u = 0; u < GM_EPI_COLS; ++u) mine[u * 32] = rs[u];
+            for (int u = 0; u < EPI_COLS; ++u) mine[u * 32] = rs[u];
             const int m = m0 + quad * 32 + lane;
-            const int nb = n0 + h * GM_EPI_COLS;
+            const int nb = n0 + h * EPI_COLS;
             constexpr int EG = 16;
-            const int ncols = m < g.M ? min(GM_EPI_COLS, g.N - nb) : 0;
+            const int ncols = m < g.M ? min(EPI_COLS, g.N - nb) : 0;
             float* y = g.y + col * dim;
             const float* x = g.x + col * dim;
 #pragma unroll 1
@@ -506,7 +515,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     if (tid == 0 && *abort_flag) {
         // after an abort, wait (bounded) for TMA copies that were issued but not consumed
         for (int kb = *consumed; kb < *issued; ++kb)
-            mbar_wait_bounded(&full[kb % GM_STAGES], (kb / GM_STAGES) & 1, g.err);
+            mbar_wait_bounded(&full[kb % STAGES], (kb / STAGES) & 1, g.err);
     }
     __syncthreads();
     cluster_sync_();   // neither CTA exits while the peer may still write into it
@@ -693,8 +702,8 @@ CUtensorMap make_map(const __half* base, int64_t rows, int64_t cols, int64_t pit
 int64_t half_pitch(int64_t cols) { return (cols + 7) / 8 * 8; }
 
 // CTAs of an M x N product: pairs of row tiles x column tiles, two CTAs each
-static unsigned gemm_grid(int64_t M, int64_t N) {
-    const int64_t nM = (M + GM_BM - 1) / GM_BM, nN = (N + GM_BN - 1) / GM_BN;
+static unsigned gemm_grid(int64_t M, int64_t N, int bn) {
+    const int64_t nM = (M + GM_BM - 1) / GM_BM, nN = (N + bn - 1) / bn;
     return (unsigned)(GM_PAIR * ((nM + GM_PAIR - 1) / GM_PAIR) * nN);
 }
 
@@ -781,8 +790,15 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     xpitch = (nb + 127) / 128 * 128;
     cb = batch_columns(na * nb);
     err = err_flag;
-    smem = GM_STAGES * STAGE_BYTES + 1024 + 256;
-    KPM_CUDA(cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int dev = 0;
+    KPM_CUDA(cudaGetDevice(&dev));
+    KPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    KPM_CUDA(cudaFuncSetAttribute(k_gemm<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)gemm_smem<256>()));
+    KPM_CUDA(cudaFuncSetAttribute(k_gemm<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)gemm_smem<128>()));
+    KPM_CUDA(cudaFuncSetAttribute(k_gemm<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)gemm_smem<64>()));
     wscale_b = offdiag_scale(B, fmax, st);
     build_f(B, wscale_b, fb_hi, fb_lo, db, pb, st);
     if (same) {
@@ -798,9 +814,9 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
         da = &da_own;
     }
     // beta: F_b is the A operand (pairs of GM_BM-row tiles); alpha: F_a is the B
-    // operand (GM_BN-row tiles)
+    // operand (lists by GM_LIST_N rows)
     block_lists(B, GM_PAIR * GM_BM, kbs_b, kbl_b, &kb_nonzero[0], &kb_total[0], st);
-    block_lists(A, GM_BN, kbs_a, kbl_a, &kb_nonzero[1], &kb_total[1], st);
+    block_lists(A, GM_LIST_N, kbs_a, kbl_a, &kb_nonzero[1], &kb_total[1], st);
 }
 
 void DenseSS::split(const float* x, const float* amax, int nc, cudaStream_t st) {
@@ -814,24 +830,43 @@ void DenseSS::split(const float* x, const float* amax, int nc, cudaStream_t st) 
     KPM_LAUNCHED();
 }
 
+// The narrowest tile whose grid is one wave: a tile's time is its k-blocks' MMAs and its
+// epilogue, both by its width, so below one wave narrower tiles give the same work to more
+// SMs (and a shorter epilogue).  Beyond one wave 256 is best: every CTA reads its A tile
+// whole, 24 KB a k-block at 128 columns for half the MMAs of the 32 KB at 256.  Measured,
+// whole sigma with 256 / 128 / 64 columns: 10 orbitals 67.1 / 59.0 / 54.7 us (three
+// columns of x 80.2 / 71.7 / 67.7), 12 orbitals 184.6 / 175.8 / 171.8 (three, where 64
+// takes 2.4 waves: 372 / 401 / 425), (13o, 5 + 5) 283 / 271 / 310 (64: 1.7 waves),
+// (13o, 7 + 6) 422 / 473 / 516.  Every width adds the same chunks in the same order, so
+// the results are the same bits.
+int DenseSS::tile_columns(int nc) const {
+    for (int bn : {64, 128})
+        if (nc * (int64_t)gemm_grid(nb, na, bn) <= nsm) return bn;
+    return 256;
+}
+
 // y[I_a][I_b] += sum_J Fb[I_b][J] x[I_a][J] (x rows from split())
 //             + sum_J x^T[I_b][J] Fa[I_a][J] + H_II x[I_a][I_b]
 void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int group,
                      cudaStream_t st) {
     const float* diag = diag_full ? x : nullptr;
+    const int bn = tile_columns(nc);
     GemmMaps maps;
     maps.fb[0] = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
     maps.fb[1] = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
-    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, GM_BN / GM_PAIR);
-    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, GM_BN / GM_PAIR);
+    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
+    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
     maps.t[0] = make_map(th.as<__half>(), nc * nb, na, pa, GM_BM);
     maps.t[1] = make_map(tl.as<__half>(), nc * nb, na, pa, GM_BM);
-    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
-    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, GM_BN / GM_PAIR);
+    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn / GM_PAIR);
+    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn / GM_PAIR);
     GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
                diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
                kbs_a.as<int>(), kbl_a.as<int>()};
-    k_gemm<<<nc * gemm_grid(nb, na), GM_THREADS, smem, st>>>(maps, g);
+    const unsigned grid = nc * gemm_grid(nb, na, bn);
+    if (bn == 256) k_gemm<256><<<grid, GM_THREADS, gemm_smem<256>(), st>>>(maps, g);
+    else if (bn == 128) k_gemm<128><<<grid, GM_THREADS, gemm_smem<128>(), st>>>(maps, g);
+    else k_gemm<64><<<grid, GM_THREADS, gemm_smem<64>(), st>>>(maps, g);
     KPM_LAUNCHED();
 }
 

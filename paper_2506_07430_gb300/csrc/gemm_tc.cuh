@@ -30,7 +30,7 @@ struct DenseSS {
     // block_lists): F_b by pairs of 128-row tiles, F_a by 256-row tiles
     DevBuf kbs_b, kbl_b, kbs_a, kbl_a;
     int64_t kb_nonzero[2] = {0, 0}, kb_total[2] = {0, 0};
-    size_t smem = 0;
+    int nsm = 0;                              // SMs of the device
     int* err = nullptr;
     // exact diagonal H_II of the whole H (same-spin diagonals and the opposite-spin
     // Coulomb sum, FP64 stored as float hi + lo, [N_a][N_b]), added by the
@@ -52,6 +52,8 @@ struct DenseSS {
     int group_m = 16;
     void autotune(cudaStream_t st);
     void launch(const float* x, float* y, const float* amax, int nc, int group, cudaStream_t st);
+    // Columns (N) of the GEMM's tiles for nc columns of a block: 256, 128 or 64.
+    int tile_columns(int nc) const;
 };
 
 }  // namespace kpm
