@@ -535,89 +535,6 @@ __global__ void k_absmax_offdiag(const double* __restrict__ fval, int64_t ns, in
     if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(mx));
 }
 
-// Split rows: src[r][c] (float, r < R, c < Cn, row pitch ld) -> hi/lo FP16 [r][pitch],
-// scaled by 2^(14 - e(amax[r / per])); pad columns [Cn, pitch) with zeros.  One thread per 4
-// columns of a row (pitch a multiple of 4): two 8-byte loads where the row is 8-byte
-// aligned, one 8-byte store per piece.
-__global__ void k_split_rows(const float* __restrict__ src, int64_t R, int64_t Cn, int64_t ld,
-                             __half* __restrict__ hi, __half* __restrict__ lo, int64_t pitch,
-                             int64_t per, const float* amax) {
-    const int64_t q = pitch >> 2;
-    const bool v2 = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 7) == 0;
-    for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
-        float sa = 1.f;
-        {
-            const float mx = amax[r / per];
-            if (mx > 0.f && isfinite(mx)) {
-                int e;
-                frexpf(mx, &e);
-                sa = ldexpf(1.f, 14 - max(e, -90));
-            }
-        }
-        for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < q;
-             g += (int64_t)gridDim.x * blockDim.x) {
-            const int64_t c = 4 * g;
-            const float* s = src + r * ld + c;
-            float v[4];
-            if (v2 && c + 3 < Cn) {
-                const float2 x0 = *reinterpret_cast<const float2*>(s);
-                const float2 x1 = *reinterpret_cast<const float2*>(s + 2);
-                v[0] = x0.x; v[1] = x0.y; v[2] = x1.x; v[3] = x1.y;
-            } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = c + u < Cn ? s[u] : 0.f;
-            }
-            __align__(8) __half h[4], l[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float t = v[u] * sa;
-                h[u] = __float2half_rn(t);
-                l[u] = __float2half_rn(t - __half2float(h[u]));
-            }
-            *reinterpret_cast<uint2*>(hi + r * pitch + c) = *reinterpret_cast<const uint2*>(h);
-            *reinterpret_cast<uint2*>(lo + r * pitch + c) = *reinterpret_cast<const uint2*>(l);
-        }
-    }
-}
-
-// Transposed split of each column (blockIdx.z): dst[c][r] = src[r][c] for src R x Cn, dst rows Cn of pitch >= R
-// (pitch even, padding rows [R, pitch) written as zeros).  Tiles of 64 rows x 32
-// columns through shared memory; each thread stores two consecutive r as a half2.
-__global__ void k_split_transpose(const float* __restrict__ src, int64_t R, int64_t Cn,
-                                  __half* __restrict__ hi, __half* __restrict__ lo,
-                                  int64_t pitch, const float* amax) {
-    __shared__ float t[64][33];
-    src += (int64_t)blockIdx.z * R * Cn;
-    hi += (int64_t)blockIdx.z * Cn * pitch;
-    lo += (int64_t)blockIdx.z * Cn * pitch;
-    float sa = 1.f;
-    {
-        const float mx = amax[blockIdx.z];
-        if (mx > 0.f && isfinite(mx)) {
-            int e;
-            frexpf(mx, &e);
-            sa = ldexpf(1.f, 14 - max(e, -90));
-        }
-    }
-    const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 64;
-    for (int k = threadIdx.y; k < 64; k += blockDim.y) {
-        const int64_t r = r0 + k, c = c0 + threadIdx.x;
-        t[k][threadIdx.x] = (r < R && c < Cn) ? src[r * Cn + c] * sa : 0.f;
-    }
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int64_t c = c0 + k, r = r0 + 2 * threadIdx.x;
-        if (c < Cn && r < pitch) {
-            const float v0 = t[2 * threadIdx.x][k], v1 = t[2 * threadIdx.x + 1][k];
-            const __half h0 = __float2half_rn(v0), h1 = __float2half_rn(v1);
-            *reinterpret_cast<__half2*>(hi + c * pitch + r) = __halves2half2(h0, h1);
-            *reinterpret_cast<__half2*>(lo + c * pitch + r) =
-                __halves2half2(__float2half_rn(v0 - __half2float(h0)),
-                               __float2half_rn(v1 - __half2float(h1)));
-        }
-    }
-}
-
 // Dense off-diagonal string Hamiltonian, split into two scaled FP16 pieces.
 // The matrix is first zeroed (k_zero_half), then every off-diagonal neighbour
 // entry (t >= 1 of the [nnbr][ns] lists) is written.
@@ -819,15 +736,11 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     block_lists(A, GM_LIST_N, kbs_a, kbl_a, &kb_nonzero[1], &kb_total[1], st);
 }
 
-void DenseSS::split(const float* x, const float* amax, int nc, cudaStream_t st) {
+void DenseSS::reserve() {
     xh.ensure((size_t)cb * na * xpitch * 2);
     xl.ensure((size_t)cb * na * xpitch * 2);
-    if (xpitch & 3) KPM_THROW(KPM_EINVAL, "split rows: pitch not a multiple of 4");
-    const int64_t q = xpitch / 4, rows = nc * na;
-    dim3 gs((unsigned)((q + 255) / 256), (unsigned)(rows < 65535 ? (rows > 0 ? rows : 1) : 65535));
-    k_split_rows<<<gs, 256, 0, st>>>(x, rows, nb, nb, xh.as<__half>(), xl.as<__half>(), xpitch,
-                                     na, amax);
-    KPM_LAUNCHED();
+    th.ensure((size_t)cb * nb * pa * 2);
+    tl.ensure((size_t)cb * nb * pa * 2);
 }
 
 // The narrowest tile whose grid is one wave: a tile's time is its k-blocks' MMAs and its
@@ -845,7 +758,7 @@ int DenseSS::tile_columns(int nc) const {
     return 256;
 }
 
-// y[I_a][I_b] += sum_J Fb[I_b][J] x[I_a][J] (x rows from split())
+// y[I_a][I_b] += sum_J Fb[I_b][J] x[I_a][J] (split copies of x in xh/xl, th/tl)
 //             + sum_J x^T[I_b][J] Fa[I_a][J] + H_II x[I_a][I_b]
 void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int group,
                      cudaStream_t st) {
@@ -871,13 +784,6 @@ void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int gr
 }
 
 void DenseSS::apply(const float* x, float* y, const float* amax, int nc, cudaStream_t st) {
-    // transposed split copy of x (cols beta x rows alpha); the row split is xh/xl
-    th.ensure((size_t)cb * nb * pa * 2);
-    tl.ensure((size_t)cb * nb * pa * 2);
-    if (pa & 1) KPM_THROW(KPM_EINVAL, "split transpose: odd pitch");
-    dim3 tb(32, 8), gt((unsigned)((nb + 31) / 32), (unsigned)((na + 63) / 64), (unsigned)nc);
-    k_split_transpose<<<gt, tb, 0, st>>>(x, na, nb, th.as<__half>(), tl.as<__half>(), pa, amax);
-    KPM_LAUNCHED();
     launch(x, y, amax, nc, group_m, st);
 }
 
@@ -902,10 +808,7 @@ void DenseSS::autotune(cudaStream_t st) {
         }
     }
     // scratch operands (zeros: the timing does not depend on the values)
-    xh.ensure((size_t)cb * na * xpitch * 2);
-    xl.ensure((size_t)cb * na * xpitch * 2);
-    th.ensure((size_t)cb * nb * pa * 2);
-    tl.ensure((size_t)cb * nb * pa * 2);
+    reserve();
     KPM_CUDA(cudaMemsetAsync(xh.p, 0, xh.bytes, st));
     KPM_CUDA(cudaMemsetAsync(xl.p, 0, xl.bytes, st));
     KPM_CUDA(cudaMemsetAsync(th.p, 0, th.bytes, st));

@@ -40,12 +40,12 @@ struct DenseSS {
     // Builds the split matrices; `same`: alpha and beta strings are identical.
     void init(const SpinTables& A, const SpinTables& B, bool same, int* err_flag,
               cudaStream_t st);
-    // xh/xl = nc columns of x split into scaled FP16 pieces [nc][N_a][xpitch] (zero
-    // padding); amax = device max|x| of each column.
-    void split(const float* x, const float* amax, int nc, cudaStream_t st);
+    // Split copies of the operand, scaled FP16 pieces with zero padding, written by the
+    // caller (k_prepare): rows of x [nc][N_a][xpitch] in xh/xl, of x^T [nc][N_b][pa] in th/tl.
+    void reserve();
     // y += (F_a (x) 1 + 1 (x) F_b) x with the off-diagonal parts of F_a, F_b, plus
     // diag_full * x (the whole exact diagonal of H); amax = device max|x|.
-    // Uses xh/xl from split(x) on the same stream.
+    // Reads xh/xl and th/tl, not x's own entries, in the products.
     void apply(const float* x, float* y, const float* amax, int nc, cudaStream_t st);
     // Rasterisation group (row tiles per group), chosen by autotune() at set-up; 16 by
     // default.

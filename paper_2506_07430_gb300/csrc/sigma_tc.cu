@@ -157,7 +157,7 @@ struct RowPass {
     const double* wr;        // [Nr][P] w_R[s] (unscaled, FP64)
     const uint16_t* wrow;    // W by input slot: NW pieces of [P][P] 16-bit (bits of the format)
     uint32_t ncols;          // TMEM columns allocated
-    const float2* rscale;    // [nblk][Nr] scale of B_R, scale of the row's integer sums (k_rowscale)
+    const float2* rscale;    // [nblk][Nr] scale of B_R, scale of the row's integer sums (k_prepare)
     float wscale;            // power-of-two scale applied to W in the image
     int NS;                  // slots in use (n(n+1)/2); slots [NS, P) are padding
     int nst;                 // A stages in shared memory (2 or 3)
@@ -330,7 +330,7 @@ __device__ __forceinline__ bool wait_phase(uint64_t* mbar, uint32_t parity, vola
 // The copy warps know nothing of rows but their targets and run ahead across them.
 // The others meet twice between rows: after the last tile, and again once they have
 // written and cleared sigma and built the next row's B_R (its slots prefetched a row
-// ahead, its scale from k_rowscale).  At 14 orbitals the turn took 31,000 cycles, a
+// ahead, its scale from k_prepare).  At 14 orbitals the turn took 31,000 cycles, a
 // fifth of the row, with the scale, its reductions and the copies of the first tiles
 // in it.
 //
@@ -710,13 +710,12 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
 // row: c_s (in units of the W image; piece 0 of W is within 2^-8 of W in either
 // format: 1 % margin) and max |B| over the lanes' slots s.
 template <bool FP16>
-__global__ void __launch_bounds__(256)
-k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
-           const uint16_t* __restrict__ rslot, const uint16_t* __restrict__ wrow,
-           const double* __restrict__ wr, int64_t Nr, int nblk, int rnexc, int ndiag, int P,
-           float wscale, int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
+__device__ __forceinline__ void
+row_scale(int64_t rg, const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
+          const uint16_t* __restrict__ rslot, const uint16_t* __restrict__ wrow,
+          const double* __restrict__ wr, int64_t Nr, int nblk, int rnexc, int ndiag, int P,
+          float wscale, int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
     constexpr int SL = (176 + 31) / 32;
-    const int64_t rg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (rg >= Nr * nblk) return;
     const int64_t blk = rg / Nr, r = rg - blk * Nr;
@@ -738,7 +737,7 @@ k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
         const float rm = e < rnexc ? rowmax[rtgt[r * rnexc + e]] : 0.f;
         const int sl = e < rnexc ? rslot[r * rnexc + e] & 0x7FFF : 0;
         const int cnt = min(32, rnexc - e0);
-#pragma unroll 4
+#pragma unroll 8
         for (int k = 0; k < cnt; ++k) {
             const float m = __shfl_sync(0xffffffffu, rm, k);
             const uint16_t* row = wrow + (size_t)__shfl_sync(0xffffffffu, sl, k) * P + lane;
@@ -777,6 +776,109 @@ k_rowscale(const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
         }
     }
     out[rg] = make_float2(fx / (sa * wscale), 1.f / fx);
+}
+
+// Operands of the row pass and of the GEMMs, from x [R][Cn] (nblk columns of a block), the
+// rows' maxima and each column's: the scales of every row, and split copies of x scaled by
+// 2^(14 - e(amax)) in FP16 pieces hi + lo, the rows [R][xpitch] and the transpose
+// [Cn][tpitch], padding columns zero in both; for BF16 operands the rows in (unscaled) BF16
+// pieces as well.
+//
+// Bound by its bytes at large sizes (4 read and 8 written per determinant: 358 us at 16
+// orbitals, 5.6 TB/s) and by its latency at small ones (8 us).  One launch for what took
+// three (four for BF16), which read x once for each copy: sigma at 16 orbitals 32.44 ->
+// 32.20 ms, at 14 (three columns) 4.74 -> 4.66, (13o, 7 + 6, BF16) 434 -> 405 us, three
+// columns of 10 orbitals 68.1 -> 59.8.  The first nscale blocks take the scales, a row a
+// warp (the longest chain of loads, so they start
+// first); the others a tile of 64 x 64 each through shared memory, two columns a thread:
+// the rows leave from registers, the transpose two rows at a time, 128 bytes a warp and
+// store either way.
+struct Prepare {
+    const float* x;            // nullptr: scales only
+    int64_t R, Cn;
+    int nblk;
+    unsigned nscale, tx, ty;   // blocks of scales; tiles across and down
+    __half *xh, *xl;
+    int64_t xpitch;
+    __half *th, *tl;
+    int64_t tpitch;
+    uint16_t *bh, *bl;         // BF16 pieces of the rows
+    const float* rowmax;
+    const float* amax;
+    const int32_t* rtgt;
+    const uint16_t* rslot;
+    const uint16_t* wrow;
+    const double* wr;
+    int rnexc, ndiag, P;
+    float wscale;
+    int nexc_c;
+    float2* rscale;
+};
+constexpr int SPLIT_T = 64;
+template <bool FP16>
+__global__ void __launch_bounds__(256) k_prepare(const Prepare p) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x < p.nscale) {
+        row_scale<FP16>((int64_t)blockIdx.x * 8 + warp, p.rowmax, p.rtgt, p.rslot, p.wrow, p.wr,
+                        p.R, p.nblk, p.rnexc, p.ndiag, p.P, p.wscale, p.nexc_c, p.amax, p.rscale);
+        return;
+    }
+    __shared__ float t[SPLIT_T][SPLIT_T + 1];
+    const unsigned tile = blockIdx.x - p.nscale, blk = tile / (p.tx * p.ty);
+    const int64_t R = p.R, Cn = p.Cn;
+    const float* src = p.x + blk * R * Cn;
+    const bool v2 = (Cn & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 7) == 0;
+    const int64_t c0 = (int64_t)(tile % p.tx) * SPLIT_T, c = c0 + 2 * lane;
+    const int64_t r0 = (int64_t)(tile / p.tx % p.ty) * SPLIT_T;
+    float2 v[SPLIT_T / 8];
+#pragma unroll
+    for (int i = 0; i < SPLIT_T / 8; ++i) {
+        const int64_t r = r0 + warp + 8 * i;
+        const float* s = src + r * Cn + c;
+        v[i] = make_float2(0.f, 0.f);
+        if (r < R) {
+            if (v2 && c + 1 < Cn) {
+                v[i] = *reinterpret_cast<const float2*>(s);
+            } else {
+                if (c < Cn) v[i].x = s[0];
+                if (c + 1 < Cn) v[i].y = s[1];
+            }
+        }
+    }
+    const float sa = x_scale(p.amax[blk], true);
+    auto put = [](float a, float b, __half* hi, __half* lo) {
+        const __half ha = __float2half_rn(a), hb = __float2half_rn(b);
+        *reinterpret_cast<__half2*>(hi) = __halves2half2(ha, hb);
+        *reinterpret_cast<__half2*>(lo) = __halves2half2(__float2half_rn(a - __half2float(ha)),
+                                                         __float2half_rn(b - __half2float(hb)));
+    };
+#pragma unroll
+    for (int i = 0; i < SPLIT_T / 8; ++i) {
+        const int k = warp + 8 * i;
+        const int64_t o = (blk * R + r0 + k) * p.xpitch + c;
+        const float a = v[i].x * sa, b = v[i].y * sa;
+        t[k][2 * lane] = a;
+        t[k][2 * lane + 1] = b;
+        if (r0 + k < R) {
+            put(a, b, p.xh + o, p.xl + o);
+            if (!FP16) {
+                const __nv_bfloat16 ha = __float2bfloat16_rn(v[i].x), hb = __float2bfloat16_rn(v[i].y);
+                *reinterpret_cast<__nv_bfloat162*>(p.bh + o) = __halves2bfloat162(ha, hb);
+                *reinterpret_cast<__nv_bfloat162*>(p.bl + o) =
+                    __halves2bfloat162(__float2bfloat16_rn(v[i].x - __bfloat162float(ha)),
+                                       __float2bfloat16_rn(v[i].y - __bfloat162float(hb)));
+            }
+        }
+    }
+    __syncthreads();
+    const int64_t r = r0 + 2 * lane;
+    if (r >= p.tpitch) return;
+#pragma unroll
+    for (int i = 0; i < SPLIT_T / 8; ++i) {
+        const int k = warp + 8 * i;
+        const int64_t o = (blk * Cn + c0 + k) * p.tpitch + r;
+        if (c0 + k < Cn) put(t[2 * lane][k], t[2 * lane + 1][k], p.th + o, p.tl + o);
+    }
 }
 
 // max |x| of each row (rowmax[r]) and of the rows of each block column of `per` rows
@@ -904,21 +1006,6 @@ __global__ void k_wdiag(const double* __restrict__ eri, const uint32_t* __restri
             }
     }
     w[i] = v;
-}
-
-// x [R][Cn] -> hi/lo BF16 pieces [R][pitch] (BF16 needs no scale); zero padding
-__global__ void k_split_rows_bf16(const float* __restrict__ src, int64_t R, int64_t Cn,
-                                  uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
-                                  int64_t pitch) {
-    const int64_t total = R * pitch;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / pitch, c = i % pitch;
-        const float v = c < Cn ? src[r * Cn + c] : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[i] = __bfloat16_as_ushort(h);
-        lo[i] = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(h)));
-    }
 }
 
 uint32_t tmem_cols(int P) {
@@ -1115,7 +1202,6 @@ void TcSigma::set_layout(int passes, cudaStream_t st) {
 }
 
 void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
-    const int64_t xp = dense.xpitch;
     const int cb = dense.cb;
     rowmax.ensure((size_t)(nsa > 0 ? cb * nsa : 1) * sizeof(float));
     for (int c = 0; c < ncol; c += cb) {
@@ -1132,20 +1218,9 @@ void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
         }
         KPM_LAUNCHED();
         const float* am = reinterpret_cast<const float*>(amax.p);
-        // split x: the FP16 pieces serve the row pass and the beta GEMM
-        dense.split(X, am, nc, st);
-        const uint16_t* xh = dense.xh.as<uint16_t>();
-        const uint16_t* xl = dense.xl.as<uint16_t>();
-        if (!fp16) {
-            xbh.ensure((size_t)cb * nsa * xp * 2);
-            xbl.ensure((size_t)cb * nsa * xp * 2);
-            k_split_rows_bf16<<<2048, 256, 0, st>>>(X, rows, nsb, xbh.as<uint16_t>(),
-                                                    xbl.as<uint16_t>(), xp);
-            KPM_LAUNCHED();
-            xh = xbh.as<uint16_t>();
-            xl = xbl.as<uint16_t>();
-        }
-        row_scales(am, nc, st);
+        prepare(X, am, nc, st);
+        const uint16_t* xh = fp16 ? dense.xh.as<uint16_t>() : xbh.as<uint16_t>();
+        const uint16_t* xl = fp16 ? dense.xl.as<uint16_t>() : xbl.as<uint16_t>();
         // opposite-spin part: rows alpha, columns beta; writes Y
         launch_rowpass(xh, xl, Y, nc, nst, rp_prefetch, st);
         // same-spin parts (dense GEMMs) and the exact diagonal, added into Y
@@ -1153,13 +1228,27 @@ void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
     }
 }
 
-void TcSigma::row_scales(const float* am, int nc, cudaStream_t st) {
+void TcSigma::prepare(const float* x, const float* am, int nc, cudaStream_t st) {
     rscale.ensure((size_t)(nsa > 0 ? dense.cb * nsa : 1) * sizeof(float2));
-    const unsigned g = (unsigned)((nc * nsa + 7) / 8);
-    auto* fn = fp16 ? k_rowscale<true> : k_rowscale<false>;
-    fn<<<g, 256, 0, st>>>(rowmax.as<float>(), rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(),
-                          wimg.as<uint16_t>(), wdiag.as<double>(), nsa, nc, noff, ndiag, P, wscale,
-                          tb->nexc, am, rscale.as<float2>());
+    unsigned tx = 0, ty = 0;
+    if (x) {
+        dense.reserve();
+        if (!fp16) {
+            xbh.ensure((size_t)dense.cb * nsa * dense.xpitch * 2);
+            xbl.ensure((size_t)dense.cb * nsa * dense.xpitch * 2);
+        }
+        if (dense.xpitch % SPLIT_T || (dense.pa & 1)) KPM_THROW(KPM_EINVAL, "split: pitch");
+        tx = (unsigned)(dense.xpitch / SPLIT_T);
+        ty = (unsigned)((nsa + SPLIT_T - 1) / SPLIT_T);
+    }
+    const Prepare p{x, nsa, nsb, nc, (unsigned)((nc * nsa + 7) / 8), tx, ty,
+                    dense.xh.as<__half>(), dense.xl.as<__half>(), dense.xpitch,
+                    dense.th.as<__half>(), dense.tl.as<__half>(), dense.pa,
+                    xbh.as<uint16_t>(), xbl.as<uint16_t>(), rowmax.as<float>(), am,
+                    rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(), wimg.as<uint16_t>(),
+                    wdiag.as<double>(), noff, ndiag, P, wscale, tb->nexc, rscale.as<float2>()};
+    auto* fn = fp16 ? k_prepare<true> : k_prepare<false>;
+    fn<<<p.nscale + nc * tx * ty, 256, 0, st>>>(p);
     KPM_LAUNCHED();
 }
 
@@ -1226,7 +1315,7 @@ void TcSigma::autotune(cudaStream_t st) {
     KPM_CUDA(cudaMemsetAsync(amax.p, 0, sizeof(unsigned), st));
     rowmax.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float));
     KPM_CUDA(cudaMemsetAsync(rowmax.p, 0, rowmax.bytes, st));
-    row_scales(reinterpret_cast<const float*>(amax.p), 1, st);
+    prepare(nullptr, reinterpret_cast<const float*>(amax.p), 1, st);
     cudaEvent_t e0, e1;
     KPM_CUDA(cudaEventCreate(&e0));
     KPM_CUDA(cudaEventCreate(&e1));

@@ -34,7 +34,7 @@ struct TcSigma {
     DevBuf err;                   // int error flag (1: a bounded wait ran out)
     DevBuf amax;                  // max |x| (float bits): operand scale, fixed-point range
     DevBuf rowmax;                // [N_a] max |x| per row: per-row fixed-point range of the row pass
-    DevBuf rscale;                // float2 [N_a] scales of a row (k_rowscale)
+    DevBuf rscale;                // float2 [N_a] scales of a row (k_prepare)
     int nst = 2;                  // A stages of the row pass (at most 3, where shared memory
                                   // allows; autotuned)
     int rp_prefetch = 0;          // L2 prefetch distance of the row pass, tiles (autotuned; none
@@ -56,8 +56,9 @@ struct TcSigma {
               const double* d_eri, const float2* d_diag, int n, double wmax, double wcolsum,
               bool use_fp16, cudaStream_t st);
     void apply(const float* x, float* y, int ncol, cudaStream_t st);
-    // Scales of every row from rowmax and max|x| (am), for the next row pass.
-    void row_scales(const float* am, int nc, cudaStream_t st);
+    // Scales of every row from rowmax and max|x| (am), for the next row pass, and the split
+    // copies of nc columns of x (none: x == nullptr).
+    void prepare(const float* x, const float* am, int nc, cudaStream_t st);
     // One row-pass launch (opposite-spin part of nc columns of y, overwriting it) from the
     // split rows xh, xl, with the given A stages and prefetch distance.
     void launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* y, int nc, int stages,

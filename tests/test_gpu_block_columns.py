@@ -52,3 +52,32 @@ def test_gemm_tile_widths_same_bits(n, na, nb):
     ref.synchronize()
     assert ((one[:1].double() - y).norm() / y.norm()).item() < 2e-6
     ref.close()
+
+
+@pytest.mark.parametrize("prec,tol", [
+    ("mixed", 2e-6),         # two FP16 pieces: 22 bits of x
+    ("mixed_bf16", 1e-5),    # two BF16 pieces: 2^-17 of each entry of x at most
+])
+@pytest.mark.parametrize("n,na,nb", [
+    (12, 2, 4),     # 66 x 495 strings: a second row of 64 x 64 tiles with two rows, odd pitch
+    (11, 2, 11),    # 55 x 1: one column
+    (11, 11, 2),    # 1 x 55: one row
+    (16, 2, 1),     # 120 x 16
+    (8, 4, 3),      # 70 x 56
+])
+def test_split_copies_at_tile_edges(prec, tol, n, na, nb):
+    import torch
+
+    from paper_2506_07430_gb300 import KPM
+    I = synthetic.integrals(n, na, nb, seed=2506840 + n)
+    k = KPM(I.h1, I.eri, I.dipole, n, na, nb, precision=prec)
+    ref = KPM(I.h1, I.eri, I.dipole, n, na, nb, precision="fp64")
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn((2, k.dim), generator=g, device="cuda")
+    y, z = k.sigma(x), ref.sigma(x.double())
+    k.synchronize()
+    ref.synchronize()
+    for c in range(2):
+        assert ((y[c].double() - z[c]).norm() / z[c].norm()).item() < tol, c
+    k.close()
+    ref.close()
