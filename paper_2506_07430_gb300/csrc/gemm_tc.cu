@@ -347,6 +347,8 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             prefetch_map(&maps.fa[i]);
         }
     }
+    // (before the allocation: a waiting CTA holds no tensor memory)
+    grid_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
                      ::"r"(su32(holder)) : "memory");
@@ -777,9 +779,9 @@ void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int gr
                diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
                kbs_a.as<int>(), kbl_a.as<int>()};
     const unsigned grid = nc * gemm_grid(nb, na, bn);
-    if (bn == 256) k_gemm<256><<<grid, GM_THREADS, gemm_smem<256>(), st>>>(maps, g);
-    else if (bn == 128) k_gemm<128><<<grid, GM_THREADS, gemm_smem<128>(), st>>>(maps, g);
-    else k_gemm<64><<<grid, GM_THREADS, gemm_smem<64>(), st>>>(maps, g);
+    if (bn == 256) launch_chained(k_gemm<256>, grid, GM_THREADS, gemm_smem<256>(), st, maps, g);
+    else if (bn == 128) launch_chained(k_gemm<128>, grid, GM_THREADS, gemm_smem<128>(), st, maps, g);
+    else launch_chained(k_gemm<64>, grid, GM_THREADS, gemm_smem<64>(), st, maps, g);
     KPM_LAUNCHED();
 }
 

@@ -145,6 +145,8 @@ __global__ void __launch_bounds__(RED_THREADS)
 k_cheb_update(const T* __restrict__ s, const T* __restrict__ c, T* __restrict__ prev, int64_t dim,
               double a, double b, int first, double* partials, unsigned* counters, double* dots,
               int64_t dstride, unsigned* step) {
+    grid_let_next();
+    grid_wait();
     // n from the device counter if given (replayable captured steps), else 0
     const int64_t n = step ? (int64_t)(*step) : 0;
     const bool last = cheb_update_cta<T>(blockIdx.x, gridDim.x, blockIdx.y, s, c, prev, dim, a, b,
@@ -204,8 +206,8 @@ static void launch_update(const T* s, const T* c, T* prev, int64_t dim, int ncol
                           double b, int first, double* partials, unsigned* counters, double* dots,
                           int64_t dstride, unsigned* step, cudaStream_t st) {
     dim3 grid(reduce_blocks(dim), ncol);
-    k_cheb_update<T><<<grid, RED_THREADS, 0, st>>>(s, c, prev, dim, a, b, first, partials,
-                                                   counters, dots, dstride, step);
+    launch_chained(k_cheb_update<T>, grid, RED_THREADS, 0, st, s, c, prev, dim, a, b, first,
+                   partials, counters, dots, dstride, step);
     KPM_LAUNCHED();
 }
 

@@ -228,6 +228,7 @@ __device__ __forceinline__ void rows_d_items(const double* __restrict__ x, const
 // alone would leave threads idle.
 __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, int64_t col) {
     extern __shared__ __align__(16) unsigned char smem[];
+    grid_let_next();
     const int nsb = (int)m.nsb, nsa = (int)m.nsa;
     const int noA = m.noffA, noB = m.noffB, NO = m.NO, K = m.K, kp = m.K | 1;
     const int nfa = m.nnbrA - 1, nfb = m.nnbrB - 1;
@@ -258,14 +259,18 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
         sFv[t] = fvA[(int64_t)(t + 1) * nsa + ia];
         sFo[t] = (uint32_t)m.fcolA[(int64_t)(t + 1) * nsa + ia] * (uint32_t)nsb;
     }
-    if (m.stage_x)
-        for (int j = threadIdx.x; j < nsb; j += blockDim.x) sX[j] = x[myrow + j];
     for (int j = threadIdx.x; j < nsb; j += blockDim.x) ptr[j] = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < NO * K; i += blockDim.x) {
         const int s = i / K, e = i - s * K;
         sB[s * kp + e] = e < noA ? flip(woo[s * NO + (sS[e] & 0x7FFF)], sS[e] >> 15)
                                  : static_cast<const double*>(m.vA)[(int64_t)s * nsa + ia];
+    }
+    // x is the previous kernel's output and y may still be its input; all above is tables
+    grid_wait();
+    if (m.stage_x) {
+        for (int j = threadIdx.x; j < nsb; j += blockDim.x) sX[j] = x[myrow + j];
+        __syncthreads();
     }
 
     // terms of J: same-spin beta, same-spin alpha, alpha off-diagonal x beta diagonal
@@ -978,7 +983,7 @@ void sigma_rows(const BatchMol& m, cudaStream_t st) {
     }
     const dim3 grid((unsigned)m.nsa, (unsigned)m.ncol);
     set_smem(k_sigma_rows, m.smem);
-    k_sigma_rows<<<grid, m.threads, m.smem, st>>>(m);
+    launch_chained(k_sigma_rows, grid, m.threads, m.smem, st, m);
     KPM_LAUNCHED();
 }
 

@@ -416,8 +416,10 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
     };
     for (int64_t j = tid; j < Nrow + RP_SINK; j += RP_THREADS) srow[j] = 0;
     load_slots(blockIdx.x, rsl, tid);
+    grid_wait();           // all above is tables and shared memory
     tc_fence_before();
     __syncthreads();
+    grid_let_next();       // (with this CTA's tensor memory allocated)
     tc_fence_after();
     const uint32_t tbase = *tmem_holder;
     constexpr uint32_t idesc = instr_desc(128, P, !FP16) | (1u << 15);  // A MN-major
@@ -818,6 +820,8 @@ constexpr int SPLIT_T = 64;
 template <bool FP16>
 __global__ void __launch_bounds__(256) k_prepare(const Prepare p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_let_next();
+    grid_wait();
     if (blockIdx.x < p.nscale) {
         row_scale<FP16>((int64_t)blockIdx.x * 8 + warp, p.rowmax, p.rtgt, p.rslot, p.wrow, p.wr,
                         p.R, p.nblk, p.rnexc, p.ndiag, p.P, p.wscale, p.nexc_c, p.amax, p.rscale);
@@ -886,6 +890,7 @@ __global__ void __launch_bounds__(256) k_prepare(const Prepare p) {
 __global__ void k_rowmax(const float* __restrict__ x, int64_t nrow, int64_t ncol, int64_t per,
                          float* __restrict__ rowmax, unsigned* out) {
     __shared__ float wmx[8];
+    grid_let_next();
     for (int64_t r = blockIdx.x; r < nrow; r += gridDim.x) {
         float mx = 0.f;
         for (int64_t j = threadIdx.x; j < ncol; j += blockDim.x) mx = fmaxf(mx, fabsf(x[r * ncol + j]));
@@ -1248,7 +1253,7 @@ void TcSigma::prepare(const float* x, const float* am, int nc, cudaStream_t st) 
                     rtgt_a.as<int32_t>(), rslot_a.as<uint16_t>(), wimg.as<uint16_t>(),
                     wdiag.as<double>(), noff, ndiag, P, wscale, tb->nexc, rscale.as<float2>()};
     auto* fn = fp16 ? k_prepare<true> : k_prepare<false>;
-    fn<<<p.nscale + nc * tx * ty, 256, 0, st>>>(p);
+    launch_chained(fn, p.nscale + nc * tx * ty, 256, 0, st, p);
     KPM_LAUNCHED();
 }
 
@@ -1275,7 +1280,8 @@ void TcSigma::launch_rowpass(const uint16_t* xh, const uint16_t* xl, float* Y, i
         KPM_CUDA(cudaEventRecord(ev[ev_used], st));
     }
     // (smem_bytes is sized for the most stages init allowed)
-    KPM_CUDA(cudaLaunchKernel(kernel, dim3(g1), dim3(RP_THREADS), args1, smem_bytes, st));
+    Chained ch(dim3(g1), dim3(RP_THREADS), smem_bytes, st);
+    KPM_CUDA(cudaLaunchKernelExC(&ch.cfg, kernel, args1));
     KPM_LAUNCHED();
     if (prof) {
         KPM_CUDA(cudaEventRecord(ev[ev_used + 1], st));
