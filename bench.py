@@ -415,7 +415,7 @@ def run_ours(args, ws, rank, local, pg):
         peak = alu_peak_tflops(args.precision, float(peaks.get("sm_max_mhz", 2070.0)))
         peak_note = ("FP32 CUDA cores 152 SM x 128 lanes x 2 x max clock" if args.precision == "fp32"
                      else "GB300 FP64 1.25 TFLOP/s")
-        kname, share = "H application (k_sigma_gather)", sig_ms / ms
+        kname, share = "H application (CUDA-core sigma)", sig_ms / ms
     achieved = flops / per_launch_s / 1e12
     traffic, traffic_src = ncu_traffic(args.workload, args.precision)
     roof = {"bound": bound, "achieved": round(achieved, 4), "peak": round(peak, 2),
