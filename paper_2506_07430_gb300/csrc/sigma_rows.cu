@@ -850,11 +850,11 @@ SigmaPath sigma_path(const SpinTables& A, const SpinTables& B, bool f64) {
     sigma_shape(m, A, B, f64);
     if (f64) {
         rows_geometry(m);
-        // A chunk of one or two entries of D (rows of 5,500 strings and more) leaves half of
-        // a thread's four to six empty and reads x again for each: 16 orbitals with 3 + 6
-        // electrons, 8008 strings a row, 90.1 ms against 76.9 in the gather kernel; chunks
-        // of six (14 orbitals, 7 + 7) 76.8 ms against 224.7
-        if (m.fc < 3 && m.fc < m.noffB) return SIGMA_GATHER;
+        // Chunks of a single entry of D (rows of about 7,000 strings and more) leave three of
+        // a thread's four empty and read x again for each: 16 orbitals with 3 + 6 electrons,
+        // 8008 strings a row, 90.1 ms against 76.9 in the gather kernel; chunks of two
+        // (15 orbitals, 2 + 7) 6.8 ms against 7.8, of six (14, 7 + 7) 76.8 against 224.7
+        if (m.fc < 2 && m.fc < m.noffB) return SIGMA_GATHER;
         return m.smem <= SMEM_MAX ? SIGMA_ROWS : SIGMA_GATHER;
     }
     // (FP32 rows of up to 252 strings, 10 orbitals, stay with the gather kernel: a

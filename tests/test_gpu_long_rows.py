@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,na,nb", [
     (14, 3, 6),     # 364 rows of 3003 strings: chunks of several entries
-    (16, 3, 6),     # 560 rows of 8008: one or two
+    (16, 3, 6),     # 560 rows of 8008: a single one
 ])
 def test_long_rows_fp64(n, na, nb):
     import torch
