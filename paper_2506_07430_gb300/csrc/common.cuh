@@ -182,7 +182,10 @@ private:
 // still runs, and waits (grid_wait) before it reads or writes anything that another kernel
 // of the step does.  What it does before that, on tables that are final when kpm_create
 // returns, and its launch overlap the predecessor's end.  A kernel lets its successor start
-// with grid_let_next; under a normal launch both do nothing.  256 moments of 8 orbitals
+// with grid_let_next; under a normal launch both do nothing.  What the kernel before writes
+// is read by ordinary loads: the read-only path (__ldg, and what the compiler makes of a
+// const __restrict__ pointer) is defined only for memory that nobody writes while the
+// kernel lives.  256 moments of 8 orbitals
 // 4152 -> 4017 us, three MIXED columns of 10 orbitals 58.2 -> 54.2 us, BF16 at 13 orbitals
 // 408 -> 402; the same bits.  The batched kernels of small molecules lose by it (7297 ->
 // 7450 us: waiting CTAs hold the shared memory that the last ones of the running kernel

@@ -483,6 +483,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             constexpr int EG = 16;
             const int ncols = m < g.M ? min(EPI_COLS, g.N - nb) : 0;
             float* y = g.y + col * dim;
+            // (x and the diagonal were final before this kernel could start; y was not)
             const float* x = g.x + col * dim;
 #pragma unroll 1
             for (int u0 = 0; u0 < ncols; u0 += EG) {

@@ -85,12 +85,14 @@ __device__ __forceinline__ bool finish_reduce(double u, double v, double* partia
 
 // Block blk (of nblk) of column col of the update; dots of step n go to
 // dots[2n], dots[2n+1].  Shared by the single-molecule kernel and the batched
-// one, so that both do the same arithmetic and reduction.
+// one, so that both do the same arithmetic and reduction.  s and c are read by ordinary
+// loads (no const __restrict__): their writers may still run when a chained update starts.
+// The loads of a few elements (FP64 two, as many as a thread has up to 622,592; FP32 four) are
+// issued before their first store, which might alias them for all the compiler knows.
 template <class T>
 __device__ __forceinline__ bool cheb_update_cta(int blk, int nblk, int col,
-                                                const T* __restrict__ s, const T* __restrict__ c,
-                                                T* __restrict__ prev, int64_t dim, double a,
-                                                double b, int first, double* partials,
+                                                const T* s, const T* c, T* prev, int64_t dim,
+                                                double a, double b, int first, double* partials,
                                                 unsigned* counters, double* dots, int64_t dstride,
                                                 int64_t n) {
     dots += 2 * n;
@@ -101,13 +103,27 @@ __device__ __forceinline__ bool cheb_update_cta(int blk, int nblk, int col,
     double ss = 0.0, tt = 0.0;
     if constexpr (sizeof(T) == 8) {
         const double k1 = (first ? 1.0 : 2.0) / a, k2 = b * k1;
-        for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < dim; i += stride) {
-            double cv = c[i];
-            double nx = k1 * s[i] - k2 * cv;
-            if (!first) nx -= prev[i];
-            prev[i] = nx;
-            ss += cv * cv;
-            tt += nx * cv;
+        for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < dim; i += 2 * stride) {
+            double cv[2], sv[2], pv[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int64_t j = i + u * stride;
+                const bool in = j < dim;
+                cv[u] = in ? c[j] : 0.0;
+                sv[u] = in ? s[j] : 0.0;
+                pv[u] = in && !first ? prev[j] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int64_t j = i + u * stride;
+                if (j < dim) {
+                    double nx = k1 * sv[u] - k2 * cv[u];
+                    if (!first) nx -= pv[u];
+                    prev[j] = nx;
+                    ss += cv[u] * cv[u];
+                    tt += nx * cv[u];
+                }
+            }
         }
     } else {
         // k1 = 2/a and k2 = 2b/a as float pairs (hi + lo): rounding them to one float
@@ -119,16 +135,23 @@ __device__ __forceinline__ bool cheb_update_cta(int blk, int nblk, int col,
         int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
         while (i < dim) {
             float gs = 0.f, gt = 0.f;
+            float cv[4], sv[4], pv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t j = i + u * stride;
+                const bool in = j < dim;
+                cv[u] = in ? c[j] : 0.f;
+                sv[u] = in ? s[j] : 0.f;
+                pv[u] = in && !first ? prev[j] : 0.f;
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (i < dim) {
-                    float cv = c[i];
-                    const float sv = s[i];
-                    float nx = fmaf(k1, sv, fmaf(-k2, cv, fmaf(k1l, sv, -k2l * cv)));
-                    if (!first) nx -= prev[i];
+                    float nx = fmaf(k1, sv[u], fmaf(-k2, cv[u], fmaf(k1l, sv[u], -k2l * cv[u])));
+                    if (!first) nx -= pv[u];
                     prev[i] = nx;
-                    gs = fmaf(cv, cv, gs);
-                    gt = fmaf(nx, cv, gt);
+                    gs = fmaf(cv[u], cv[u], gs);
+                    gt = fmaf(nx, cv[u], gt);
                 }
                 i += stride;
             }
@@ -142,7 +165,7 @@ __device__ __forceinline__ bool cheb_update_cta(int blk, int nblk, int col,
 
 template <class T>
 __global__ void __launch_bounds__(RED_THREADS)
-k_cheb_update(const T* __restrict__ s, const T* __restrict__ c, T* __restrict__ prev, int64_t dim,
+k_cheb_update(const T* s, const T* c, T* prev, int64_t dim,
               double a, double b, int first, double* partials, unsigned* counters, double* dots,
               int64_t dstride, unsigned* step) {
     grid_let_next();

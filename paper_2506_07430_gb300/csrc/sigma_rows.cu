@@ -185,7 +185,7 @@ __global__ void k_dense_f(const int32_t* __restrict__ fcol, const float* __restr
 
 // D of FT entries at a time over the items (group of FT entries, J) of a chunk.
 template <int FT>
-__device__ __forceinline__ void rows_d_items(const double* __restrict__ x, const double* sB, double* sD,
+__device__ __forceinline__ void rows_d_items(const double* x, const double* sB, double* sD,
                                              const uint32_t* rowoff, int K, int kp,
                                              const uint16_t* __restrict__ slotT, int nsb, int f0,
                                              int f1) {
@@ -205,14 +205,14 @@ __device__ __forceinline__ void rows_d_items(const double* __restrict__ x, const
         for (; e + 4 <= K; e += 4) {
             double a[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = __ldg(x + rowoff[e + u] + J);
+            for (int u = 0; u < 4; ++u) a[u] = x[rowoff[e + u] + J];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
                 for (int i = 0; i < FT; ++i) acc[i] = fma(bp[i][e + u], a[u], acc[i]);
         }
         for (; e < K; ++e) {
-            const double a = __ldg(x + rowoff[e] + J);
+            const double a = x[rowoff[e] + J];
 #pragma unroll
             for (int i = 0; i < FT; ++i) acc[i] = fma(bp[i][e], a, acc[i]);
         }
@@ -233,8 +233,9 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
     const int noA = m.noffA, noB = m.noffB, NO = m.NO, K = m.K, kp = m.K | 1;
     const int nfa = m.nnbrA - 1, nfb = m.nnbrB - 1;
     const int64_t dim = m.nsa * m.nsb;
-    const double* __restrict__ x = static_cast<const double*>(m.x) + col * dim;
-    double* __restrict__ y = static_cast<double*>(m.y) + col * dim;
+    // (ordinary loads of x: its writer may still run when this CTA starts)
+    const double* x = static_cast<const double*>(m.x) + col * dim;
+    double* y = static_cast<double*>(m.y) + col * dim;
     double* sB = reinterpret_cast<double*>(smem);                 // [NO][kp] signed W of this row
     double* sD = sB + (size_t)NO * kp;                       // [fc][nsb]
     double* sP = sD + (size_t)m.fc * nsb;                    // [parts][nsb] if parts > 1
@@ -275,7 +276,7 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
 
     // terms of J: same-spin beta, same-spin alpha, alpha off-diagonal x beta diagonal
     const int nt = nfb + nfa + noA;
-    const double* __restrict__ xr = m.stage_x ? sX : x + myrow;
+    const double* xr = m.stage_x ? sX : x + myrow;
     for (int w = threadIdx.x; w < nsb * m.parts; w += blockDim.x) {
         const int part = w / nsb, J = w - part * nsb;
         const int t0 = (int)((int64_t)nt * part / m.parts);
@@ -307,20 +308,20 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
             for (; u + 4 <= end; u += 4) {
                 double xv[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = __ldg(x + sFo[u + i] + J);
+                for (int i = 0; i < 4; ++i) xv[i] = x[sFo[u + i] + J];
                 a0 = fma(sFv[u], xv[0], a0);
                 a1 = fma(sFv[u + 1], xv[1], a1);
                 a0 = fma(sFv[u + 2], xv[2], a0);
                 a1 = fma(sFv[u + 3], xv[3], a1);
             }
-            for (; u < end; ++u) a0 = fma(sFv[u], __ldg(x + sFo[u] + J), a0);
+            for (; u < end; ++u) a0 = fma(sFv[u], x[sFo[u] + J], a0);
             t = max(t, min(t1, nfb + nfa));
         }
         {
             const int end = t1 - nfb - nfa;
             for (int e = t - nfb - nfa; e < end; ++e) {
                 const double v = __ldg(vB + (int64_t)(sS[e] & 0x7FFF) * nsb + J);
-                a1 = fma(flip(v, sS[e] >> 15), __ldg(x + rowoff[e] + J), a1);
+                a1 = fma(flip(v, sS[e] >> 15), x[rowoff[e] + J], a1);
             }
         }
         if (m.parts > 1) sP[part * nsb + J] = a0 + a1;

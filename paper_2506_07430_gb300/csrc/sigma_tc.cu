@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
         // without swizzle), two entries e at a time; the diagonal column from w_R in FP64
         auto build_b = [&](int64_t idx, const uint16_t* sl) {
             const int64_t rg = row_all(idx), ir = row_own(rg);
-            const float bscale = __ldg(&p.rscale[rg].x);
+            const float bscale = p.rscale[rg].x;   // (k_prepare may have ended after this CTA's start: no __ldg)
 #pragma unroll 4
             for (int i = rt; i < KR / 2 * P; i += RP_ROW_THREADS) {
                 const int e = i / P * 2, nn = i - (i / P) * P;
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
             // abort at any time)
             // sigma out, cleared for the next item, whose B_R is built meanwhile
             {
-                const float inv = __ldg(&p.rscale[rg].y);
+                const float inv = p.rscale[rg].y;
                 const int64_t nout = Nc - lo < Nrow ? Nc - lo : Nrow;   // this pass's targets
                 for (int64_t j = rt; j < Nrow; j += RP_ROW_THREADS) {
                     if (j < nout) p.Y[rg * Nc + lo + j] = (float)srow[j] * inv;
@@ -710,13 +710,14 @@ __global__ void __launch_bounds__(RP_THREADS, 1) k_rowpass(const RowPass p) {
 
 // Scale of B_R and of the row's integer sums (see "Fixed-point range"), one warp per
 // row: c_s (in units of the W image; piece 0 of W is within 2^-8 of W in either
-// format: 1 % margin) and max |B| over the lanes' slots s.
+// format: 1 % margin) and max |B| over the lanes' slots s.  (rowmax and amax by ordinary
+// loads: k_rowmax may still run when this kernel starts.)
 template <bool FP16>
 __device__ __forceinline__ void
-row_scale(int64_t rg, const float* __restrict__ rowmax, const int32_t* __restrict__ rtgt,
+row_scale(int64_t rg, const float* rowmax, const int32_t* __restrict__ rtgt,
           const uint16_t* __restrict__ rslot, const uint16_t* __restrict__ wrow,
           const double* __restrict__ wr, int64_t Nr, int nblk, int rnexc, int ndiag, int P,
-          float wscale, int nexc_c, const float* __restrict__ amax, float2* __restrict__ out) {
+          float wscale, int nexc_c, const float* amax, float2* out) {
     constexpr int SL = (176 + 31) / 32;
     const int lane = threadIdx.x & 31;
     if (rg >= Nr * nblk) return;
