@@ -28,8 +28,7 @@
 // row: one SWIZZLE_64B atom row), TMA pipeline of four stages (narrower tiles six or
 // eight; full/empty mbarriers), one warp issues TMA,
 // one issues MMAs, eight warps drain accumulator chunks (see k_gemm) and run the
-// epilogue; clusters of two CTAs on vertically adjacent tiles share (multicast)
-// the B tile.  All waits are bounded.
+// epilogue.  All waits are bounded.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -87,8 +86,8 @@ constexpr int GM_CK = 64 / GM_BK;               // k-blocks per accumulation chu
 #define GM_BACKOFF_NS 256
 #endif
 constexpr uint32_t A_BYTES = GM_BM * GM_BK * 2;  // per piece
-// CTA pairs (clusters of two) on vertically adjacent tiles share the B tile: each
-// CTA loads half of its rows and multicasts them into both
+// Consecutive CTAs take vertically adjacent tiles in pairs that share a list of k-blocks
+// and read the same B tile at about the same time (from L2)
 constexpr int GM_PAIR = 2;
 template <int BN>
 constexpr uint32_t stage_bytes() { return 2 * A_BYTES + 2 * Tile<BN>::B_BYTES; }
@@ -132,25 +131,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(su32(bar))
         : "memory");
 }
-// the same load multicast into every CTA of `mask` (same shared-memory offset,
-// completing bytes on the mbarrier at the same offset in each)
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                               uint64_t* bar, uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-        " [%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(su32(bar)), "h"(mask)
-        : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// all threads of both CTAs of the cluster
-__device__ __forceinline__ void cluster_sync_() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -170,13 +150,6 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
 __device__ __forceinline__ void mma_commit_(uint64_t* b) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  ::"r"(su32(b)) : "memory");
-}
-// arrive (once MMAs complete) on the mbarrier at this offset in every CTA of mask
-__device__ __forceinline__ void mma_commit_mc(uint64_t* b, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-        " [%0], %1;"
-        ::"r"(su32(b)), "h"(mask) : "memory");
 }
 __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -261,13 +234,8 @@ __device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
 }
 
-// Cluster pairs: the two CTAs of a cluster compute row tiles 2 p and 2 p + 1 of
-// the same column tile and share its B operand: CTA r loads B rows
-// [n0 + 128 r, n0 + 128 r + 128) of each piece and multicasts them to both, so
-// each CTA reads 64 of the 96 KB of a stage from L2.  A stage is reloaded only
-// when the MMAs of both CTAs have released it (the MMA commits arrive on the
-// "empty" barrier of both CTAs), and both CTAs sync at the start (barriers
-// initialised) and at the end (no multicast or remote arrive left in flight).
+// Pairs: CTAs 2 p and 2 p + 1 compute row tiles 2 p and 2 p + 1 of the same column tile.
+// Each loads its own A and the whole B tile by plain TMA and waits for no other CTA.
 //
 // Accumulation in chunks: the MMA thread restarts the accumulator every ck
 // k-blocks, alternating two tensor-memory accumulators of BN columns; the
@@ -277,10 +245,10 @@ __device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
 // growing like sqrt(K); in chunks, each accumulator sums a short run and the
 // running sum takes one rounding per chunk.
 template <int BN>
-__global__ void __cluster_dims__(GM_PAIR, 1, 1) __launch_bounds__(GM_THREADS, 1)
+__global__ void __launch_bounds__(GM_THREADS, 1)
 k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     constexpr int STAGES = Tile<BN>::STAGES, EPI_COLS = Tile<BN>::EPI_COLS;
-    constexpr uint32_t B_BYTES = Tile<BN>::B_BYTES, B_HALF = B_BYTES / GM_PAIR;
+    constexpr uint32_t B_BYTES = Tile<BN>::B_BYTES;
     constexpr uint32_t STAGE_BYTES = stage_bytes<BN>();
     static_assert(STAGES * STAGE_BYTES >= GM_EPI_WARPS * EPI_COLS * 32 * 4, "epilogue staging");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -296,7 +264,6 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     int* consumed = issued + 1;                       // stages the MMA thread passed
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t crank = cluster_rank();
     // grouped rasterisation over pairs of row tiles: groups of GROUP_M pairs walk
     // all column tiles, so the group's A panels and the current B panels stay in L2
     const int GROUP_M = g.group_m;
@@ -313,13 +280,11 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     const int first_m = (b / gsize) * GROUP_M;
     const int gm = min(nMP - first_m, GROUP_M);
     const int mp = first_m + (b % gsize) % gm;
-    // (with an odd number of row tiles the last pair's second tile lies past M:
-    // its A loads read the zero fill and its epilogue writes nothing)
-    const int m0 = (mp * GM_PAIR + (int)crank) * GM_BM;
+    const int m0 = (mp * GM_PAIR + (int)(blockIdx.x % GM_PAIR)) * GM_BM;
     const int n0 = ((b % gsize) / gm) * BN;
-    // k-blocks the pair visits (both CTAs the same, as they share the B loads): those
-    // of F_b where the pair's 256 rows have a nonzero, then those of F_a where the
-    // 256-row list tile of F_a around the B tile has one; accumulation chunks do not cross from one to the other
+    // k-blocks the pair visits: those of F_b where the pair's 256 rows have a nonzero, then
+    // those of F_a where the 256-row list tile of F_a around the B tile has one;
+    // accumulation chunks do not cross from one to the other
     const int* kl1 = g.kbl_b + g.kbs_b[mp];
     const int nk1 = g.kbs_b[mp + 1] - g.kbs_b[mp];
     const int* kl2 = g.kbl_a + g.kbs_a[n0 / GM_LIST_N];
@@ -330,7 +295,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init_(&full[s], 1);
-            mbar_init_(&empty[s], GM_PAIR);   // the MMA commits of both CTAs
+            mbar_init_(&empty[s], 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init_(&accf[i], 1);
@@ -349,6 +314,8 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     }
     // (before the allocation: a waiting CTA holds no tensor memory)
     grid_wait();
+    // (with an odd number of row tiles the last pair's second tile lies past M)
+    if (m0 >= g.M) return;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
                      ::"r"(su32(holder)) : "memory");
@@ -356,7 +323,6 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     }
     tc_before();
     __syncthreads();
-    cluster_sync_();   // the peer's barriers are initialised before any multicast or remote arrive
     tc_after();
     const uint32_t tmem = *holder;
 
@@ -377,11 +343,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 const int ma = beta ? m0 : trow_ + m0;
                 tma_load_2d(su32(st), mA, kx, ma, &full[s]);
                 tma_load_2d(su32(st + A_BYTES), mA + 1, kx, ma, &full[s]);
-                // this CTA's half of the B rows, into both CTAs
-                const uint32_t hb = crank * B_HALF;
-                const int nh = (beta ? xrow : 0) + n0 + (int)crank * (BN / GM_PAIR);
-                tma_load_2d_mc(su32(st + 2 * A_BYTES + hb), mB, kx, nh, &full[s], 0x3);
-                tma_load_2d_mc(su32(st + 2 * A_BYTES + B_BYTES + hb), mB + 1, kx, nh, &full[s], 0x3);
+                const int nb = (beta ? xrow : 0) + n0;
+                tma_load_2d(su32(st + 2 * A_BYTES), mB, kx, nb, &full[s]);
+                tma_load_2d(su32(st + 2 * A_BYTES + B_BYTES), mB + 1, kx, nb, &full[s]);
                 *(volatile int*)issued = kb + 1;
             }
         }
@@ -423,7 +387,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                         const uint32_t off = j * 32;
                         mma_ss(d, sw_desc(a0 + off), sw_desc(b0 + off), idesc, 1);
                     }
-                    mma_commit_mc(&empty[s], 0x3);   // stage s released in both CTAs
+                    mma_commit_(&empty[s]);   // stage s released
                 }
                 if (!ok) break;
                 mma_commit_(&accf[c & 1]);
@@ -521,7 +485,6 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             mbar_wait_bounded(&full[kb % STAGES], (kb / STAGES) & 1, g.err);
     }
     __syncthreads();
-    cluster_sync_();   // neither CTA exits while the peer may still write into it
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem)
                      : "memory");
@@ -770,12 +733,12 @@ void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int gr
     GemmMaps maps;
     maps.fb[0] = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
     maps.fb[1] = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
-    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
-    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
+    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, bn);
+    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, bn);
     maps.t[0] = make_map(th.as<__half>(), nc * nb, na, pa, GM_BM);
     maps.t[1] = make_map(tl.as<__half>(), nc * nb, na, pa, GM_BM);
-    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn / GM_PAIR);
-    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn / GM_PAIR);
+    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn);
+    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn);
     GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
                diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
                kbs_a.as<int>(), kbl_a.as<int>()};
