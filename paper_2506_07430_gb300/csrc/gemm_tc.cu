@@ -33,6 +33,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <array>
@@ -191,7 +192,10 @@ struct GemmArgs {
     float* y;                  // y[n * ldy + m] += sums / (wscale sa) + diagonal
     int64_t ldy;
     const float* amax;         // [ncol] max |x| of the split vector operand (operand scale sa)
-    float ratio, inv_wa;       // wscale_a / wscale_b, 1 / wscale_a (powers of two)
+    // The sums are kept at the smaller of the two matrices' scales w (powers of two): to_w_b
+    // = w / wscale_b and to_w_a = w / wscale_a, both at most 1, so that however far apart the
+    // magnitudes of F_a and F_b are, no sum (below 2^45) leaves the range of a float.
+    float to_w_b, to_w_a, inv_w;
     // exact diagonal term (if x != nullptr): y[n*ldy+m] += d[n*ldy+m] * x[n*ldy+m], the
     // diagonal H_II evaluated in FP64 and stored as float (hi, lo)
     const float* x;
@@ -406,11 +410,12 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 ok = wait_or_abort(&accf[c & 1], (c >> 1) & 1, abort_flag, g.err, GM_BACKOFF_NS);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
-            // from the scale of F_b's product to that of F_a's (a power of two)
-            if (c == nchunk1 && g.ratio != 1.f) {
+            // from the scale of F_b's product to the common one, and from F_a's (exact)
+            if (c == nchunk1 && g.to_w_b != 1.f) {
 #pragma unroll
-                for (int u = 0; u < EPI_COLS; ++u) rs[u] *= g.ratio;
+                for (int u = 0; u < EPI_COLS; ++u) rs[u] *= g.to_w_b;
             }
+            const float f = c < nchunk1 ? 1.f : g.to_w_a;
             tc_after();
             const uint32_t src = trow + (uint32_t)((c & 1) * BN);
 #pragma unroll
@@ -418,14 +423,15 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                 uint32_t r[32];
                 ld32(src + (uint32_t)(q * 32), r);
 #pragma unroll
-                for (int u = 0; u < 32; ++u) rs[q * 32 + u] += __uint_as_float(r[u]);
+                for (int u = 0; u < 32; ++u)
+                    rs[q * 32 + u] = fmaf(__uint_as_float(r[u]), f, rs[q * 32 + u]);
             }
             tc_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_(&acce[c & 1]);
         }
         if (ok && !*abort_flag) {
-            float scale = (nchunk == nchunk1 ? g.ratio : 1.f) * g.inv_wa;
+            float scale = (nchunk == nchunk1 ? g.to_w_b : 1.f) * g.inv_w;
             {
                 const float mx = g.amax[col];
                 if (mx > 0.f && isfinite(mx)) {
@@ -606,7 +612,8 @@ static double offdiag_scale(const SpinTables& T, DevBuf& scratch, cudaStream_t s
     if (!(mx > 0.0)) return 1.0;
     int e;
     std::frexp(mx, &e);  // mx < 2^e
-    return std::ldexp(1.0, 14 - e);
+    // (at most 2^300: entries below 2^-324 times a float vanish in a float)
+    return std::ldexp(1.0, 14 - std::max(e, -286));
 }
 
 static void build_f(const SpinTables& T, double ws, DevBuf& hi, DevBuf& lo, DevBuf& dg,
@@ -739,8 +746,9 @@ void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int gr
     maps.t[1] = make_map(tl.as<__half>(), nc * nb, na, pa, GM_BM);
     maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn);
     maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn);
-    GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(wscale_a / wscale_b), (float)(1.0 / wscale_a),
-               diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
+    const double w = std::min(wscale_a, wscale_b);
+    GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(w / wscale_b), (float)(w / wscale_a),
+               (float)(1.0 / w), diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
                kbs_a.as<int>(), kbl_a.as<int>()};
     const unsigned grid = nc * gemm_grid(nb, na, bn);
     if (bn == 256) launch_chained(k_gemm<256>, grid, GM_THREADS, gemm_smem<256>(), st, maps, g);
