@@ -678,7 +678,6 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     pa = half_pitch(na);
     pb = half_pitch(nb);
     xpitch = (nb + 127) / 128 * 128;
-    cb = batch_columns(na * nb);
     err = err_flag;
     int dev = 0;
     KPM_CUDA(cudaGetDevice(&dev));
@@ -707,13 +706,6 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     // operand (lists by GM_LIST_N rows)
     block_lists(B, GM_PAIR * GM_BM, kbs_b, kbl_b, &kb_nonzero[0], &kb_total[0], st);
     block_lists(A, GM_LIST_N, kbs_a, kbl_a, &kb_nonzero[1], &kb_total[1], st);
-}
-
-void DenseSS::reserve() {
-    xh.ensure((size_t)cb * na * xpitch * 2);
-    xl.ensure((size_t)cb * na * xpitch * 2);
-    th.ensure((size_t)cb * nb * pa * 2);
-    tl.ensure((size_t)cb * nb * pa * 2);
 }
 
 // The narrowest tile whose grid is one wave: a tile's time is its k-blocks' MMAs and its
@@ -782,7 +774,10 @@ void DenseSS::autotune(cudaStream_t st) {
         }
     }
     // scratch operands (zeros: the timing does not depend on the values)
-    reserve();
+    xh.ensure(x_bytes(1));
+    xl.ensure(x_bytes(1));
+    th.ensure(t_bytes(1));
+    tl.ensure(t_bytes(1));
     KPM_CUDA(cudaMemsetAsync(xh.p, 0, xh.bytes, st));
     KPM_CUDA(cudaMemsetAsync(xl.p, 0, xl.bytes, st));
     KPM_CUDA(cudaMemsetAsync(th.p, 0, th.bytes, st));

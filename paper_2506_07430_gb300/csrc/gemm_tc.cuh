@@ -9,8 +9,8 @@ int64_t half_pitch(int64_t cols);
 
 // Columns of a block that the tensor-core sigma takes in one set of launches: three (x, y
 // and z of a request) up to 2^24 determinants, where one column's tiles leave a last wave
-// half empty or (below 13 orbitals) most SMs idle; their split copies take 16 bytes per
-// column and determinant.
+// half empty or (below 13 orbitals) most SMs idle; their split copies take 8 bytes per
+// column and determinant (12 for BF16).
 inline int batch_columns(int64_t dim) { return dim <= ((int64_t)1 << 24) ? 3 : 1; }
 
 // sigma += F_b-part + F_a-part of H applied to x (FP32 [N_a][N_b]); see gemm_tc.cu.
@@ -23,8 +23,7 @@ struct DenseSS {
     DevBuf* fa_lo = nullptr;
     DevBuf* da = nullptr;
     int64_t xpitch = 0;                       // row pitch of xh/xl: N_b rounded up to 128
-    int cb = 1;                               // columns per launch (batch_columns)
-    DevBuf xh, xl, th, tl;                    // split copies of x and x^T, cb columns
+    DevBuf xh, xl, th, tl;                    // split copies of x and x^T (TcSigma::hold)
     DevBuf fmax;                              // scratch for max |F_off|
     // per tile of the split matrix, the k-blocks that hold a nonzero (CSR; see
     // block_lists): F_b by pairs of 128-row tiles, F_a by 256-row tiles
@@ -42,7 +41,8 @@ struct DenseSS {
               cudaStream_t st);
     // Split copies of the operand, scaled FP16 pieces with zero padding, written by the
     // caller (k_prepare): rows of x [nc][N_a][xpitch] in xh/xl, of x^T [nc][N_b][pa] in th/tl.
-    void reserve();
+    size_t x_bytes(int nc) const { return (size_t)nc * na * xpitch * 2; }   // each of xh, xl
+    size_t t_bytes(int nc) const { return (size_t)nc * nb * pa * 2; }       // each of th, tl
     // y += (F_a (x) 1 + 1 (x) F_b) x with the off-diagonal parts of F_a, F_b, plus
     // diag_full * x (the whole exact diagonal of H); amax = device max|x|.
     // Reads xh/xl and th/tl, not x's own entries, in the products.

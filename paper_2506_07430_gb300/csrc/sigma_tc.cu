@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <map>
@@ -1207,9 +1208,46 @@ void TcSigma::set_layout(int passes, cudaStream_t st) {
     smem_bytes = sm;
 }
 
+int TcSigma::hold(int ncol, cudaStream_t st) {
+    const int want = std::min(ncol, batch_columns(dim));
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    KPM_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) captured = true;
+    if (want <= held || (held > 0 && cap != cudaStreamCaptureStatusNone)) return std::min(want, held);
+    std::vector<DevBuf*> grown;
+    auto room = [&](DevBuf& b, size_t bytes) {
+        if (bytes <= b.bytes) return;
+        if (captured && b.p) {
+            retired.emplace_back();
+            std::swap(b.p, retired.back().p);
+            std::swap(b.bytes, retired.back().bytes);
+        }
+        grown.push_back(&b);
+        b.alloc(bytes);
+    };
+    auto rooms = [&](int nc) {
+        room(rowmax, (size_t)(nsa > 0 ? nc * nsa : 1) * sizeof(float));
+        room(rscale, (size_t)(nsa > 0 ? nc * nsa : 1) * sizeof(float2));
+        for (DevBuf* b : {&dense.xh, &dense.xl}) room(*b, dense.x_bytes(nc));
+        for (DevBuf* b : {&dense.th, &dense.tl}) room(*b, dense.t_bytes(nc));
+        if (!fp16)
+            for (DevBuf* b : {&xbh, &xbl}) room(*b, dense.x_bytes(nc));
+        held = nc;
+    };
+    const int before = std::max(held, 1);
+    held = 0;
+    try {
+        rooms(want);
+    } catch (const Error& e) {
+        if (e.status != KPM_ENOMEM || want == before) throw;
+        for (DevBuf* b : grown) b->release();
+        rooms(before);
+    }
+    return std::min(want, held);
+}
+
 void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
-    const int cb = dense.cb;
-    rowmax.ensure((size_t)(nsa > 0 ? cb * nsa : 1) * sizeof(float));
+    const int cb = hold(ncol, st);
     for (int c = 0; c < ncol; c += cb) {
         const int nc = ncol - c < cb ? ncol - c : cb;
         const int64_t rows = nc * nsa;
@@ -1235,14 +1273,8 @@ void TcSigma::apply(const float* x, float* y, int ncol, cudaStream_t st) {
 }
 
 void TcSigma::prepare(const float* x, const float* am, int nc, cudaStream_t st) {
-    rscale.ensure((size_t)(nsa > 0 ? dense.cb * nsa : 1) * sizeof(float2));
     unsigned tx = 0, ty = 0;
     if (x) {
-        dense.reserve();
-        if (!fp16) {
-            xbh.ensure((size_t)dense.cb * nsa * dense.xpitch * 2);
-            xbl.ensure((size_t)dense.cb * nsa * dense.xpitch * 2);
-        }
         if (dense.xpitch % SPLIT_T || (dense.pa & 1)) KPM_THROW(KPM_EINVAL, "split: pitch");
         tx = (unsigned)(dense.xpitch / SPLIT_T);
         ty = (unsigned)((nsa + SPLIT_T - 1) / SPLIT_T);
@@ -1321,6 +1353,7 @@ void TcSigma::autotune(cudaStream_t st) {
     KPM_CUDA(cudaMemsetAsync(zl.p, 0, zl.bytes, st));
     KPM_CUDA(cudaMemsetAsync(amax.p, 0, sizeof(unsigned), st));
     rowmax.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float));
+    rscale.ensure((size_t)(nsa > 0 ? nsa : 1) * sizeof(float2));
     KPM_CUDA(cudaMemsetAsync(rowmax.p, 0, rowmax.bytes, st));
     prepare(nullptr, reinterpret_cast<const float*>(amax.p), 1, st);
     cudaEvent_t e0, e1;

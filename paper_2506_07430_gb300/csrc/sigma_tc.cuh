@@ -3,6 +3,7 @@
 #include "common.cuh"
 #include "gemm_tc.cuh"
 
+#include <deque>
 #include <vector>
 
 namespace kpm {
@@ -56,6 +57,16 @@ struct TcSigma {
               const double* d_eri, const float2* d_diag, int n, double wmax, double wcolsum,
               bool use_fp16, cudaStream_t st);
     void apply(const float* x, float* y, int ncol, cudaStream_t st);
+    // Operand buffers for blocks of ncol columns: room for as many of them as one set of
+    // launches takes (batch_columns), or for as many as before (at least one) where the
+    // device has no memory for more.
+    // Returns the columns per set of launches.  Buffers grow to the widest block seen and
+    // are not moved during a stream capture; buffers that a captured graph may name are
+    // kept until the context goes.
+    int hold(int ncol, cudaStream_t st);
+    int held = 0;                 // columns the buffers have room for
+    bool captured = false;        // launches of apply have been captured
+    std::deque<DevBuf> retired;   // outgrown buffers of captured launches
     // Scales of every row from rowmax and max|x| (am), for the next row pass, and the split
     // copies of nc columns of x (none: x == nullptr).
     void prepare(const float* x, const float* am, int nc, cudaStream_t st);
