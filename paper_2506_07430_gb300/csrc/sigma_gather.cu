@@ -272,10 +272,11 @@ k_dipole(const double* __restrict__ psi, T* __restrict__ y, int64_t nsa, int64_t
 // psi[J_a][:] (coalesced across the block's threads).  FP64 operations bound it (two a
 // clock and SM): one FMA per off-diagonal entry, and the 2 m diagonal entries of a
 // determinant as one more, with dA[I_a] + dB[I_b] from two tables over the halves of the
-// occupation mask.  Coefficients with their sign come from a table of d and -d, entries
+// occupation mask, or summed over the mask where a row has fewer strings than the tables
+// have entries (DIAG_TABLES false; the same sums in the same order).  Coefficients with their sign come from a table of d and -d, entries
 // from the packed table, 4 bytes per term.  14 orbitals: 3.69 ms with the diagonal entries
 // one by one and the sign applied per term, 2.04 ms here; 2.0 ms at the FP64 rate.
-template <class T>
+template <class T, bool DIAG_TABLES>
 __global__ void __launch_bounds__(512)
 k_dipole_rows(const double* __restrict__ psi, T* __restrict__ y, int64_t nsb,
               const int32_t* __restrict__ tgtA, const uint16_t* __restrict__ pqA,
@@ -288,24 +289,24 @@ k_dipole_rows(const double* __restrict__ psi, T* __restrict__ y, int64_t nsb,
     double* dd = row + nsb;                              // [2][nn] d, -d
     double* lo = dd + 2 * nn;                            // [2^hb] sum of d_qq over mask bits < hb
     double* hi = lo + (1 << hb);                         // [2^hb] the rest
-    double* cA = hi + (1 << hb);                         // [noffA] signed coefficients
+    double* cA = DIAG_TABLES ? hi + (1 << hb) : lo;      // [noffA] signed coefficients
     int64_t* oA = reinterpret_cast<int64_t*>(cA + noffA);  // [noffA] row offsets
-    __shared__ double own;
     const int64_t ia = blockIdx.x;
     for (int64_t j = threadIdx.x; j < nsb; j += blockDim.x) row[j] = psi[ia * nsb + j];
     for (int i = threadIdx.x; i < nn; i += blockDim.x) {
         dd[i] = d[i];
         dd[nn + i] = -d[i];
     }
-    for (int i = threadIdx.x; i < (2 << hb); i += blockDim.x) {
-        const int base = i >> hb ? hb : 0;
-        double s = 0.0;
-        for (uint32_t mk = i & ((1 << hb) - 1); mk; mk &= mk - 1) {
-            const int q = __ffs(mk) - 1 + base;
-            if (q < n) s += d[q * n + q];
+    if (DIAG_TABLES)
+        for (int i = threadIdx.x; i < (2 << hb); i += blockDim.x) {
+            const int base = i >> hb ? hb : 0;
+            double s = 0.0;
+            for (uint32_t mk = i & ((1 << hb) - 1); mk; mk &= mk - 1) {
+                const int q = __ffs(mk) - 1 + base;
+                if (q < n) s += d[q * n + q];
+            }
+            lo[i] = s;
         }
-        lo[i] = s;
-    }
     // off-diagonal entries of the row: entry order with the diagonal ones left out
     for (int e = threadIdx.x; e < nexcA; e += blockDim.x) {
         const int64_t k = ia * nexcA + e;
@@ -318,12 +319,20 @@ k_dipole_rows(const double* __restrict__ psi, T* __restrict__ y, int64_t nsb,
         oA[e - diag] = (int64_t)tgtA[k] * nsb;
     }
     __syncthreads();
-    if (threadIdx.x == 0)
-        own = lo[maskA[ia] & ((1u << hb) - 1u)] + hi[maskA[ia] >> hb];
-    __syncthreads();
+    // sum of d_qq over a mask: its bits below hb, then the rest
+    auto diag = [&](uint32_t mk) {
+        if (DIAG_TABLES) return lo[mk & ((1u << hb) - 1u)] + hi[mk >> hb];
+        double s[2] = {0.0, 0.0};
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            for (uint32_t m = h ? mk >> hb : mk & ((1u << hb) - 1u); m; m &= m - 1)
+                s[h] += dd[(__ffs(m) - 1 + h * hb) * (n + 1)];
+        return s[0] + s[1];
+    };
+    // (not in warps without a string: the FP64 unit is what the block is bound by)
+    const double own = threadIdx.x < nsb ? diag(maskA[ia]) : 0.0;
     for (int64_t ib = threadIdx.x; ib < nsb; ib += blockDim.x) {
-        const uint32_t mb = maskB[ib];
-        double a0 = (own + (lo[mb & ((1u << hb) - 1u)] + hi[mb >> hb])) * row[ib], a1 = 0.0;
+        double a0 = (own + diag(maskB[ib])) * row[ib], a1 = 0.0;
         int e = 0;
         for (; e + 8 <= noffA; e += 8) {
             double v[8];
@@ -360,15 +369,21 @@ static void launch_dipole(const SpinTables& A, const SpinTables& B, const double
                           const double* psi, T* y, cudaStream_t st) {
     if (A.ns * B.ns == 0) return;
     const int n = A.n, noffA = A.m * (n - A.m), noffB = B.m * (n - B.m);
-    const size_t smem = sizeof(double) * ((size_t)B.ns + 2 * n * n + (2 << ((n + 1) / 2)) +
+    // short rows: the tables would cost more than the row's own sums (16 orbitals, 8 + 1:
+    // 158 us with them, 88 without; 18 orbitals, 1 + 1: 12.4 and 8.2 us; 18 orbitals, 9 + 2,
+    // rows of 153: 2236 and 1750)
+    const int entries = 2 << ((n + 1) / 2);
+    const bool tables = B.ns > entries;
+    const size_t smem = sizeof(double) * ((size_t)B.ns + 2 * n * n + (tables ? entries : 0) +
                                           2 * (size_t)noffA);
     if (smem <= 200 * 1024) {
+        auto* fn = tables ? k_dipole_rows<T, true> : k_dipole_rows<T, false>;
         // per device; cheap, and the dipole runs once per request
-        KPM_CUDA(cudaFuncSetAttribute(k_dipole_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        KPM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       200 * 1024));
         // as many threads as keep 16 warps or more on an SM
         const int threads = B.ns <= 128 ? 128 : smem > 56 * 1024 ? 512 : 256;
-        k_dipole_rows<T><<<(unsigned)A.ns, threads, smem, st>>>(
+        fn<<<(unsigned)A.ns, threads, smem, st>>>(
             psi, y, B.ns, A.tgt.as<int32_t>(), A.pq.as<uint16_t>(), A.sgn.as<int8_t>(), A.nexc,
             noffA, A.masks.as<uint32_t>(), B.masks.as<uint32_t>(), B.pkT.as<uint32_t>(), noffB, d,
             n);
