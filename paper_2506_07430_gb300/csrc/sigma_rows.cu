@@ -262,7 +262,8 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
     }
     for (int j = threadIdx.x; j < nsb; j += blockDim.x) ptr[j] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < NO * K; i += blockDim.x) {
+    // (read for D only, which strings without an off-diagonal entry do not have)
+    for (int i = noB > 0 ? threadIdx.x : NO * K; i < NO * K; i += blockDim.x) {
         const int s = i / K, e = i - s * K;
         sB[s * kp + e] = e < noA ? flip(woo[s * NO + (sS[e] & 0x7FFF)], sS[e] >> 15)
                                  : static_cast<const double*>(m.vA)[(int64_t)s * nsa + ia];
@@ -850,6 +851,13 @@ SigmaPath sigma_path(const SpinTables& A, const SpinTables& B, bool f64) {
     BatchMol m{};
     sigma_shape(m, A, B, f64);
     if (f64) {
+        // Few terms a determinant: its thread in the gather kernel is done before a row's
+        // tables are staged.  512 moments, gather and row kernel: (2; 1,1) 10 terms 2.69 and
+        // 3.21 ms, (4; 2,1) 34 terms 3.47 and 3.74, (5; 1,1) 35 terms 3.74 both (x, y and z
+        // 3.82 and 3.50), (4; 2,2) 48 terms 4.00 and 3.47.  Without opposite-spin entries
+        // (8; 4,0) 54 terms 3.21 and 3.47, (10; 5,0) 127 terms 4.52 and 4.25.
+        const int terms = m.nexcA * m.nexcB + m.nnbrA + m.nnbrB;
+        if (terms < (m.noffB > 0 ? 35 : 64)) return SIGMA_GATHER;
         rows_geometry(m);
         // Chunks of a single entry of D (rows of about 7,000 strings and more) leave three of
         // a thread's four empty and read x again for each: 16 orbitals with 3 + 6 electrons,
