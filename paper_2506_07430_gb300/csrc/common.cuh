@@ -161,16 +161,22 @@ struct PairTables {
         DevBuf c;       // double [n][ns] the same of (ii|qq)
         DevBuf dense;   // float [ns][ld] off-diagonal string Hamiltonian (k_same_dense)
         int64_t ld = 0;
+        void release() {
+            for (DevBuf* d : {&otgt, &oslot, &slotT, &back, &revT, &stgt, &v, &c, &dense}) d->release();
+        }
     };
     SigmaPath path = SIGMA_GATHER;
     bool f64 = false;
     DevBuf woo;         // T [NO][NO] (pq|rs)
     Spin a, b_own;
     Spin* b = nullptr;
+    // without memory for the tables: none, and path SIGMA_GATHER
     void build(const SpinTables& A, const SpinTables& B, const double* eri, bool f64,
                cudaStream_t st);
     void fill(BatchMol& m) const;   // after sigma_shape
 private:
+    void build_tables(const SpinTables& A, const SpinTables& B, const double* eri,
+                      cudaStream_t st);
     void build_spin(Spin& t, const SpinTables& T, const double* eri, SigmaPath path, bool f64,
                     cudaStream_t st);
 };

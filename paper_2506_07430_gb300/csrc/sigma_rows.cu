@@ -955,6 +955,23 @@ void PairTables::build(const SpinTables& A, const SpinTables& B, const double* e
     f64 = f64_;
     path = sigma_path(A, B, f64);
     if (path == SIGMA_GATHER) return;
+    try {
+        build_tables(A, B, eri, st);
+    } catch (const Error& e) {
+        // no memory for the row kernels' tables (the dense F of 48620 strings is 9.5 GB, five
+        // times everything else that such a context holds): the gather kernel needs none
+        if (e.status != KPM_ENOMEM) throw;
+        KPM_CUDA(cudaStreamSynchronize(st));
+        woo.release();
+        a.release();
+        b_own.release();
+        b = nullptr;
+        path = SIGMA_GATHER;
+    }
+}
+
+void PairTables::build_tables(const SpinTables& A, const SpinTables& B, const double* eri,
+                              cudaStream_t st) {
     const int NO = A.n * (A.n - 1) / 2;
     woo.alloc((size_t)NO * NO * (f64 ? 8 : 4) + 8);
     if (NO > 0) {
