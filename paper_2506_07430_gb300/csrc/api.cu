@@ -567,11 +567,26 @@ kpm_status rec_collect(kpm_ctx* c, double* out, int nm_stride) {
 
 }  // namespace
 
-extern "C" {
+size_t kpm::context_bytes(int norb, int nalpha, int nbeta, int ncol, kpm_precision prec,
+                          bool lean) {
+    SpinTables ta, tb_own;
+    spin_shape(ta, norb, nalpha);
+    if (nalpha != nbeta) spin_shape(tb_own, norb, nbeta);
+    const SpinTables& tb = nalpha != nbeta ? tb_own : ta;
+    const size_t dim = (size_t)ta.ns * tb.ns, n2 = (size_t)norb * norb;
+    const bool f64 = prec == KPM_FP64;
+    size_t v = 3 * ncol * dim * (f64 ? 8 : 4);        // the recursion's vectors
+    v += f64 ? 0 : dim * sizeof(float2);              // exact diagonal
+    v += spin_table_bytes(ta) + (nalpha != nbeta ? spin_table_bytes(tb) : 0);
+    v += 8 * n2 * n2 + (prec == KPM_FP32 ? 4 * n2 * n2 : 0) + 32 * n2;   // integrals
+    if (prec == KPM_FP64 || prec == KPM_FP32) v += PairTables::bytes(ta, tb, f64, !lean);
+    else v += TcSigma::bytes(ta, tb, prec == KPM_MIXED, lean ? 1 : ncol);
+    return v;
+}
 
-kpm_status kpm_create(const double* h1, const double* eri, const double* dipole, int norb,
-                      int nalpha, int nbeta, kpm_precision prec, void* cuda_stream,
-                      kpm_ctx** out) {
+kpm_status kpm::create_context(const double* h1, const double* eri, const double* dipole,
+                               int norb, int nalpha, int nbeta, kpm_precision prec, bool lean,
+                               void* cuda_stream, kpm_ctx** out) {
     if (out) *out = nullptr;
     std::unique_ptr<kpm_ctx> c;
     kpm_status s = guarded(nullptr, [&] {
@@ -615,7 +630,8 @@ kpm_status kpm_create(const double* h1, const double* eri, const double* dipole,
             c->d_diag.alloc((size_t)c->dim * sizeof(float2));
             exact_diagonal(c->ta, *c->tb, c->d_eri.as<double>(), norb, c->d_diag.as<float2>(), c->st);
         }
-        if (prec == KPM_FP64 || prec == KPM_FP32)
+        if (prec == KPM_FP64 || (prec == KPM_FP32 &&
+                                 !(lean && sigma_path(c->ta, *c->tb, false) == SIGMA_SLOTS)))
             c->pairs.build(c->ta, *c->tb, c->d_eri.as<double>(), prec == KPM_FP64, c->st);
         if (prec == KPM_MIXED || prec == KPM_MIXED_BF16) {
             // W over unordered pairs {p<=q}: rows (pq|rs) and the one-body row k_pq.
@@ -643,6 +659,7 @@ kpm_status kpm_create(const double* h1, const double* eri, const double* dipole,
             c->d_diag.alloc((size_t)c->dim * sizeof(float2));
             exact_diagonal(c->ta, *c->tb, c->d_eri.as<double>(), norb, c->d_diag.as<float2>(), c->st);
             c->tc.reset(new TcSigma());
+            if (lean) c->tc->most = 1;
             c->tc->init(c->ta, *c->tb, c->d_h1.as<double>(), c->d_eri.as<double>(),
                         c->d_diag.as<float2>(), norb, wmax, wcol, prec == KPM_MIXED, c->st);
         }
@@ -650,6 +667,14 @@ kpm_status kpm_create(const double* h1, const double* eri, const double* dipole,
     });
     if (s == KPM_OK) *out = c.release();
     return s;
+}
+
+extern "C" {
+
+kpm_status kpm_create(const double* h1, const double* eri, const double* dipole, int norb,
+                      int nalpha, int nbeta, kpm_precision prec, void* cuda_stream,
+                      kpm_ctx** out) {
+    return create_context(h1, eri, dipole, norb, nalpha, nbeta, prec, false, cuda_stream, out);
 }
 
 void kpm_destroy(kpm_ctx* ctx) {

@@ -106,6 +106,9 @@ struct Binom {
 };
 Binom make_binom();
 
+// n, m and the sizes that follow from them
+void spin_shape(SpinTables& t, int n, int m);
+size_t spin_table_bytes(const SpinTables& t);   // what build_spin_tables allocates
 void build_spin_tables(SpinTables& t, int n, int m, const double* d_h1, const double* d_eri,
                        cudaStream_t st);
 
@@ -170,6 +173,8 @@ struct PairTables {
     DevBuf woo;         // T [NO][NO] (pq|rs)
     Spin a, b_own;
     Spin* b = nullptr;
+    // bytes that build allocates; dense: with the FP32 path's dense string Hamiltonians
+    static size_t bytes(const SpinTables& A, const SpinTables& B, bool f64, bool dense);
     // without memory for the tables: none, and path SIGMA_GATHER
     void build(const SpinTables& A, const SpinTables& B, const double* eri, bool f64,
                cudaStream_t st);
@@ -301,6 +306,18 @@ void cheb_update_batch_f64(const BatchMol* mols, int nmol, int64_t blocks, int k
                            cudaStream_t st);
 void cheb_update_batch_f32(const BatchMol* mols, int nmol, int64_t blocks, int k,
                            cudaStream_t st);
+
+// ---------------------------------------------------------------- contexts
+
+// kpm_create; lean: without the buffers that only buy speed at the price of memory beyond
+// the vectors' own (the dense string Hamiltonians of the FP32 path, whose contexts then run
+// the gather kernel; split copies of more than one column on the tensor-core paths).
+kpm_status create_context(const double* h1, const double* eri, const double* dipole, int norb,
+                          int nalpha, int nbeta, kpm_precision prec, bool lean,
+                          void* cuda_stream, kpm_ctx** out);
+// Device bytes of such a context with a recursion of ncol columns begun on it, to within
+// the reduction scratch, the moments and the allocator's granularity.
+size_t context_bytes(int norb, int nalpha, int nbeta, int ncol, kpm_precision prec, bool lean);
 
 // ---------------------------------------------------------------- recursion helpers
 

@@ -33,7 +33,6 @@
 #include <unordered_map>
 
 #include "common.cuh"
-#include "gemm_tc.cuh"
 
 using namespace kpm;
 
@@ -62,6 +61,7 @@ struct Req {
     bool deflate = false;
     double e0 = 0.0;
     size_t mem = 0;
+    bool lean = false;            // fits the whole budget only without the buffers for speed
     double t_submit = 0, t_admit = 0, t_done = 0;
     bool done = false;
     std::atomic<bool> cancelled{false};
@@ -81,31 +81,11 @@ struct Slot {
     std::string fail_msg;
 };
 
-// Device bytes a request keeps resident (vectors, workspaces, tables).
-size_t estimate_bytes(int n, int na, int nb, int ncol, kpm_precision prec) {
-    int64_t sa = binom(n, na), sb = binom(n, nb), dim = sa * sb;
-    size_t esz = prec == KPM_FP64 ? 8 : 4;
-    size_t v = (size_t)dim * esz * 3 * ncol + (size_t)dim * 8;
-    v += prec == KPM_FP64 ? 0 : (size_t)dim * 8;   // exact diagonal (hi, lo floats)
-    if (prec == KPM_MIXED || prec == KPM_MIXED_BF16) {
-        // split FP16 copies of x and x^T, dense split string Hamiltonians
-        v += (size_t)dim * 8 * batch_columns(dim) + (size_t)4 * sa * ((sa + 7) / 8 * 8);
-        if (na != nb) v += (size_t)4 * sb * ((sb + 7) / 8 * 8);
-    }
-    auto tables = [&](int m, int64_t ns) {
-        int64_t nexc = m * (n - m + 1);
-        int64_t nnbr = 1 + (int64_t)m * (n - m) + binom(m, 2) * binom(n - m, 2);
-        int P = ((n * (n + 1) / 2 + 1 + 15) / 16) * 16;
-        // (off-diagonal lists, pair targets and merged-diagonal sums of the row kernels too)
-        const int64_t pairs = prec == KPM_FP64 || prec == KPM_FP32
-                                  ? 13 * nexc + 10 * n * (n - 1) / 2 + 8 * n +
-                                        (prec == KPM_FP32 ? 4 * (ns + 3) : 0)
-                                  : 0;
-        return (size_t)ns * (4 + 14 * nexc + 16 * nnbr + 12 * P + pairs);
-    };
-    v += tables(na, sa) + (na == nb ? 0 : tables(nb, sb));
-    v += (size_t)n * n * n * n * 12 + (64 << 20);
-    return v;
+// Device bytes a request keeps resident: its context, psi0 and 64 MB for what is not counted
+// singly (reduction scratch, moments, graphs, the allocator's granularity).
+size_t estimate_bytes(int n, int na, int nb, int ncol, kpm_precision prec, bool lean) {
+    return context_bytes(n, na, nb, ncol, prec, lean) + (size_t)binom(n, na) * binom(n, nb) * 8 +
+           (64 << 20);
 }
 
 }  // namespace
@@ -220,8 +200,8 @@ void kpm_server::complete(Slot& s, bool resident_slot) {
 void kpm_server::setup(Slot& s) {
     Req& r = *s.req;
     KPM_CUDA(cudaStreamCreateWithFlags(&s.st, cudaStreamNonBlocking));
-    kpm_status st = kpm_create(r.h1.data(), r.eri.data(), r.dip.data(), r.norb, r.na, r.nb,
-                               cfg.precision, s.st, &s.ctx);
+    kpm_status st = create_context(r.h1.data(), r.eri.data(), r.dip.data(), r.norb, r.na, r.nb,
+                                   cfg.precision, r.lean, s.st, &s.ctx);
     if (st != KPM_OK) KPM_THROW(st, "%s", kpm_last_error(nullptr));
     int64_t dim = kpm_dim(s.ctx);
     s.psi.alloc((size_t)dim * 8);
@@ -404,7 +384,11 @@ kpm_status kpm_server_submit(kpm_server* s, const kpm_request* q, uint64_t* id) 
     r->kernel = q->kernel;
     r->deflate = q->deflate != 0;
     r->e0 = q->e0;
-    r->mem = estimate_bytes(n, q->nalpha, q->nbeta, r->ncol, s->cfg.precision);
+    r->mem = estimate_bytes(n, q->nalpha, q->nbeta, r->ncol, s->cfg.precision, false);
+    if (r->mem > s->cfg.mem_budget_bytes) {
+        r->lean = true;
+        r->mem = estimate_bytes(n, q->nalpha, q->nbeta, r->ncol, s->cfg.precision, true);
+    }
     if (r->mem > s->cfg.mem_budget_bytes) {
         set_thread_error("request needs more device memory than the server budget");
         return KPM_ENOMEM;

@@ -950,6 +950,20 @@ void PairTables::build_spin(Spin& t, const SpinTables& T, const double* eri, Sig
     }
 }
 
+size_t PairTables::bytes(const SpinTables& A, const SpinTables& B, bool f64, bool dense) {
+    const SigmaPath path = sigma_path(A, B, f64);
+    if (path == SIGMA_GATHER || (path == SIGMA_SLOTS && !dense)) return 0;
+    const size_t NO = A.n * (A.n - 1) / 2;
+    // as build_spin allocates
+    auto spin = [&](const SpinTables& T) {
+        const size_t ns = T.ns, ne = ns * T.m * (T.n - T.m);
+        const size_t common = 8 * ne + 8 * NO * ns;
+        return path == SIGMA_ROWS ? common + 5 * ne + 8 * T.n * ns
+                                  : common + 2 * NO * ns + 4 * ns * ((ns + 3) / 4 * 4);
+    };
+    return NO * NO * (f64 ? 8 : 4) + spin(A) + (&A != &B ? spin(B) : 0);
+}
+
 void PairTables::build(const SpinTables& A, const SpinTables& B, const double* eri, bool f64_,
                        cudaStream_t st) {
     f64 = f64_;

@@ -1208,8 +1208,18 @@ void TcSigma::set_layout(int passes, cudaStream_t st) {
     smem_bytes = sm;
 }
 
+size_t TcSigma::bytes(const SpinTables& A, const SpinTables& B, bool fp16, int ncol) {
+    const size_t sa = A.ns, sb = B.ns, pa = half_pitch(A.ns), pb = half_pitch(B.ns);
+    const size_t xp = (sb + 127) / 128 * 128;                  // (also the slot table's pitch)
+    const size_t P = (A.n * (A.n + 1) / 2 + 1 + 15) / 16 * 16;
+    const size_t nc = std::min(ncol, batch_columns(A.ns * B.ns));
+    return 2 * P * xp + 6 * sa * A.m * (A.n - A.m) + 8 * sa * P +       // slots, entries, w_R
+           4 * sb * pb + (&A != &B ? 4 * sa * pa : 0) +                 // split F
+           nc * (sa * xp * (fp16 ? 4 : 8) + sb * pa * 4 + 12 * sa);     // split x and x^T
+}
+
 int TcSigma::hold(int ncol, cudaStream_t st) {
-    const int want = std::min(ncol, batch_columns(dim));
+    const int want = std::min({ncol, batch_columns(dim), most});
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     KPM_CUDA(cudaStreamIsCapturing(st, &cap));
     if (cap != cudaStreamCaptureStatusNone) captured = true;

@@ -56,6 +56,8 @@ struct TcSigma {
     void init(const SpinTables& ta, const SpinTables& tb, const double* d_h1,
               const double* d_eri, const float2* d_diag, int n, double wmax, double wcolsum,
               bool use_fp16, cudaStream_t st);
+    // Device bytes of the tables that init builds, and of the buffers for ncol columns.
+    static size_t bytes(const SpinTables& A, const SpinTables& B, bool fp16, int ncol);
     void apply(const float* x, float* y, int ncol, cudaStream_t st);
     // Operand buffers for blocks of ncol columns: room for as many of them as one set of
     // launches takes (batch_columns), or for as many as before (at least one) where the
@@ -65,6 +67,7 @@ struct TcSigma {
     // kept until the context goes.
     int hold(int ncol, cudaStream_t st);
     int held = 0;                 // columns the buffers have room for
+    int most = 64;                // never hold more (lean contexts: 1)
     bool captured = false;        // launches of apply have been captured
     std::deque<DevBuf> retired;   // outgrown buffers of captured launches
     // Scales of every row from rowmax and max|x| (am), for the next row pass, and the split

@@ -205,13 +205,22 @@ __global__ void k_pack_tables(const int32_t* __restrict__ tgtT, const uint16_t* 
     }
 }
 
-void build_spin_tables(SpinTables& t, int n, int m, const double* d_h1, const double* d_eri,
-                       cudaStream_t st) {
+void spin_shape(SpinTables& t, int n, int m) {
     t.n = n;
     t.m = m;
     t.ns = binom64(n, m);
     t.nexc = m * (n - m + 1);
     t.nnbr = (int)(1 + (int64_t)m * (n - m) + binom64(m, 2) * binom64(n - m, 2));
+}
+
+size_t spin_table_bytes(const SpinTables& t) {
+    return (size_t)t.ns * (4 + 14 * (size_t)t.nexc + 4 * (size_t)t.m * (t.n - t.m) +
+                           16 * (size_t)t.nnbr);
+}
+
+void build_spin_tables(SpinTables& t, int n, int m, const double* d_h1, const double* d_eri,
+                       cudaStream_t st) {
+    spin_shape(t, n, m);
     Binom B = make_binom();
     t.masks.alloc(t.ns * sizeof(uint32_t));
     size_t ne = (size_t)t.ns * t.nexc;
