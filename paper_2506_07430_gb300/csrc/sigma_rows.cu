@@ -421,6 +421,42 @@ __device__ __forceinline__ void fma2(uint64_t& acc, uint64_t a, uint64_t b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
+// One determinant in the order of the gather kernel, which touches its neighbours alone.
+// The tiled products also multiply by the zeros of the dense F and of padded tables, and an
+// infinity or NaN times zero would spread along whole rows and columns: k_opp_slots takes
+// every element that came out not finite from here.
+__device__ __noinline__ float gather_one(const BatchMol& m, const float* x, int64_t ia,
+                                         int64_t ib) {
+    const int64_t nsa = m.nsa, nsb = m.nsb;
+    const float* fvA = static_cast<const float*>(m.fvalA);
+    const float* fvB = static_cast<const float*>(m.fvalB);
+    const float* V = static_cast<const float*>(m.V);
+    const int n = m.n, n2 = n * n;
+    float acc = 0.f;
+    for (int t = 1; t < m.nnbrB; ++t)
+        acc += fvB[(int64_t)t * nsb + ib] * x[ia * nsb + m.fcolB[(int64_t)t * nsb + ib]];
+    for (int t = 1; t < m.nnbrA; ++t)
+        acc += fvA[(int64_t)t * nsa + ia] * x[(int64_t)m.fcolA[(int64_t)t * nsa + ia] * nsb + ib];
+    for (int f = 0; f < m.nexcB; ++f) {
+        const int64_t jb = m.tgtBT[(int64_t)f * nsb + ib];
+        const int pb = m.pqBT[(int64_t)f * nsb + ib];
+        float inner = 0.f;
+        // off-diagonal alpha entries first; diagonal by diagonal is in the exact diagonal
+        for (int pass = 0; pass < (pb % (n + 1) == 0 ? 1 : 2); ++pass)
+            for (int e = 0; e < m.nexcA; ++e) {
+                const int64_t k = ia * m.nexcA + e;
+                const int g = m.pqA[k];
+                if ((g % (n + 1) == 0) != (pass == 1)) continue;
+                inner += float(m.sgnA[k]) * V[(int64_t)g * n2 + pb] *
+                         x[(int64_t)m.tgtA[k] * nsb + jb];
+            }
+        acc += float(m.sgnBT[(int64_t)f * nsb + ib]) * inner;
+    }
+    const float2 d = m.diag[ia * nsb + ib];
+    const float xv = x[ia * nsb + ib];
+    return acc + fmaf(d.x, xv, d.y * xv);
+}
+
 // Opposite-spin part and diagonal of one row, FP32, added into y.  At FP32 rate one
 // shared-memory load per FMA (k_sigma_rows) would bound the row at a quarter of the
 // FMA rate or less, so here D is a register-tiled product over all pairs s, whether
@@ -556,6 +592,7 @@ k_opp_slots(const __grid_constant__ BatchMol m) {
                 const float2 d = m.diag[(int64_t)myrow + j];
                 const float xv = __ldg(x + myrow + j);
                 acc = fmaf(d.x, xv, fmaf(d.y, xv, acc));
+                if (!isfinite(acc)) acc = gather_one(m, x, ia, j);
             }
             y[myrow + j] = acc;
         }
