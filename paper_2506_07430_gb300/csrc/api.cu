@@ -1,5 +1,8 @@
 // extern "C" entry points of include/kpm.h: context set-up, sigma/dipole
 // dispatch, the KPM recursion loop, Lanczos bounds and the spectrum.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -1114,30 +1117,58 @@ kpm_status kpm_moments_host(kpm_ctx* ctx, const double* psi0_host, unsigned comp
 }
 
 // Device buffer of a thread's reconstructions, kept between calls up to 4 MiB (allocating
-// and freeing four buffers took 130 us of every call) and freed with the thread.  A
-// pointer that the device no longer knows (another device, a reset) is dropped.
+// and freeing four buffers took 130 us of every call) and freed with the thread.  The driver
+// numbers every allocation of a process anew, so a kept pointer whose number has changed
+// (the device was reset, the address may be another allocation's) is dropped, not used or
+// freed.
 struct SpectrumSpace {
     static constexpr size_t KEEP = (size_t)4 << 20;
     DevBuf buf;
     int device = -1;
+    unsigned long long id = 0;
+    // the number of the allocation at p, 0 if there is none
+    static unsigned long long number(const void* p) {
+        static const auto fn = [] {
+            void* f = nullptr;
+            cudaDriverEntryPointQueryResult q;
+            if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000,
+                                                 cudaEnableDefault, &q) != cudaSuccess ||
+                q != cudaDriverEntryPointSuccess) {
+                cudaGetLastError();
+                f = nullptr;
+            }
+            return reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(f);
+        }();
+        unsigned long long v = 0;
+        if (!fn || !p || fn(&v, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)p) != CUDA_SUCCESS)
+            return 0;
+        return v;
+    }
+    void settle(bool keep) {
+        if (!buf.p) return;
+        if (id == 0 || number(buf.p) != id) {
+            buf.p = nullptr;
+            buf.bytes = 0;
+        } else if (!keep) {
+            buf.release();
+        }
+    }
     double* get(size_t bytes) {
         int dev = 0;
         KPM_CUDA(cudaGetDevice(&dev));
-        cudaPointerAttributes at{};
-        if (buf.p && (dev != device || cudaPointerGetAttributes(&at, buf.p) != cudaSuccess ||
-                      at.type != cudaMemoryTypeDevice)) {
-            cudaGetLastError();
-            if (at.type == cudaMemoryTypeDevice || dev != device) buf.release();
-            buf.p = nullptr;
-            buf.bytes = 0;
-        }
+        settle(dev == device);
         device = dev;
-        buf.ensure(bytes);
+        if (bytes > buf.bytes) {
+            buf.alloc(bytes);
+            id = number(buf.p);
+        }
         return buf.as<double>();
     }
+    // (a buffer without a number goes at once)
     void put() {
-        if (buf.bytes > KEEP) buf.release();
+        if (buf.bytes > KEEP || id == 0) buf.release();
     }
+    ~SpectrumSpace() { settle(false); }
 };
 
 // Reconstruction between host arrays: one device buffer [moments | damped | omega |
