@@ -24,11 +24,11 @@
 // diagonals and the opposite-spin Coulomb sums, evaluated in FP64 and stored as
 // float hi + lo per determinant) times x, hi and lo multiplied separately.
 //
-// Kernel: CTA tile 128 x 256 (or narrower, see tile_columns), k-block 32 (64 bytes per
-// row: one SWIZZLE_64B atom row), TMA pipeline of four stages (narrower tiles six or
-// eight; full/empty mbarriers), one warp issues TMA,
-// one issues MMAs, eight warps drain accumulator chunks (see k_gemm) and run the
-// epilogue.  All waits are bounded.
+// Kernel: pairs of CTAs on tiles of 256 x 256 (or narrower, see tile_columns), each CTA
+// 128 of the rows, k-block 32 (64 bytes per row: one SWIZZLE_64B atom row), TMA pipeline of
+// six stages (eight for narrower tiles; full/empty mbarriers), one warp issues TMA,
+// one issues MMAs for the pair, eight warps drain accumulator chunks (see k_gemm) and run
+// the epilogue.  All waits are bounded.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -46,13 +46,11 @@
 namespace kpm {
 namespace {
 
-// k-block 32 (64-byte rows, SWIZZLE_64B) four stages deep, or 64 (128-byte rows,
-// SWIZZLE_128B) two stages deep: the same 192 KB of shared memory.  Four stages
-// keep three k-blocks of loads in flight (about 2300 cycles of MMA to hide the
-// L2 latency, against 1500 with two stages of 64).  Measured at 16 orbitals,
-// both products: 18.0 ms (32, accumulation chunks of two k-blocks), 19.8 ms
-// (64), 22.0 ms (32 with one-k-block chunks: the epilogue then drains a chunk
-// every 800 cycles of MMA).
+// k-block 32 (64-byte rows, SWIZZLE_64B) six stages deep, or 64 (128-byte rows,
+// SWIZZLE_128B) three stages deep: the same 192 KB of shared memory.  Chunks of 64 of K
+// either way (one-k-block chunks of 32 make the epilogue drain one every 800 cycles of MMA:
+// 22.0 ms for both products at 16 orbitals where two-k-block chunks took 18.0, on the kernels
+// with a tile per CTA).
 #ifndef GM_BK_N
 #define GM_BK_N 32
 #endif
@@ -66,8 +64,8 @@ constexpr int GM_EPI_WARPS = 8;
 template <int BN>
 struct Tile {
     static constexpr int EPI_COLS = BN / 2;
-    static constexpr int STAGES = (BN == 256 ? 4 : BN == 128 ? 6 : 8) * 32 / GM_BK;
-    static constexpr uint32_t B_BYTES = BN * GM_BK * 2;   // per piece
+    static constexpr int STAGES = (BN == 256 ? 6 : 8) * 32 / GM_BK;
+    static constexpr uint32_t B_BYTES = BN / 2 * GM_BK * 2;   // per piece, a CTA's half
     static_assert(GM_LIST_N % BN == 0 && EPI_COLS % 32 == 0, "tile geometry");
 };
 constexpr int GM_TMA_WARP = GM_EPI_WARPS;       // producer (one thread)
@@ -82,19 +80,20 @@ constexpr int GM_THREADS = 32 * (GM_EPI_WARPS + 2);
 // the chunks into FP32 running sums in registers (round to nearest) keeps it to
 // a few units of 2^-24.
 constexpr int GM_CK = 64 / GM_BK;               // k-blocks per accumulation chunk
-// poll interval of the epilogue warps' waits (a chunk accumulates for microseconds)
+// poll interval of the epilogue warps' waits (14 orbitals, three columns: 4.696 ms with 256,
+// 4.690 with 32, 4.693 with none)
 #ifndef GM_BACKOFF_NS
-#define GM_BACKOFF_NS 256
+#define GM_BACKOFF_NS 32
 #endif
 constexpr uint32_t A_BYTES = GM_BM * GM_BK * 2;  // per piece
-// Consecutive CTAs take vertically adjacent tiles in pairs that share a list of k-blocks
-// and read the same B tile at about the same time (from L2)
+// Pairs of CTAs (clusters of two) on vertically adjacent tiles
 constexpr int GM_PAIR = 2;
 template <int BN>
 constexpr uint32_t stage_bytes() { return 2 * A_BYTES + 2 * Tile<BN>::B_BYTES; }
 template <int BN>
 constexpr size_t gemm_smem() { return Tile<BN>::STAGES * stage_bytes<BN>() + 1024 + 256; }
 constexpr long long GM_WAIT = 4000000000LL;
+constexpr long long GM_DRAIN = 20000000LL;   // after an abort, per stage: ~10 ms
 
 __device__ __forceinline__ uint32_t su32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -114,23 +113,51 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
         : "=r"(ok) : "r"(su32(b)), "r"(parity) : "memory");
     return ok != 0;
 }
+// the same for a phase that threads of the other CTA arrive on (mbar_arrive_cluster)
+__device__ __forceinline__ bool mbar_test_cluster(uint64_t* b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(su32(b)), "r"(parity) : "memory");
+    return ok != 0;
+}
 // bounded wait; returns false (and flags the error) if it ran out
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* b, uint32_t parity, int* err) {
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* b, uint32_t parity, int* err,
+                                                  long long limit) {
     long long t0 = clock64();
     while (!mbar_test(b, parity)) {
-        if (clock64() - t0 > GM_WAIT) {
+        if (clock64() - t0 > limit) {
             atomicExch(err, 1);
             return false;
         }
     }
     return true;
 }
+// into this CTA's shared memory; the bytes are counted on `bar`, a shared::cluster address
+// in either CTA of the pair
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            uint64_t* bar) {
+                                            uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(su32(bar))
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
         : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// shared::cluster address of the same variable in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// all threads of both CTAs of the cluster
+__device__ __forceinline__ void cluster_sync_() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -145,12 +172,16 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
                                        uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
 }
-__device__ __forceinline__ void mma_commit_(uint64_t* b) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(su32(b)) : "memory");
+// arrive, once the MMAs issued so far have completed, on the mbarrier at this offset in both
+// CTAs of the pair
+__device__ __forceinline__ void mma_commit_pair(uint64_t* b) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+        " [%0], %1;"
+        ::"r"(su32(b)), "h"((uint16_t)0x3) : "memory");
 }
 __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -182,8 +213,8 @@ __device__ __forceinline__ uint64_t sw_desc(uint32_t saddr) {
 
 template <int BN>
 __host__ __device__ constexpr uint32_t gemm_idesc() {
-    // D F32, A/B F16, K-major, N = BN, M = 128
-    return (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(GM_BM >> 4) << 24);
+    // D F32, A/B F16, K-major, N = BN, M = 256 over the pair
+    return (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(GM_PAIR * GM_BM >> 4) << 24);
 }
 
 struct GemmArgs {
@@ -220,10 +251,11 @@ struct GemmMaps {
 // bounded wait that also gives up when another role has aborted; roles off the
 // critical path sleep backoff_ns between polls so that they leave the issue
 // slots to the MMA and TMA threads
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool wait_or_abort(uint64_t* b, uint32_t parity, volatile int* abort_flag,
                                               int* err, unsigned backoff_ns = 0) {
     long long t0 = clock64();
-    while (!mbar_test(b, parity)) {
+    while (!(CLUSTER ? mbar_test_cluster(b, parity) : mbar_test(b, parity))) {
         if (backoff_ns) __nanosleep(backoff_ns);
         if (*abort_flag) return false;
         if (clock64() - t0 > GM_WAIT) {
@@ -234,12 +266,28 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* b, uint32_t parity, vola
     }
     return true;
 }
-__device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
+// On a shared::cluster address.  Relaxed: what it orders are reads of tensor memory, by the
+// tcgen05 fences on either side; no other memory is handed over.  (With release and acquire
+// at cluster scope a chunk's turn took 5,300 cycles: sigma at 16 orbitals 39.1 ms, 32.1 so.)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t b) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(b) : "memory");
 }
 
-// Pairs: CTAs 2 p and 2 p + 1 compute row tiles 2 p and 2 p + 1 of the same column tile.
-// Each loads its own A and the whole B tile by plain TMA and waits for no other CTA.
+// Pairs: CTAs 2 p and 2 p + 1 (a cluster) compute row tiles 2 p and 2 p + 1 of the same
+// column tile with MMAs over both SMs (cta_group::2, M = 256): each CTA loads its own 128 rows
+// of A and half of the rows of B by plain TMA into its own shared memory, and the tensor
+// cores of both read both halves of B.  The even CTA's MMA thread issues for the pair: both
+// CTAs' loads count their bytes on its "full" barriers, its commits arrive on the "empty" and
+// "accumulated" barriers of both, and the epilogue warps of both arrive on its "drained"
+// ones.  Each CTA keeps its own rows of the accumulator in its tensor memory.  The pair
+// syncs once its barriers are initialised and again before it gives up the tensor memory,
+// so nothing is in flight towards a CTA that has ended.
+// Why pairs: an MMA of one CTA alone (128 x 256 x 16, 128 cycles) reads 12 KB of shared
+// memory, and its k-block's loads write 48 KB per 768 cycles: 160 bytes a cycle, more than
+// the 128 there are.  With half of B in each SM it is 64 + 43.  sigma with a tile per CTA and
+// with pairs, same bits: 16 orbitals 36.5 and 32.2 ms, 14 (three columns) 4.95 and 4.69,
+// (13o, 7 + 6, BF16) 422 and 405 us; where the grid is one wave the pair's syncs cost what it
+// gains (10 orbitals, three columns, 53.8 and 54.3 us).
 //
 // Accumulation in chunks: the MMA thread restarts the accumulator every ck
 // k-blocks, alternating two tensor-memory accumulators of BN columns; the
@@ -249,7 +297,7 @@ __device__ __forceinline__ void mbar_arrive_(uint64_t* b) {
 // growing like sqrt(K); in chunks, each accumulator sums a short run and the
 // running sum takes one rounding per chunk.
 template <int BN>
-__global__ void __launch_bounds__(GM_THREADS, 1)
+__global__ void __cluster_dims__(GM_PAIR, 1, 1) __launch_bounds__(GM_THREADS, 1)
 k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     constexpr int STAGES = Tile<BN>::STAGES, EPI_COLS = Tile<BN>::EPI_COLS;
     constexpr uint32_t B_BYTES = Tile<BN>::B_BYTES;
@@ -264,10 +312,10 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     uint64_t* acce = accf + 2;            // [2] accumulator drained (epilogue warps)
     uint32_t* holder = reinterpret_cast<uint32_t*>(acce + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(holder + 1);
-    int* issued = const_cast<int*>(abort_flag) + 1;   // stages whose TMA loads were issued
-    int* consumed = issued + 1;                       // stages the MMA thread passed
+    int* consumed = const_cast<int*>(abort_flag) + 1;   // stages the MMA thread passed
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t crank = cluster_rank();   // blockIdx.x % GM_PAIR; 0: issues the MMAs
     // grouped rasterisation over pairs of row tiles: groups of GROUP_M pairs walk
     // all column tiles, so the group's A panels and the current B panels stay in L2
     const int GROUP_M = g.group_m;
@@ -284,7 +332,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     const int first_m = (b / gsize) * GROUP_M;
     const int gm = min(nMP - first_m, GROUP_M);
     const int mp = first_m + (b % gsize) % gm;
-    const int m0 = (mp * GM_PAIR + (int)(blockIdx.x % GM_PAIR)) * GM_BM;
+    // (with an odd number of row tiles the last pair's second tile lies past M:
+    // its A loads read the zero fill and its epilogue writes nothing)
+    const int m0 = (mp * GM_PAIR + (int)crank) * GM_BM;
     const int n0 = ((b % gsize) / gm) * BN;
     // k-blocks the pair visits: those of F_b where the pair's 256 rows have a nonzero, then
     // those of F_a where the 256-row list tile of F_a around the B tile has one;
@@ -303,10 +353,9 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init_(&accf[i], 1);
-            mbar_init_(&acce[i], GM_EPI_WARPS);
+            mbar_init_(&acce[i], GM_PAIR * GM_EPI_WARPS);
         }
         *abort_flag = 0;
-        *issued = 0;
         *consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         for (int i = 0; i < 2; ++i) {
@@ -318,15 +367,13 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     }
     // (before the allocation: a waiting CTA holds no tensor memory)
     grid_wait();
-    // (with an odd number of row tiles the last pair's second tile lies past M)
-    if (m0 >= g.M) return;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;"
                      ::"r"(su32(holder)) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_before();
-    __syncthreads();
+    cluster_sync_();   // both CTAs' barriers initialised, both halves of the tensor memory held
     tc_after();
     const uint32_t tmem = *holder;
 
@@ -339,27 +386,32 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                     !wait_or_abort(&empty[s], ((kb / STAGES) - 1) & 1, abort_flag, g.err))
                     break;
                 unsigned char* st = smem + s * STAGE_BYTES;
-                mbar_expect_tx(&full[s], STAGE_BYTES);
+                // the pair's bytes, counted in the even CTA (the odd one's may land first)
+                if (crank == 0) mbar_expect_tx(&full[s], GM_PAIR * STAGE_BYTES);
+                const uint32_t bar = mapa(su32(&full[s]), 0);
                 const bool beta = kb < nk1;
                 const int kx = (beta ? kl1[kb] : kl2[kb - nk1]) * GM_BK;
                 const CUtensorMap* mA = beta ? maps.fb : maps.t;
                 const CUtensorMap* mB = beta ? maps.x : maps.fa;
                 const int ma = beta ? m0 : trow_ + m0;
-                tma_load_2d(su32(st), mA, kx, ma, &full[s]);
-                tma_load_2d(su32(st + A_BYTES), mA + 1, kx, ma, &full[s]);
-                const int nb = (beta ? xrow : 0) + n0;
-                tma_load_2d(su32(st + 2 * A_BYTES), mB, kx, nb, &full[s]);
-                tma_load_2d(su32(st + 2 * A_BYTES + B_BYTES), mB + 1, kx, nb, &full[s]);
-                *(volatile int*)issued = kb + 1;
+                tma_load_2d(su32(st), mA, kx, ma, bar);
+                tma_load_2d(su32(st + A_BYTES), mA + 1, kx, ma, bar);
+                // this CTA's half of the B rows
+                const int nh = (beta ? xrow : 0) + n0 + (int)crank * (BN / GM_PAIR);
+                tma_load_2d(su32(st + 2 * A_BYTES), mB, kx, nh, bar);
+                tma_load_2d(su32(st + 2 * A_BYTES + B_BYTES), mB + 1, kx, nh, bar);
             }
+            // (the last stages' commits have arrived before this CTA may end)
+            for (int kb = max(0, nk - STAGES); kb < nk; ++kb)
+                if (!wait_or_abort(&empty[kb % STAGES], (kb / STAGES) & 1, abort_flag, g.err)) break;
         }
     } else if (warp == GM_MMA_WARP) {
-        if (lane == 0) {
-            // MMA issuer: chunk c accumulates its k-blocks (at most ck) into buffer c & 1
+        if (lane == 0 && crank == 0) {
+            // MMA issuer of the pair: chunk c accumulates its k-blocks (at most ck) into buffer c & 1
             constexpr uint32_t idesc = gemm_idesc<BN>();
             for (int c = 0; c < nchunk; ++c) {
                 const uint32_t d = tmem + (uint32_t)((c & 1) * BN);
-                if (c >= 2 && !wait_or_abort(&acce[c & 1], ((c >> 1) - 1) & 1, abort_flag, g.err))
+                if (c >= 2 && !wait_or_abort<true>(&acce[c & 1], ((c >> 1) - 1) & 1, abort_flag, g.err))
                     break;
                 tc_after();
                 const bool beta = c < nchunk1;
@@ -391,10 +443,10 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
                         const uint32_t off = j * 32;
                         mma_ss(d, sw_desc(a0 + off), sw_desc(b0 + off), idesc, 1);
                     }
-                    mma_commit_(&empty[s]);   // stage s released
+                    mma_commit_pair(&empty[s]);   // stage s released in both CTAs
                 }
                 if (!ok) break;
-                mma_commit_(&accf[c & 1]);
+                mma_commit_pair(&accf[c & 1]);
             }
         }
     } else {
@@ -428,7 +480,7 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
             }
             tc_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_(&acce[c & 1]);
+            if (lane == 0) mbar_arrive_cluster(mapa(su32(&acce[c & 1]), 0));
         }
         if (ok && !*abort_flag) {
             float scale = (nchunk == nchunk1 ? g.to_w_b : 1.f) * g.inv_w;
@@ -485,14 +537,15 @@ k_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
     }
     tc_before();
     __syncthreads();
-    if (tid == 0 && *abort_flag) {
-        // after an abort, wait (bounded) for TMA copies that were issued but not consumed
-        for (int kb = *consumed; kb < *issued; ++kb)
-            mbar_wait_bounded(&full[kb % STAGES], (kb / STAGES) & 1, g.err);
+    if (tid == 0 && crank == 0 && *abort_flag) {
+        // after an abort, wait (bounded) for the pair's copies that may still be in flight: the
+        // other CTA has long issued those of the stages that were free
+        for (int kb = *consumed; kb < min(nk, *consumed + STAGES); ++kb)
+            mbar_wait_bounded(&full[kb % STAGES], (kb / STAGES) & 1, g.err, GM_DRAIN);
     }
-    __syncthreads();
+    cluster_sync_();   // the other CTA's waits are over too, and its arrivals here done
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem)
                      : "memory");
 }
 
@@ -712,10 +765,10 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
 // epilogue, both by its width, so below one wave narrower tiles give the same work to more
 // SMs (and a shorter epilogue).  Beyond one wave 256 is best: every CTA reads its A tile
 // whole, 24 KB a k-block at 128 columns for half the MMAs of the 32 KB at 256.  Measured,
-// whole sigma with 256 / 128 / 64 columns: 10 orbitals 67.1 / 59.0 / 54.7 us (three
-// columns of x 80.2 / 71.7 / 67.7), 12 orbitals 184.6 / 175.8 / 171.8 (three, where 64
-// takes 2.4 waves: 372 / 401 / 425), (13o, 5 + 5) 283 / 271 / 310 (64: 1.7 waves),
-// (13o, 7 + 6) 422 / 473 / 516.  Every width adds the same chunks in the same order, so
+// whole sigma with 256 / 128 / 64 columns: 10 orbitals 51.9 / 44.0 / 40.1 us (three
+// columns of x 65.4 / 58.1 / 53.9), 12 orbitals 167 / 158 / 153 (three, where 64
+// takes 2.4 waves: 349 / 378 / 401), (13o, 5 + 5) 263 / 252 / 290 (64: 1.7 waves),
+// (13o, 7 + 6) 403 / 449 / 493.  Every width adds the same chunks in the same order, so
 // the results are the same bits.
 int DenseSS::tile_columns(int nc) const {
     for (int bn : {64, 128})
@@ -732,12 +785,12 @@ void DenseSS::launch(const float* x, float* y, const float* amax, int nc, int gr
     GemmMaps maps;
     maps.fb[0] = make_map(fb_hi.as<__half>(), nb, nb, pb, GM_BM);
     maps.fb[1] = make_map(fb_lo.as<__half>(), nb, nb, pb, GM_BM);
-    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, bn);
-    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, bn);
+    maps.x[0] = make_map(xh.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
+    maps.x[1] = make_map(xl.as<__half>(), nc * na, nb, xpitch, bn / GM_PAIR);
     maps.t[0] = make_map(th.as<__half>(), nc * nb, na, pa, GM_BM);
     maps.t[1] = make_map(tl.as<__half>(), nc * nb, na, pa, GM_BM);
-    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn);
-    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn);
+    maps.fa[0] = make_map(fa_hi->as<__half>(), na, na, pa, bn / GM_PAIR);
+    maps.fa[1] = make_map(fa_lo->as<__half>(), na, na, pa, bn / GM_PAIR);
     const double w = std::min(wscale_a, wscale_b);
     GemmArgs g{(int)nb, (int)na, nc, y, nb, amax, (float)(w / wscale_b), (float)(w / wscale_a),
                (float)(1.0 / w), diag, diag ? diag_full : nullptr, err, group, kbs_b.as<int>(), kbl_b.as<int>(),
