@@ -258,7 +258,7 @@ kpm_status kpm_moments_deflated(kpm_ctx* ctx, const double* psi0_dev, double e0,
  * molecules do not pay one set of launches each.  Per molecule the arithmetic
  * and reduction order are those of kpm_moments: the moments are identical.
  *   ctxs       [count] distinct contexts, all KPM_FP64 or all KPM_FP32 (the
- *              CUDA-core gather path), on one device.
+ *              CUDA-core paths), on one device.
  *   psi0_dev   [count] FP64 device ground states, psi0_dev[i] of ctxs[i]'s dim.
  *   a, b       [count] host rescaling of each molecule (as kpm_moments).
  *   moments_host  host [count][popcount(comp_mask)][nmoments].

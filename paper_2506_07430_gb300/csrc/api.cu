@@ -420,14 +420,14 @@ void rec_advance(kpm_ctx* c, int nsteps) {
 }
 
 // Batched steps (kpm_moments_batch, kpm_recursion_advance_batch): contexts of
-// one batch are distinct, on one device, all on the gather path (FP64 or FP32).
+// one batch are distinct, on one device, all in FP64 or all in FP32.
 void check_batch(kpm_ctx* const* ctxs, int count) {
     const kpm_ctx* c0 = ctxs[0];
     for (int i = 0; i < count; ++i) {
         const kpm_ctx* c = ctxs[i];
         if (!c) KPM_THROW(KPM_EINVAL, "context %d is NULL", i);
         if (c->prec != KPM_FP64 && c->prec != KPM_FP32)
-            KPM_THROW(KPM_EINVAL, "batched steps run the gather path: FP64 or FP32 contexts "
+            KPM_THROW(KPM_EINVAL, "batched steps run the CUDA-core paths: FP64 or FP32 contexts "
                                   "only (context %d)", i);
         if (c->prec != c0->prec) KPM_THROW(KPM_EINVAL, "contexts of a batch share one precision");
         if (c->device != c0->device) KPM_THROW(KPM_EINVAL, "contexts of a batch share one device");
@@ -1116,8 +1116,9 @@ kpm_status kpm_moments_host(kpm_ctx* ctx, const double* psi0_host, unsigned comp
     return kpm_moments(ctx, ctx->psi_tmp.as<double>(), comp_mask, a, b, nmoments, moments_host);
 }
 
-// Device buffer of a thread's reconstructions, kept between calls up to 4 MiB (allocating
-// and freeing four buffers took 130 us of every call) and freed with the thread.  The driver
+// Device buffer of a thread's reconstructions, kept between calls up to 4 MiB (with four
+// buffers allocated and freed by each call the smallest took 153 us, 35 so) and freed with the
+// thread.  The driver
 // numbers every allocation of a process anew, so a kept pointer whose number has changed
 // (the device was reset, the address may be another allocation's) is dropped, not used or
 // freed.

@@ -170,6 +170,7 @@ struct PairTables {
     };
     SigmaPath path = SIGMA_GATHER;
     bool f64 = false;
+    int nsm = 0;        // SMs of the device
     DevBuf woo;         // T [NO][NO] (pq|rs)
     Spin a, b_own;
     Spin* b = nullptr;
@@ -234,7 +235,7 @@ void launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaSt
 // its sigma and update work and its first block in each flattened grid.  All
 // molecules of a batch share the path (FP64, or FP32 with the exact diagonal).
 struct BatchMol {
-    // sigma: y = H x (gather path), x and y [ncol][nsa * nsb]
+    // sigma: y = H x, x and y [ncol][nsa * nsb]
     const void* x;
     void* y;
     int64_t nsa, nsb;
@@ -269,6 +270,7 @@ struct BatchMol {
     int NO, K;          // pairs n (n - 1) / 2; terms of D: noffA + 1 (FP32: + 2), or 0
                         // without electrons
     int fc, ft, parts, stage_x, threads, ts;   // geometry (rows_geometry, opp_choose)
+    int nsm;            // SMs of the device
     int64_t ldA, ldB;
     size_t smem;
     const int32_t* otgtA;

@@ -593,15 +593,6 @@ __global__ void k_mark_blocks(const int32_t* __restrict__ fcol, int64_t ns, int 
     mark[(r / rows) * nkb + c / GM_BK] = 1;
 }
 
-// diag[r] = F[r][r] (entry t = 0), as float hi + lo.
-__global__ void k_diag_pair(const double* __restrict__ fval, int64_t ns, float2* __restrict__ d) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= ns) return;
-    const double v = fval[r];
-    const float h = (float)v;
-    d[r] = make_float2(h, (float)(v - (double)h));
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     static std::once_flag once;
@@ -669,8 +660,8 @@ static double offdiag_scale(const SpinTables& T, DevBuf& scratch, cudaStream_t s
     return std::ldexp(1.0, 14 - std::max(e, -286));
 }
 
-static void build_f(const SpinTables& T, double ws, DevBuf& hi, DevBuf& lo, DevBuf& dg,
-                    int64_t pitch, cudaStream_t st) {
+static void build_f(const SpinTables& T, double ws, DevBuf& hi, DevBuf& lo, int64_t pitch,
+                    cudaStream_t st) {
     const int64_t n = T.ns * pitch;
     hi.alloc(n * 2);
     lo.alloc(n * 2);
@@ -685,10 +676,6 @@ static void build_f(const SpinTables& T, double ws, DevBuf& hi, DevBuf& lo, DevB
             lo.as<__half>(), pitch);
         KPM_LAUNCHED();
     }
-    dg.alloc(T.ns * sizeof(float2));
-    k_diag_pair<<<(unsigned)((T.ns + 255) / 256), 256, 0, st>>>(T.fval64.as<double>(), T.ns,
-                                                                 dg.as<float2>());
-    KPM_LAUNCHED();
 }
 
 // Lists, per tile of `rows` rows of the split matrix of T, the k-blocks holding a
@@ -742,18 +729,16 @@ void DenseSS::init(const SpinTables& A, const SpinTables& B, bool same, int* err
     KPM_CUDA(cudaFuncSetAttribute(k_gemm<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)gemm_smem<64>()));
     wscale_b = offdiag_scale(B, fmax, st);
-    build_f(B, wscale_b, fb_hi, fb_lo, db, pb, st);
+    build_f(B, wscale_b, fb_hi, fb_lo, pb, st);
     if (same) {
         wscale_a = wscale_b;
         fa_hi = &fb_hi;
         fa_lo = &fb_lo;
-        da = &db;
     } else {
         wscale_a = offdiag_scale(A, fmax, st);
-        build_f(A, wscale_a, fa_hi_own, fa_lo_own, da_own, pa, st);
+        build_f(A, wscale_a, fa_hi_own, fa_lo_own, pa, st);
         fa_hi = &fa_hi_own;
         fa_lo = &fa_lo_own;
-        da = &da_own;
     }
     // beta: F_b is the A operand (pairs of GM_BM-row tiles); alpha: F_a is the B
     // operand (lists by GM_LIST_N rows)

@@ -17,11 +17,10 @@ inline int batch_columns(int64_t dim) { return dim <= ((int64_t)1 << 24) ? 3 : 1
 struct DenseSS {
     int64_t na = 0, nb = 0, pa = 0, pb = 0;   // strings and FP16 row pitches per spin
     double wscale_a = 1.0, wscale_b = 1.0;    // power-of-two scales of the split matrices
-    DevBuf fa_hi_own, fa_lo_own, da_own;      // alpha matrices (own copy if N_a != N_b)
-    DevBuf fb_hi, fb_lo, db;                  // beta matrices, diagonal of F_b (float hi/lo)
+    DevBuf fa_hi_own, fa_lo_own;              // alpha matrices (own copy if N_a != N_b)
+    DevBuf fb_hi, fb_lo;                      // beta matrices
     DevBuf* fa_hi = nullptr;
     DevBuf* fa_lo = nullptr;
-    DevBuf* da = nullptr;
     int64_t xpitch = 0;                       // row pitch of xh/xl: N_b rounded up to 128
     DevBuf xh, xl, th, tl;                    // split copies of x and x^T (TcSigma::hold)
     DevBuf fmax;                              // scratch for max |F_off|

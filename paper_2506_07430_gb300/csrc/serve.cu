@@ -16,8 +16,8 @@
 // status at once and its slot and budget are released; the others go on.
 //
 // Every request's arithmetic is what it would be alone: its own context, the
-// same kernels, launch shapes and reduction grids (on the FP64 / FP32 gather
-// path, requests that advance by the same number of steps in a round share
+// same kernels, launch shapes and reduction grids (on the FP64 / FP32 CUDA-core
+// paths, requests that advance by the same number of steps in a round share
 // batched launches whose per-request work is that of the single launches), so
 // its result does not depend on what else is resident.  All waits are bounded (kpm_server_wait's timeout; the worker's
 // condition-variable waits).
@@ -264,7 +264,7 @@ void kpm_server::run() {
                 continue;
             }
         }
-        // On the gather path (FP64, FP32) the requests that advance by the same
+        // On the CUDA-core paths (FP64, FP32) the requests that advance by the same
         // number of steps share one sigma and one update launch per step
         // (kpm_recursion_advance_batch); each result is identical either way.
         // A failed advance (or an injected failure) finishes that request with

@@ -21,8 +21,8 @@
 // thread computes D only for its string's own entries, so no term is wasted.  At
 // FP64 this is what matters: the FP64 pipe takes two FMA per clock and SM (a 64th of the
 // FP32 rate), everything else hides behind it.  One column at 12 orbitals: 9.50 ms with a
-// thread per determinant (three FP64 operations per pair of table entries), 3.39 ms here,
-// 2.7 ms at the FP64 rate.
+// thread per determinant (three FP64 operations per pair of table entries), 3.39 ms here
+// (1.5 of the two FMA), 2.6 ms at the FP64 rate.
 // k_opp_slots / k_same_dense (larger FP32 molecules): see there.  Three columns at 12
 // orbitals: 4.33 ms with a thread per determinant (two gathers per FMA), 0.88 ms here.
 #include "common.cuh"
@@ -830,11 +830,11 @@ void launch_same(const BatchMol& m, cudaStream_t st) {
         launch_same_v<BM, BN, false>(m, st);
 }
 
-// The tile whose last wave over the 152 SMs wastes the least, in 64 x 64 units
+// The tile whose last wave over the SMs wastes the least, in 64 x 64 units
 void same_spin(const BatchMol& m, cudaStream_t st) {
     auto cost = [&](int bm, int bn) {
         const int64_t t = (m.nsa + bm - 1) / bm * ((m.nsb + bn - 1) / bn) * m.ncol;
-        return (t + 151) / 152 * (bm / 64) * (bn / 64);
+        return (t + m.nsm - 1) / m.nsm * (bm / 64) * (bn / 64);
     };
     const int64_t c44 = cost(128, 128), c24 = cost(64, 128), c22 = cost(64, 64);
     if (c44 <= c24 && c44 <= c22) launch_same<128, 128>(m, st);
@@ -881,9 +881,12 @@ void opp_slots(const BatchMol& m, cudaStream_t st) {
 SigmaPath sigma_path(const SpinTables& A, const SpinTables& B, bool f64) {
     // 16-bit targets, 32-bit element offsets
     if (A.ns * B.ns >= ((int64_t)1 << 31) || B.ns > 32767 || A.ns > 65535) return SIGMA_GATHER;
-    // A CTA per row: below 100 rows of more than two gather tiles each the gather
-    // kernel's CTA per 128 columns fills more of the chip (its three times as many FP64
-    // operations on ceil(nsb / 128) times as many SMs)
+    // A CTA per row: few rows of more than two gather tiles each leave most SMs idle, which
+    // the gather kernel's CTA per 128 columns fills.  Gather and row kernels, one column: 16
+    // rows of 12870 strings FP64 1.72 and 18.9 ms, FP32 0.40 and 1.47; 12 of 924 FP64 0.107
+    // and 0.197, FP32 0.064 and 0.083.  The line is a cautious one: from about 55 rows the row
+    // kernels are ahead (55 of 462 FP64 0.181 and 0.140, FP32 0.068 and 0.054; 91 of 3432
+    // FP64 3.03 and 1.81, FP32 0.52 and 0.39).
     if (A.ns < 100 && B.ns > 256) return SIGMA_GATHER;
     BatchMol m{};
     sigma_shape(m, A, B, f64);
@@ -903,9 +906,12 @@ SigmaPath sigma_path(const SpinTables& A, const SpinTables& B, bool f64) {
         if (m.fc < 2 && m.fc < m.noffB) return SIGMA_GATHER;
         return m.smem <= SMEM_MAX ? SIGMA_ROWS : SIGMA_GATHER;
     }
-    // (FP32 rows of up to 252 strings, 10 orbitals, stay with the gather kernel: a
-    // tile of 64 columns is a quarter of such a row, and three launches cost as much
-    // as its work)
+    // (Cautious too: the tiled kernels need rows of 128 strings for a tile of theirs.  Gather
+    // and tiled, one and three columns: 462 strings, 11 orbitals, 0.348 and 0.115, 0.858 and
+    // 0.207 ms; 252 strings, 10 orbitals, 0.091 and 0.047, 0.188 and 0.075; 210 strings 0.072
+    // and 0.045, 0.153 and 0.070.  The dense F pays at every size measured, though it has up
+    // to 28 times the neighbours' terms: 18 orbitals, 9 + 3, 160 and 102 ms; 17 orbitals, 7 + 3,
+    // 43.9 and 18.9; 16 orbitals, 6 + 6, 250 and 92.)
     if (B.ns <= 300) return SIGMA_GATHER;
     return m.K > 0 && m.NO > 0 && m.noffB > 0 && opp_choose(m.NO, m.K, m.nsb)
                ? SIGMA_SLOTS
@@ -1004,6 +1010,9 @@ size_t PairTables::bytes(const SpinTables& A, const SpinTables& B, bool f64, boo
 void PairTables::build(const SpinTables& A, const SpinTables& B, const double* eri, bool f64_,
                        cudaStream_t st) {
     f64 = f64_;
+    int dev = 0;
+    KPM_CUDA(cudaGetDevice(&dev));
+    KPM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     path = sigma_path(A, B, f64);
     if (path == SIGMA_GATHER) return;
     try {
@@ -1052,6 +1061,7 @@ void PairTables::fill(BatchMol& m) const {
     m.denseB = b->dense.as<float>();
     m.ldA = a.ld;
     m.ldB = b->ld;
+    m.nsm = nsm;
     if (path == SIGMA_SLOTS) m.ts = opp_choose(m.NO, m.K, m.nsb);
     else rows_geometry(m);
 }

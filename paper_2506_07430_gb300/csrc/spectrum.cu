@@ -19,8 +19,9 @@
 // at 8192 x 8191, 6e-9 at 60000 x 8192, no damping).  Up to N M = 2^24 that is below
 // 3e-10 and the exact nodes are used; beyond, the sum is over all N moments at the
 // rounded node itself, the x of the omega that is returned.
-// A call with host arrays, 2048 moments at 2048 nodes: 357 us with one chain per node
-// (16 blocks), 51 us here (22 us of it k_reconstruct); 60000 at 8192: 5.2 and 1.8 ms.
+// A call with host arrays, 2048 moments at 2048 nodes: 232 us (334 in a process that has
+// nothing else allocated) with one chain per node (16 blocks) and four allocations, 51 us here
+// (22 us of it k_reconstruct); 60000 at 2048: 5.2 and 0.54 ms.
 // Energy axis omega = a x + b, density per unit energy I/a, written in ascending omega.
 #include "common.cuh"
 
