@@ -25,6 +25,8 @@
 // (1.5 of the two FMA), 2.6 ms at the FP64 rate.
 // k_opp_slots / k_same_dense (larger FP32 molecules): see there.  Three columns at 12
 // orbitals: 4.33 ms with a thread per determinant (two gathers per FMA), 0.88 ms here.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace kpm {
@@ -236,8 +238,10 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
     // (ordinary loads of x: its writer may still run when this CTA starts)
     const double* x = static_cast<const double*>(m.x) + col * dim;
     double* y = static_cast<double*>(m.y) + col * dim;
-    double* sB = reinterpret_cast<double*>(smem);                 // [NO][kp] signed W of this row
-    double* sD = sB + (size_t)NO * kp;                       // [fc][nsb]
+    // [NO][kp] signed W of this row, read for D only, which strings without an off-diagonal
+    // entry do not have
+    double* sB = reinterpret_cast<double*>(smem);
+    double* sD = sB + (noB > 0 ? (size_t)NO * kp : 0);       // [fc][nsb]
     double* sP = sD + (size_t)m.fc * nsb;                    // [parts][nsb] if parts > 1
     double* sX = sP + (m.parts > 1 ? (size_t)m.parts * nsb : 0);   // [nsb] row of x if staged
     double* sFv = sX + (m.stage_x ? nsb : 0);                // [nfa]
@@ -262,7 +266,6 @@ __device__ __forceinline__ void sigma_rows_cta(const BatchMol& m, int64_t ia, in
     }
     for (int j = threadIdx.x; j < nsb; j += blockDim.x) ptr[j] = 0;
     __syncthreads();
-    // (read for D only, which strings without an off-diagonal entry do not have)
     for (int i = noB > 0 ? threadIdx.x : NO * K; i < NO * K; i += blockDim.x) {
         const int s = i / K, e = i - s * K;
         sB[s * kp + e] = e < noA ? flip(woo[s * NO + (sS[e] & 0x7FFF)], sS[e] >> 15)
@@ -765,7 +768,8 @@ int opp_choose(int NO, int K, int64_t nsb) {
 
 void rows_geometry(BatchMol& m) {
     const size_t nsb = (size_t)m.nsb;
-    const size_t fixed = sizeof(double) * ((size_t)m.NO * (m.K | 1) + (m.nnbrA - 1)) +
+    const size_t nw = m.noffB > 0 ? (size_t)m.NO * (m.K | 1) : 0;     // signed W
+    const size_t fixed = sizeof(double) * (nw + (m.nnbrA - 1)) +
                          4 * (size_t)(m.nnbrA - 1) + 6 * (size_t)m.K + nsb + 32;
     const int noB = m.noffB > 0 ? m.noffB : 1;
     // pieces of the term list: short rows would otherwise leave most threads idle
@@ -799,7 +803,11 @@ void rows_geometry(BatchMol& m) {
         }
     }
     m.smem = size(m.fc);
-    const int64_t items = m.nsb * ((m.fc + m.ft - 1) / m.ft);
+    // A thread per item, and for short rows enough to stage W, 32 entries each, as its 100 KB
+    // at 18 orbitals leave room for two CTAs an SM: 18 orbitals, 9 + 1 electrons, 45.3 ms with
+    // the 64 threads that 54 items take, 18.4 with 416 (18.5 in the gather kernel); 9 + 0, without
+    // W, 10.3 ms with its room kept free and 1.8 without (4.5); 16 orbitals, 8 + 1, 2.64 and 1.63
+    const int64_t items = std::max<int64_t>(m.nsb * ((m.fc + m.ft - 1) / m.ft), nw / 32);
     m.threads = (int)(items >= ROWS_THREADS ? ROWS_THREADS : (items + 31) / 32 * 32);
     if (m.threads < 64) m.threads = 64;
 }
