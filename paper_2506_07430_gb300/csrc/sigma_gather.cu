@@ -293,9 +293,11 @@ k_dipole_rows(const double* __restrict__ psi, T* __restrict__ y, int64_t nsb,
     int64_t* oA = reinterpret_cast<int64_t*>(cA + noffA);  // [noffA] row offsets
     const int64_t ia = blockIdx.x;
     for (int64_t j = threadIdx.x; j < nsb; j += blockDim.x) row[j] = psi[ia * nsb + j];
-    for (int i = threadIdx.x; i < nn; i += blockDim.x) {
-        dd[i] = d[i];
-        dd[nn + i] = -d[i];
+    // (the diagonal alone where no beta string has an off-diagonal entry)
+    for (int i = threadIdx.x; i < (noffB > 0 ? nn : n); i += blockDim.x) {
+        const int g = noffB > 0 ? i : i * (n + 1);
+        dd[g] = d[g];
+        dd[nn + g] = -d[g];
     }
     if (DIAG_TABLES)
         for (int i = threadIdx.x; i < (2 << hb); i += blockDim.x) {
